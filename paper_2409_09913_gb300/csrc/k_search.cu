@@ -584,7 +584,9 @@ __global__ void __launch_bounds__(256) merge_kernel(const uint64_t* __restrict__
         if (!ERQ_DCHECK(L >= 0 && L < ck.lists, ck.status, 0)) break;
         int n = inter_cnt[L];
         if (!ERQ_DCHECK(n >= 0 && n <= lstride, ck.status, 0)) n = 0;
-        if (s_fill + n > sortn) {          // uniform: s_fill is shared
+        const bool full = s_fill + n > sortn;
+        __syncthreads();                   // every thread has read s_fill before any appends to it,
+        if (full) {                        // so `full` is uniform
             block_bitonic_u64(buf, sortn);
             for (int i = kp + threadIdx.x; i < sortn; i += blockDim.x) buf[i] = kEmptyKey;
             __syncthreads();
