@@ -47,6 +47,10 @@ __device__ __forceinline__ int warp_incl_scan(int v) {
 // ---- k_linalg.cu
 cudaError_t launch_rotate_fp64(const float* X, const int64_t* gather, const float* C, const int32_t* cl,
                                const float* P, float* out, int64_t n, int D, cudaStream_t s);
+cudaError_t launch_rotate_fp64_if(const uint32_t* flag, const float* X, const int64_t* gather, const float* C,
+                                  const int32_t* cl, const float* P, float* out, int64_t n, int D, cudaStream_t s);
+cudaError_t launch_rotate_tc(const float* X, const int64_t* gather, const float* C, const int32_t* cl, const float* P,
+                             float* out, int64_t n, int D, cudaStream_t s);   // k_rotate_tc.cu
 cudaError_t launch_sgemm(bool nt, const float* A, const float* B, float* C, int64_t M, int N, int K, float alpha,
                          const float* addend, cudaStream_t s);
 cudaError_t launch_sqdist(const float* Q, const float* qn, const float* C, const float* cn, float* out, int64_t nq,

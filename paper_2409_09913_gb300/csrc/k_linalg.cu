@@ -23,6 +23,11 @@ namespace erq {
 // sequential "acc += res * p" of a plain FP64 loop: the result is bit-identical
 // to any implementation that sums in ascending k.
 // Tile 64 rows x 64 columns, 256 threads, 4x4 outputs per thread, BK = 16.
+// The FP64 pipe bounds it (0.75 TFLOP/s).  launch_rotate_fp64 therefore takes
+// the sliced tensor-core form of the same sums (k_rotate_tc.cu: 100,000 x 768
+// in 3 ms instead of 156) wherever it can allocate its digits; this kernel runs
+// inside a stream capture and, with `flag`, for a block that the sliced form
+// gave up on.
 // ---------------------------------------------------------------------------
 constexpr int R64_BM = 64, R64_BN = 64, R64_BK = 16;
 
@@ -31,7 +36,8 @@ __global__ void __launch_bounds__(256) rotate_fp64_kernel(const float* __restric
                                                           const float* __restrict__ C,
                                                           const int32_t* __restrict__ cl,
                                                           const float* __restrict__ P, float* __restrict__ out,
-                                                          int64_t n, int D) {
+                                                          int64_t n, int D, const uint32_t* __restrict__ flag) {
+    if (flag && *flag == 0u) return;
     __shared__ float As[R64_BK][R64_BM + 4];
     __shared__ float Bs[R64_BK][R64_BN + 4];
     const int tid = threadIdx.x;
@@ -106,6 +112,12 @@ __global__ void __launch_bounds__(256) rotate_fp64_kernel(const float* __restric
 cudaError_t launch_rotate_fp64(const float* X, const int64_t* gather, const float* C, const int32_t* cl,
                                const float* P, float* out, int64_t n, int D, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
+    const cudaError_t e = launch_rotate_tc(X, gather, C, cl, P, out, n, D, s);
+    return e != cudaErrorNotSupported ? e : launch_rotate_fp64_if(nullptr, X, gather, C, cl, P, out, n, D, s);
+}
+
+cudaError_t launch_rotate_fp64_if(const uint32_t* flag, const float* X, const int64_t* gather, const float* C,
+                                  const int32_t* cl, const float* P, float* out, int64_t n, int D, cudaStream_t s) {
     const int64_t slab = 65535ll * R64_BM;
     for (int64_t r0 = 0; r0 < n; r0 += slab) {
         const int64_t m = n - r0 < slab ? n - r0 : slab;
@@ -113,7 +125,7 @@ cudaError_t launch_rotate_fp64(const float* X, const int64_t* gather, const floa
         // rows are addressed through `gather` when given, else directly
         count_launch();
         rotate_fp64_kernel<<<grid, 256, 0, s>>>(gather ? X : X + r0 * D, gather ? gather + r0 : nullptr, C,
-                                                cl ? cl + r0 : nullptr, P, out + r0 * D, m, D);
+                                                cl ? cl + r0 : nullptr, P, out + r0 * D, m, D, flag);
     }
     return cudaGetLastError();
 }
