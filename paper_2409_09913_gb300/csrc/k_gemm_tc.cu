@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(gemm::THREADS, 1) gemm_tc_kernel(gemm::Args a)
                 const int s = it % STAGES;
                 if (!mbar_wait_warp(full0 + 8 * s, (it / STAGES) & 1, abort_flag)) { ok = false; break; }
                 tc_fence_after();
-                if (lane == 0) {
+                if (elect_one()) {
                     const uint32_t st = smem_u32(sm + s * STAGE);
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(gemm::THREADS, 1) gemm_tc_kernel(gemm::Args a)
                 __syncwarp();
             }
         }
-        if (lane == 0) mma_commit(done_bar);
+        if (elect_one()) mma_commit(done_bar);
         __syncwarp();
         mbar_wait_warp(done_bar, 0, abort_flag);
     } else {

@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(gemm2::THREADS, 1)
                 const int s = it % STAGES;
                 if (!mbar_wait_warp(full0 + 8 * s, (it / STAGES) & 1, abort_flag)) { ok = false; break; }
                 tc_fence_after();
-                if (lane == 0) {
+                if (elect_one()) {
                     const uint32_t st = smem_u32(sm + s * STAGE);
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(gemm2::THREADS, 1)
                 __syncwarp();
             }
         }
-        if (lane == 0) mma_commit(done_bar);
+        if (elect_one()) mma_commit(done_bar);
         __syncwarp();
         mbar_wait_drain(done_bar, 0);
         __syncwarp();

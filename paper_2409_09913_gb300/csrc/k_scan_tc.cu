@@ -786,14 +786,14 @@ __global__ void __launch_bounds__(THREADS, 1)
                         break;
                     }
                     tc_fence_after();
-                    if (lane == 0) {
+                    const uint32_t ta = tmem + ACOL + (s * RP + b) * (KB / 2);
+                    const uint64_t tq = sdesc(smem_u32(sm + Smem::q + s * TILE_Q));
+                    if (elect_one()) {
                         if (has) {
-                            const uint32_t ta = tmem + ACOL + (s * RP + b) * (KB / 2);
-                            const uint32_t tq = smem_u32(sm + Smem::q + s * TILE_Q);
 #pragma unroll
                             for (int k = 0; k < KB / 16; ++k) {         // 32 bytes of K per instruction
-                                if (F8) mma_f8_ta(dt, ta + k * 8, sdesc(tq + k * 32), idesc, (kb | k) != 0);
-                                else mma_f16_ta(dt, ta + k * 8, sdesc(tq + k * 32), idesc, (kb | k) != 0);
+                                if (F8) mma_f8_ta(dt, ta + k * 8, tq + 2 * k, idesc, (kb | k) != 0);
+                                else mma_f16_ta(dt, ta + k * 8, tq + 2 * k, idesc, (kb | k) != 0);
                             }
                         }
                         mma_commit(bars + C::b_empty_st(s));          // query tile and TMEM stage free
@@ -807,7 +807,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             mbar_arrive(bars + C::b_empty_item(ib));
         }
         // all issued MMAs complete before TMEM is released
-        if (lane == 0) mma_commit(bars + C::b_done());
+        if (elect_one()) mma_commit(bars + C::b_done());
         __syncwarp();
         mbar_wait_drain(bars + C::b_done(), 0);
         __syncwarp();
