@@ -461,24 +461,36 @@ extern "C" erq_status erq_build_index(const float* X, int64_t N, int32_t D, cons
 // Search
 // ---------------------------------------------------------------------------
 // Work-item shape of the scan: queries per item (the tensor-core MMA's N
-// extent) and rows per item.  Heuristic for k' <= 32: 128 queries per item when
-// a probed cluster has more than 96 probing queries on average, else 64; for
-// larger k' 32; 4,096 rows; the autotuned or forced shape wins.
-static void choose_scan_shape(const erq_index* ix, int prec, int kp, int64_t nq, int maxp, int* qn, int* rr) {
-    if (prec == ERQ_PREC_FP32) {
+// extent) and rows per item; the autotuned or forced shape wins.  For k' <= 32,
+// 128 queries per item (twice the MMA width for one conversion of the codes)
+// when a probed cluster has more than 72 probing queries on average, else 64
+// (10,000 queries x 16 of 2,048 lists, 78 a list: 0.38 ms with 64, 0.31 with
+// 128; 512 x 64 of 512, 64 a list: 0.095 with 64, 0.16 with 128); for larger
+// k' 32.  FP32 precision has two query parts per tile and stops at 64.  Rows:
+// at most 8,192, and few enough that the items can fill the chip twice (a
+// single query's 16 lists of 200 rows are 32 one-block items instead of 16).
+static void choose_scan_shape(const erq_index* ix, int prec, int kp, int64_t nq, int maxp, int sms, int* qn, int* rr) {
+    if (prec == ERQ_PREC_FP32 && kp > 128) {              // the CUDA-core scan
         *qn = 64;
         *rr = ix->force_rr > 0 ? ix->force_rr : 4096;
         return;
     }
     const int cls = kp <= 32 ? 0 : 1;
     const int64_t work = nq * (int64_t)maxp;
-    int q = cls == 0 ? ((double)work / ix->nlist > 96.0 ? 128 : 64) : 32, r = 4096;
+    const double per_list = (double)work / ix->nlist;
+    int q = cls == 0 ? (per_list > 72.0 && prec != ERQ_PREC_FP32 ? 128 : 64) : 32;
+    // rows of all items: the probed lists' rows, once per chunk of queries
+    const double lists = (double)std::min<int64_t>(ix->nlist, work);
+    const double chunks = std::max(1.0, (double)work / lists / q);
+    const double rows = (double)ix->N * lists / ix->nlist * chunks;
+    int r = 8192;
+    if (rows < 8192.0 * 2 * sms) r = std::max(128, (int)(rows / (2.0 * sms)) / 128 * 128);
     const erq_index::ScanTune& t = ix->tune[cls];
-    if (t.valid && work <= 4 * t.work && 4 * work >= t.work) {
+    if (prec != ERQ_PREC_FP32 && t.valid && work <= 4 * t.work && 4 * work >= t.work) {
         q = t.qn;
         r = t.rr;
     }
-    if (ix->force_qn > 0 && scan_tc_shape_ok(ix->force_qn, kp)) q = ix->force_qn;
+    if (ix->force_qn > 0 && scan_tc_shape_ok(ix->force_qn, kp) && (prec != ERQ_PREC_FP32 || ix->force_qn <= 64)) q = ix->force_qn;
     if (ix->force_rr > 0) r = ix->force_rr;
     *qn = q;
     *rr = r;
@@ -623,7 +635,13 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     // ---- phase A workspace (sizes known on the host)
     // queries per work item of the scan kernels
     int QT = 64, RR = 4096;
-    choose_scan_shape(ix, prec, kp, nq, maxp, &QT, &RR);
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    choose_scan_shape(ix, prec, kp, nq, maxp, sms, &QT, &RR);
+    // FP32 precision runs on the tensor cores too (two FP16 query parts) up to
+    // the list sizes that path has
+    const bool tcp = prec != ERQ_PREC_FP32 || tc_available(prec, D, kp);
     ix->last_qn = QT;
     ix->last_rr = RR;
     Carver plan(nullptr, 0);
@@ -657,12 +675,12 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
         T((uint64_t*)nullptr, 1);                                        // 19 (unused)
         T((__half*)nullptr, prec == ERQ_PREC_FP16 ? (size_t)nq * D : 1); // 20 Qh
         T((int32_t*)nullptr, nq);                                        // 21 eQ
-        T((uint64_t*)nullptr, prec == ERQ_PREC_FP32 ? 1 : nq);           // 22 query-wide thresholds
+        T((uint64_t*)nullptr, tcp ? nq : 1);                             // 22 query-wide thresholds
         T((__half*)nullptr, (size_t)nq * D);                              // 23 Q hi
         T((__half*)nullptr, (size_t)nq * D);                              // 24 Q lo
         T((float*)nullptr, (!explicit_probe && nlist > 1) ? (size_t)nq * ((nlist + 31) / 32) : 1);  // 25 group minima
         T((unsigned char*)nullptr, prec == ERQ_PREC_FP8 ? (size_t)nq * Dq : 1);   // 26 e4m3 queries
-        T((float*)nullptr, prec == ERQ_PREC_FP8 ? (size_t)nq : 1);                // 27 their scales
+        T((float*)nullptr, prec == ERQ_PREC_FP16 ? 1 : (size_t)nq);               // 27 scales (e4m3, or FP32's two parts)
         T((int32_t*)nullptr, nlist);                                     // 28 touch_c
     };
     void* sl[29];
@@ -759,6 +777,12 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
                                   : launch_row_topk_fast(sqd, nq, nlist, nlist, maxp, probe, nullptr, maxp, s);
         if (e != cudaSuccess) return cuda_fail(e, "probe select");
     }
+    if (prec == ERQ_PREC_FP32 && tcp && !ts) {
+        // q' in two FP16 parts (over the parts of q, which the probe has read)
+        if ((e = launch_query_prep(Qrot, nq, D, eQ, nullptr, (__half*)sl[23], (__half*)sl[24], s, (float*)sl[27])) !=
+            cudaSuccess)
+            return cuda_fail(e, "rotated query split");
+    }
     ERQ_TRY(mark(2));
     // ---- plan
     pa.probe = probe_use;
@@ -777,7 +801,10 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     // ||q_r - c||^2 (or -<q_r, c>) of the probed pairs: the probe's own values
     // when it computed them (the FP32 expansion ||q_r||^2 + ||c||^2 - 2<q_r, c>
     // with an FP32-accurate product), else computed directly below
-    const bool dqc_from_probe = !explicit_probe && nlist > 1;
+    // FP32 precision computes them directly: the probe's product drops its low
+    // bits at every tensor-core step, and that bias (1e-5 of an estimate at D =
+    // 960) is most of an FP32 estimate's error
+    const bool dqc_from_probe = !explicit_probe && nlist > 1 && (ts || prec != ERQ_PREC_FP32);
     pa.sqd = dqc_from_probe ? sqd : nullptr;
     pa.dqc = dqc;
     DevChecks ck;
@@ -831,9 +858,10 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     pb.take<uint64_t>((size_t)Ltot * lstride);
     pb.take<int32_t>(Ltot);
     pb.take<int64_t>(1);
-    const bool tcp = prec != ERQ_PREC_FP32;
     pb.take<int4>(tcp ? nitems : 0);
     pb.take<int4>(tcp ? nitems * QT : 0);
+    const int tc_grid = (int)std::min<int64_t>(nitems, sms);
+    pb.take<uint64_t>(tcp ? scan_spill_entries(QT, tc_grid) : 0);
     if (async && ix->ws_b_bytes < pb.off)
         ERQ_CHECK_CUDA(cudaStreamSynchronize(s));   // growing the buffer frees the old one
     ERQ_TRY(ensure_ws(&ix->ws_b, &ix->ws_b_bytes, pb.off));
@@ -844,6 +872,7 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     int64_t* n_items_d = cb.take<int64_t>(1);
     int4* itemd = cb.take<int4>(tcp ? nitems : 0);
     int4* itemq = cb.take<int4>(tcp ? nitems * QT : 0);
+    uint64_t* spill = cb.take<uint64_t>(tcp ? scan_spill_entries(QT, tc_grid) : 0);
     ERQ_CHECK_CUDA(cudaMemcpyAsync(n_items_d, pa.item_off + 2 * nlist, 8, cudaMemcpyDeviceToDevice, s));
     ck.items = nitems;
     ck.lists = Ltot;
@@ -852,13 +881,14 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
 
     if ((e = launch_plan_items(pa, items, s)) != cudaSuccess) return cuda_fail(e, "plan items");
     if (tcp && (e = launch_item_tables(items, n_items_d, nitems, ix->list_off, ix->poff, pa.qoff, pa.qlist, dqc,
-                                       pa.qbase, pa.slot_off, maxp, RR, QT, nlist, itemd, itemq, pa.stats, ck, s)) !=
+                                       pa.qbase, pa.slot_off, maxp, RR, QT, nlist, itemd, itemq,
+                                       prec == ERQ_PREC_FP32 ? nullptr : pa.stats, ck, s)) !=
                    cudaSuccess)
         return cuda_fail(e, "item tables");
     ERQ_TRY(mark(3));
     // ---- scan
     ScanLaunch L;
-    L.Qrot = Qrot; L.Qh = sl[20]; L.Q8 = sl[26]; L.qscale = (const float*)sl[27]; L.Dq = Dq; L.status = ix->status; L.N = ix->N; L.codes = ix->codes; L.g_const = ix->g_const; L.f_res = ix->f_res; L.list_off = ix->list_off;
+    L.Qrot = Qrot; L.Qh = prec == ERQ_PREC_FP32 ? sl[23] : sl[20]; L.Ql = sl[24]; L.Q8 = sl[26]; L.qscale = (const float*)sl[27]; L.Dq = Dq; L.status = ix->status; L.N = ix->N; L.codes = ix->codes; L.g_const = ix->g_const; L.f_res = ix->f_res; L.list_off = ix->list_off;
     L.list_ids = ix->list_ids; L.qlist = pa.qlist; L.qoff = pa.qoff; L.items = items; L.n_items = n_items_d;
     L.dqc = dqc; L.slot_off = pa.slot_off; L.qbase = pa.qbase; L.inter = inter; L.inter_cnt = inter_cnt;
     L.maxp = maxp; L.D = D; L.B = ix->B; L.kp = kp; L.RR = RR; L.qn = QT; L.nlist = nlist;
@@ -872,18 +902,17 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     L.stall_stage = ix->stall_stage;
     if (tcp) ERQ_CHECK_CUDA(cudaMemsetAsync(L.tq, 0xff, sizeof(uint64_t) * nq, s));
     ERQ_CHECK_CUDA(cudaMemsetAsync(ix->dctr, 0, sizeof(unsigned int), s));
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    L.grid = (int)std::min<int64_t>(nitems, (int64_t)sms * (prec == ERQ_PREC_FP32 ? scan_fp32_blocks_per_sm(kp, ix->B) : 1));
-    if (prec == ERQ_PREC_FP32) {
+    L.spill = spill;
+    L.grid = tcp ? tc_grid : (int)std::min<int64_t>(nitems, (int64_t)sms * scan_fp32_blocks_per_sm(kp, ix->B));
+    if (!tcp) {
         if ((e = launch_scan_fp32(L, s)) != cudaSuccess) return cuda_fail(e, "scan fp32");
     } else {
         ERQ_TRY(scan_tc(L, prec, s));
     }
     ERQ_TRY(mark(4));
     // ---- merge, re-rank
-    if ((e = launch_merge(inter, inter_cnt, pa.qbase, nq, kp, lstride, cand, ck, s)) != cudaSuccess)
+    if ((e = launch_merge(inter, inter_cnt, pa.qbase, nq, kp, lstride, tcp ? (const unsigned long long*)sl[22] : nullptr, cand,
+                          ck, s)) != cudaSuccess)
         return cuda_fail(e, "merge");
     ERQ_TRY(mark(5));
     if ((e = launch_rerank(cand, nq, kp, ix->X, Q, D, k, do_rerank ? 1 : 0, ip, ids, dists, p->cand_ids, p->cand_est,
@@ -1334,7 +1363,7 @@ extern "C" erq_status erq_merge_topk(const int64_t* cand_ids, const float* value
     ck.lists = nq;
     cudaError_t e = launch_make_keys(cand_ids, values, nq * (int64_t)m, 0, neg, keys, s);
     if (e == cudaSuccess) e = launch_one_list_per_query(nq, m, counts, off, s);
-    if (e == cudaSuccess) e = launch_merge(keys, counts, off, nq, k, m, cand, ck, s);
+    if (e == cudaSuccess) e = launch_merge(keys, counts, off, nq, k, m, nullptr, cand, ck, s);
     if (e == cudaSuccess) e = launch_keys_to_pairs(cand, nq * (int64_t)k, neg, ids_out, vals_out, s);
     const cudaError_t ef = cudaFreeAsync(ws, s);
     if (e != cudaSuccess) return cuda_fail(e, "erq_merge_topk");

@@ -43,9 +43,10 @@ struct PlanArgs {
 
 struct ScanLaunch {
     const float* Qrot;
-    const void* Qh;             // FP16 rotated queries (tensor-core path)
+    const void* Qh;             // FP16 rotated queries (tensor-core path; FP32 precision: their high parts)
+    const void* Ql;             // FP32 precision: low parts (scaled by 1 / qscale, as Qh then is)
     const void* Q8;             // e4m3 rotated queries, rows of Dq bytes (kind::f8f6f4 path)
-    const float* qscale;        // their per-query power-of-two scales
+    const float* qscale;        // per-query power-of-two scales of Q8, or of Qh + Ql
     int64_t Dq;
     uint32_t* status;
     int64_t N;
@@ -63,6 +64,7 @@ struct ScanLaunch {
     const int64_t* qbase;
     uint64_t* inter;
     int32_t* inter_cnt;
+    uint64_t* spill;            // tensor-core path: continuation of the CTAs' candidate lists
     const int4* itemd;          // tensor-core path: per-item {rb0 lo, rb0 hi, rows, queries}
     const int4* itemq;          // tensor-core path: per-item query slots
     const float4* rowmeta;      // tensor-core path: per padded row {g, f_res/2, id, 0}
@@ -126,8 +128,10 @@ cudaError_t launch_make_keys(const int64_t* ids, const float* vals, int64_t n, i
 cudaError_t launch_keys_to_pairs(const uint64_t* keys, int64_t n, int neg, int64_t* ids, float* vals, cudaStream_t s);
 cudaError_t launch_one_list_per_query(int64_t nq, int m, int32_t* counts, int64_t* off, cudaStream_t s);
 cudaError_t launch_merge(const uint64_t* inter, const int32_t* inter_cnt, const int64_t* qbase, int64_t nq, int kp,
-                         int lstride, uint64_t* cand, const DevChecks& ck, cudaStream_t s);
+                         int lstride, const unsigned long long* tq, uint64_t* cand, const DevChecks& ck,
+                         cudaStream_t s);
 int scan_list_stride(int precision, int kp, int qn);
+int64_t scan_spill_entries(int qn, int grid);
 cudaError_t launch_item_tables(const int4* items, const int64_t* n_items, int64_t items_bound, const int64_t* list_off,
                                const int64_t* poff, const int64_t* qoff, const int64_t* qlist, const float* dqc,
                                const int64_t* qbase, const int32_t* slot_off, int maxp, int RR, int qn, int nlist,

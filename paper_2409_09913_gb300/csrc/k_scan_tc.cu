@@ -5,7 +5,7 @@
 // A work item is (cluster, up to QN of the queries that probe it, up to RR
 // stored rows).  Operands of one MMA (kind::f16, M = 128, N = npad, K = 16):
 //   A = 128 stored rows of the cluster, codes expanded to 2*ybar_u - (2^B-1),
-//       odd integers in [-255, 255] and therefore exact in FP16, held in
+//       odd integers in [-511, 511] and therefore exact in FP16, held in
 //       tensor memory (row = lane, two FP16 values per column);
 //   B = the item's queries (rotated q' in FP16), npad = the query count rounded
 //       up to a multiple of 16, K-major, 128-byte swizzled rows gathered from
@@ -14,7 +14,7 @@
 // to a multiple of 32 rows and stored as [tiles of 32 rows][K blocks of 64]
 // [B words][32 rows] of 8 bytes, i.e. exactly B bits per coordinate (the
 // layout is given at unpack_codes); the 128 rows of one row block and K block
-// are four contiguous 256*B-byte pieces fetched by one 3-D TMA load.
+// are four contiguous 256*B-byte pieces fetched by one TMA load.
 //
 // The estimate is est = ||q_r - c||^2 + g + (f_res / 2) * acc with g, f_res the
 // stored per-row factors, or for the inner-product metric the ranking score
@@ -25,44 +25,47 @@
 // One persistent CTA per SM takes work items from a global counter (items are
 // ordered by decreasing cluster size).  A stage group is up to RP = 2 row
 // blocks of 128 rows that share the stage's query tile; a stage is one
-// 64-coordinate K block of the group.  Warp roles (27 warps):
-//   warps 0-3    estimate tiles: warp w reads TMEM lanes 32w .. 32w + 31 (its
-//                32 rows, all queries) of each finished row-block accumulator,
-//                frees the accumulator as soon as its last columns are in
-//                registers, and stores g + (f_res/2) acc into one of EB
-//                query-major tiles in shared memory;
-//   warps 4-11   converters, two sets of four that take alternate stages:
-//                warp w unpacks the codes of rows 32 (w % 4) .. + 31 of both
-//                row blocks of its stages from the raw stage in shared memory
-//                into FP16 (or e4m3) values in the stage's TMEM columns;
-//   warp 12      code loader: publishes the items, per row block a bulk copy of
-//                the rows' factors and ids, per stage one TMA load of the packed
-//                codes per row block into a raw ring that is released as soon as
-//                the converters have read it (so loads run up to RS stages
-//                ahead, independent of the tensor cores; RS is even, so that
-//                each raw slot is always converted by the same converter set
-//                and its phases are awaited in order);
-//   warps 13-14  query loaders: per stage the item's query rows (128 bytes
-//                each) by TMA gather4 into the stage's swizzled B tile, the
-//                stages taken in turn by the two warps;
-//   warps 15, 16 MMA issuers of row blocks 0 and 1 (one elected thread each;
-//                warp 15 owns the tensor memory); each commits once per stage to
-//                the stage's release barrier, which frees the query tile and the
-//                stage's TMEM code columns;
-//   warps 17-26  filters (NFX = 10), pipelined behind the tiles through full /
-//                empty tile barriers: warp f owns the query slots f + NFX j and
-//                filters their rows (float pre-filter against the threshold,
-//                exact keys, ballots) into per-query candidate lists; a full
-//                list is compacted by a warp bitonic sort to its k' smallest.
-//                A query starts from the smallest k'-th key published so far by
-//                its items, which is never below its final k'-th key, so each
-//                list stays a superset of what the item contributes.
-// Accumulators are double-buffered per row block, so the epilogue of one stage
-// group overlaps the MMAs of the next.
+// 64-coordinate K block of the group, a unit one row block of a stage.  Units
+// are numbered through the CTA's life, and so are row blocks.  Warp roles (28
+// warps):
+//   warps 0-7    epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (its 32
+//                rows) of every finished accumulator, 16 queries at a time, the
+//                even 16-column groups in warps 0-3 and the odd ones in 4-7; one
+//                compare per value against the query's threshold (in the units
+//                of g + (f_res/2) acc) and one vote per query; a query with a
+//                candidate gets its exact keys appended to the query's list in
+//                shared memory (one atomic per query and warp).  Lists beyond
+//                their shared capacity continue in global memory; after a row
+//                block the lists above TRIG entries are cut to (about) their k'
+//                smallest, which also lowers the query's threshold;
+//   warps 8-23   converters, four sets of four warps: set U % 4 unpacks unit U,
+//                one thread per row, from the raw ring in shared memory into FP16
+//                (or e4m3) values in TMEM slot U % AS;
+//   warp 24      code loader: publishes the items, per row block a bulk copy of
+//                the rows' factors and ids, per unit one TMA load of the packed
+//                codes into a raw ring that is released as soon as the
+//                converters have read it (the ring's length is a multiple of
+//                four, so that each slot belongs to one converter set, which
+//                awaits its phases in order);
+//   warps 25, 26 query loaders: per stage the item's query rows by TMA gather4
+//                into the stage's swizzled B tile, the stages taken in turn;
+//   warp 27      MMA issuer (one elected thread; owner of the tensor memory).
+//                Row blocks take the accumulators in turn (NACC of them), so
+//                that one is drained while the others fill.
+// Measured before this arrangement (per-role clocks; 10,000 queries x 16 lists
+// of 400k x 960): the issuer waited 44 % of its time for converted codes
+// (a unit takes one warp about 1,200 cycles, so eight converter warps gave one
+// unit per 600 cycles against 128-256 of tensor time), and with 128 queries
+// per item a single estimate tile between four tile warps and ten filter warps
+// serialised both; an admission cost 2,000-3,000 cycles of one filter warp.
+// A query starts from the smallest threshold published so far by its items,
+// which is never below its final k'-th key, so each list stays a superset of
+// what the item contributes.
 // Every mbarrier wait is bounded (the limit is a kernel argument): on expiry
 // the kernel records ERQ_ETIMEOUT in the status word, every role stops at its
-// next wait (the abort flag), the copies and MMAs already issued are drained
-// (bounded), TMEM is freed and the kernel returns.
+// next wait (the abort flag; the epilogue warps agree on it at their named
+// barrier), the copies and MMAs already issued are drained (bounded), TMEM is
+// freed and the kernel returns.
 #include <algorithm>
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -73,6 +76,7 @@
 #include "erq_kernels.cuh"
 #include "erq_search.cuh"
 #include "tc_common.cuh"
+#include "warp_sort.cuh"
 
 namespace erq {
 
@@ -81,51 +85,53 @@ namespace tc {
 constexpr int MR = 128;          // stored rows per row block (MMA M = TMEM lanes)
 static_assert(MR == 128, "four 32-row lane quarters per row block");
 constexpr int KB = 64;           // FP16 elements per K block (one 128-byte swizzle row)
-constexpr int RP = 2;            // row blocks per stage group (one accumulator and one issuer each)
-constexpr int MS = 8;            // row-factor buffers
-constexpr int RSMAX = 8;         // raw-code ring slots at most
-constexpr int W_CV = 4;          // converter warps 4..11 (row block (w - 4) / 4, lane quarter w % 4)
-constexpr int W_LD = 12;         // code loader and item publisher
-constexpr int W_QL = 13;         // query-tile loaders 13 .. 13 + NQL - 1 (stage g: loader g % NQL)
+constexpr int RP = 2;            // row blocks per stage group
+constexpr int MS = 4;            // row-factor buffers
+constexpr int AS = 8;            // TMEM slots of converted units (32 columns each)
+constexpr int RSMAX = 16;        // raw-code ring slots at most
+constexpr int NEP = 16;          // epilogue warps 0 .. NEP - 1 (a multiple of four)
+constexpr int W_CV = NEP;        // converter warps: set (w - W_CV) / 4, lane quarter w % 4
+constexpr int NSET = 2;
+constexpr int W_LD = W_CV + 4 * NSET;   // code loader and item publisher
+constexpr int W_QL = W_LD + 1;          // query-tile loaders (stage g: loader g % NQL)
 constexpr int NQL = 2;
-constexpr int W_MMA = W_QL + NQL;   // MMA issuers (row block 0, TMEM owner; row block 1)
-constexpr int W_FX = W_MMA + 2;     // filter warps W_FX .. W_FX + NFX - 1
-constexpr int NFX = 10;
-constexpr int NWARP = W_FX + NFX;
+constexpr int W_MMA = W_QL + NQL;       // MMA issuer, TMEM owner
+constexpr int NWARP = W_MMA + 1;
 constexpr int THREADS = 32 * NWARP;
 constexpr int TMEM_COLS = 512;
+constexpr int ACOL = TMEM_COLS - AS * (KB / 2);   // first TMEM column of the code slots
 constexpr int KCAP = 128;        // largest k' of the tensor-core path
+constexpr int SP = 128;          // entries of a list's continuation in global memory
+constexpr int BAR_EP = 1;        // named barrier of the epilogue warps
+static_assert(AS % NSET == 0 && W_CV % 4 == 0, "a set owns whole slots and its warps their lane quarters");
 
 // Work-item capacities: QN queries per item at most (the MMA's N extent), KC
-// list entries per query, NBUF accumulator buffers per row block, LS stages of
-// query tiles and TMEM code columns, EB estimate tiles (with two the filters
-// work on one while the other fills), RAWK KB of raw-code ring, and LG: the
-// per-query candidate lists live in the item's output list slots in global
-// memory (LG = 1) instead of shared memory.
-template <int QN_, int KC_, int NBUF_, int LS_, int EB_, int RAWK_, int LG_>
+// shared list entries per query, TRIG entries above which a list is cut after a
+// row block, LS query-tile stages of QB bytes per query, RAWK KB of raw ring.
+template <int QN_, int KC_, int TRIG_, int LS_, int QB_, int RAWK_>
 struct Cfg {
-    static constexpr int QN = QN_, KC = KC_, NBUF = NBUF_, LS = LS_, EB = EB_, LG = LG_;
+    static constexpr int QN = QN_, KC = KC_, TRIG = TRIG_, LS = LS_, QB = QB_;
+    static constexpr int NACC = ACOL / QN;           // accumulators
     static constexpr int RAW_BYTES = RAWK_ * 1024;
-    static constexpr int KS = KC <= 64 ? 64 : 256;   // sort width of a list compaction
-    static constexpr int TILE_Q = QN * 128;          // one stage's query tile: QN rows of 128 bytes
-    static constexpr int ACOL = NBUF * RP * QN;      // first TMEM column of the code stages
-    static_assert(ACOL + LS * RP * (KB / 2) <= TMEM_COLS, "tensor memory budget");
-    static_assert(LS % 2 == 0, "the two converter sets take alternate stages and must own whole slots");
-    static_assert(QN % 32 == 0 && KC >= 64 && (QN + NFX - 1) / NFX <= 32, "item shape");
+    static constexpr int TILE_Q = QN * QB;           // one stage's query tile
+    static_assert(NACC >= RP && QN % 32 == 0, "a stage group's accumulators fit");
+    // entries after a row block: at most TRIG before it and 128 new ones
+    static_assert(KC % 32 == 0 && TRIG <= KC && TRIG + MR <= KC + SP, "list capacity");
     struct Smem {
         // offsets in bytes from a 1024-aligned base
-        static constexpr int q = 0;                              // LS x [QN][128 B] query tiles, swizzled
-        static constexpr int raw = q + LS * TILE_Q;              // raw-code ring (RS slots of RP x B KB)
-        static constexpr int est = raw + RAW_BYTES;              // EB x [QN][MR] f32 g + (f_res/2) acc
-        static constexpr int lists = est + EB * QN * MR * 4;     // [QN][KC] u64 candidate keys (LG = 0)
-        static constexpr int meta = lists + (LG ? 0 : QN * KC * 8);   // MS x [MR] float4 {g, f_res/2, id, 0}
+        static constexpr int q = 0;                              // LS x [QN][QB] query tiles, swizzled
+        static constexpr int raw = q + LS * TILE_Q;              // raw-code ring (RS slots of B KB)
+        static constexpr int lists = raw + RAW_BYTES;            // [QN][KC] u64 candidate keys
+        static constexpr int meta = lists + QN * KC * 8;         // MS x [MR] float4 {g, f_res/2, id, 0}
         static constexpr int iq = meta + MS * MR * 16;           // 2 x [QN] int4 {query row, dqc bits, list lo, hi}
         static constexpr int tq = iq + 2 * QN * 16;              // 2 x [QN] u64 query-wide threshold at publication
-        static constexpr int qsc = tq + 2 * QN * 8;              // 2 x [QN] f32 query scale (e4m3 path)
+        static constexpr int tau = tq + 2 * QN * 8;              // [QN] u64 admission key
+        static constexpr int thr = tau + QN * 8;                 // [QN] f32 relaxed threshold (NaN: no query)
+        static constexpr int cnt = thr + QN * 4;                 // [QN] u32 list fill
+        static constexpr int qsc = cnt + QN * 4;                 // 2 x [QN] f32 query scale
         static constexpr int itd = qsc + 2 * QN * 4;             // 2 x int4 {rb0 lo, rb0 hi, rows, queries | -1}
-        static constexpr int ids = itd + 2 * 16;                 // EB x [MR] u32 ids of the tile's rows
-        static constexpr int bars = ids + EB * MR * 4;
-        static constexpr int nbars = 2 * RSMAX + 2 * LS + LS * RP + 2 * NBUF * RP + 2 * MS + 4 + 2 + 2 * EB;
+        static constexpr int bars = itd + 2 * 16;
+        static constexpr int nbars = 2 * RSMAX + 2 * LS + 2 * AS + 2 * NACC + 2 * MS + 4 + 2;
         static constexpr int tmem_slot = bars + nbars * 8;
         static constexpr int abort_flag = tmem_slot + 4;
         static constexpr int total = abort_flag + 4 + 1024;      // + alignment slack
@@ -135,28 +141,30 @@ struct Cfg {
     static constexpr int b_full_raw(int s) { return 8 * s; }
     static constexpr int b_empty_raw(int s) { return 8 * (RSMAX + s); }
     static constexpr int b_full_q(int s) { return 8 * (2 * RSMAX + s); }
-    static constexpr int b_empty_st(int s) { return 8 * (2 * RSMAX + LS + s); }
-    static constexpr int b_full_a(int s, int b) { return 8 * (2 * RSMAX + 2 * LS + s * RP + b); }
-    static constexpr int b_tfull(int u, int b) { return 8 * (2 * RSMAX + 2 * LS + LS * RP + u * RP + b); }
-    static constexpr int b_tempty(int u, int b) { return 8 * (2 * RSMAX + 2 * LS + LS * RP + NBUF * RP + u * RP + b); }
-    static constexpr int B0 = 2 * RSMAX + 2 * LS + LS * RP + 2 * NBUF * RP;
-    static constexpr int b_full_meta(int m) { return 8 * (B0 + m); }
-    static constexpr int b_empty_meta(int m) { return 8 * (B0 + MS + m); }
-    static constexpr int b_full_item(int i) { return 8 * (B0 + 2 * MS + i); }
-    static constexpr int b_empty_item(int i) { return 8 * (B0 + 2 * MS + 2 + i); }
-    static constexpr int b_done() { return 8 * (B0 + 2 * MS + 4); }
+    static constexpr int b_empty_q(int s) { return 8 * (2 * RSMAX + LS + s); }
+    static constexpr int B0 = 2 * RSMAX + 2 * LS;
+    static constexpr int b_full_a(int s) { return 8 * (B0 + s); }
+    static constexpr int b_empty_a(int s) { return 8 * (B0 + AS + s); }
+    static constexpr int b_tfull(int u) { return 8 * (B0 + 2 * AS + u); }
+    static constexpr int b_tempty(int u) { return 8 * (B0 + 2 * AS + NACC + u); }
+    static constexpr int B1 = B0 + 2 * AS + 2 * NACC;
+    static constexpr int b_full_meta(int m) { return 8 * (B1 + m); }
+    static constexpr int b_empty_meta(int m) { return 8 * (B1 + MS + m); }
+    static constexpr int b_full_item(int i) { return 8 * (B1 + 2 * MS + i); }
+    static constexpr int b_empty_item(int i) { return 8 * (B1 + 2 * MS + 2 + i); }
+    static constexpr int b_done() { return 8 * (B1 + 2 * MS + 4); }
     // a barrier nothing arrives on (the test stall of the bounded-wait path)
-    static constexpr int b_never() { return 8 * (B0 + 2 * MS + 5); }
-    static constexpr int b_tile_full(int t) { return 8 * (B0 + 2 * MS + 6 + t); }
-    static constexpr int b_tile_empty(int t) { return 8 * (B0 + 2 * MS + 6 + EB + t); }
+    static constexpr int b_never() { return 8 * (B1 + 2 * MS + 5); }
 };
-using CfgA = Cfg<64, 64, 2, 4, 2, 64, 0>;    // k' <= 32, up to 64 queries per item
-using CfgW = Cfg<128, 64, 1, 4, 1, 48, 1>;   // k' <= 32, up to 128 queries per item (twice the MMA width)
-using CfgB = Cfg<32, 160, 2, 4, 2, 64, 0>;   // k' <= 128, up to 32 queries per item
+using CfgA = Cfg<64, 160, 96, 6, 128, 48>;    // k' <= 32, up to 64 queries per item
+using CfgW = Cfg<128, 96, 88, 4, 128, 40>;    // k' <= 32, up to 128 queries per item
+using CfgB = Cfg<32, 256, 160, 6, 128, 48>;   // k' <= 128, up to 32 queries per item
+using CfgA32 = Cfg<64, 160, 96, 4, 256, 48>;  // the same with two query parts (FP32 precision)
+using CfgB32 = Cfg<32, 256, 160, 6, 256, 48>;
 
-// arrivals that complete a phase of the item-release barrier: every lane of the
-// query loader, the converters, the two issuers, the tile warps and the filters
-constexpr int kItemReleasers = 32 * (NQL + 8 + 2 + 4 + NFX);
+// arrivals that complete a phase of the item-release barrier: one per warp of
+// the epilogue, the converters, the query loaders and the issuer
+constexpr int kItemReleasers = NEP + 4 * NSET + NQL + 1;
 
 // Packed codes of one stored row and one 64-coordinate K block -> 32 TMEM
 // columns of FP16 pairs 2u - (2^B - 1) (column c holds coordinates 2c, 2c+1).
@@ -345,6 +353,8 @@ struct Args {
     unsigned int* work_ctr;       // items taken after the first grid-size ones (zero at launch)
     uint64_t* inter;
     int32_t* inter_cnt;
+    int lstride;                  // entries of an output list
+    uint64_t* spill;              // [grid][QN][SP] continuation of the CTAs' lists
     unsigned long long* tq;       // [nq] query-wide admission threshold (k'-th key of a finished item)
     const float* qscale;          // e4m3 path: per-query power-of-two scale of the e4m3 values
     uint32_t* status;
@@ -364,77 +374,101 @@ __device__ __forceinline__ int64_t rb0_of(int4 d) { return (int64_t)(uint32_t)d.
 
 using namespace tc;
 
-__device__ __forceinline__ uint64_t shfl_xor_u64(uint64_t x, int m) {
-    const uint32_t lo = __shfl_xor_sync(0xffffffffu, (uint32_t)x, m);
-    const uint32_t hi = __shfl_xor_sync(0xffffffffu, (uint32_t)(x >> 32), m);
-    return ((uint64_t)hi << 32) | lo;
-}
-__device__ __forceinline__ uint64_t shfl_u64(uint64_t x, int src) {
-    const uint32_t lo = __shfl_sync(0xffffffffu, (uint32_t)x, src);
-    const uint32_t hi = __shfl_sync(0xffffffffu, (uint32_t)(x >> 32), src);
-    return ((uint64_t)hi << 32) | lo;
-}
-
-// Ascending warp bitonic sort of N (a power of two >= 64) keys held as element
-// e = i*32 + lane in v[i].
-template <int N>
-__device__ __forceinline__ void warp_sort(uint64_t (&v)[N / 32], int lane) {
-#pragma unroll
-    for (int size = 2; size <= N; size <<= 1) {
-#pragma unroll
-        for (int d = size >> 1; d > 0; d >>= 1) {
-#pragma unroll
-            for (int i = 0; i < N / 32; ++i) {
-                const int e = i * 32 + lane;
-                const bool asc = (e & size) == 0 || size == N;
-                if (d >= 32) {                     // partner in another register of this lane
-                    const int j = i ^ (d / 32);
-                    if (j > i) {
-                        const uint64_t x = v[i], y = v[j];
-                        v[i] = (x < y) == asc ? x : y;
-                        v[j] = (x < y) == asc ? y : x;
-                    }
-                } else {
-                    const uint64_t p = shfl_xor_u64(v[i], d);
-                    const bool lower = (e & d) == 0;
-                    const bool keep_min = lower == asc;
-                    v[i] = keep_min ? (p < v[i] ? p : v[i]) : (p > v[i] ? p : v[i]);
-                }
-            }
-        }
-    }
-}
-
-// A threshold on the estimate tile's values (g + (f_res/2) acc) that admits
-// every value v with fl(dq + v) <= tf: tf - dq, raised by 2^-20 of
-// |tf| + |dq| to cover the roundings of fl(dq + v) and of this expression
-// (each within 2^-24 of the magnitudes involved) and by 2^-120 for the
-// absolute error of subnormal results; +inf stays +inf.
+// A threshold on the accumulator values (g + (f_res/2) acc) that admits every
+// value v with fl(dq + v) <= tf: tf - dq, raised by 2^-20 of |tf| + |dq| to
+// cover the roundings of fl(dq + v) and of this expression (each within 2^-24
+// of the magnitudes involved) and by 2^-120 for the absolute error of
+// subnormal results; +inf stays +inf.
 __device__ __forceinline__ float relaxed_threshold(float tf, float dq) {
     return (tf - dq) + (0x1p-20f * (fabsf(tf) + fabsf(dq)) + 0x1p-120f);
 }
 
-// Keep the kp smallest keys of one query's list (cnt <= KS entries) in its
-// first kp slots, sorted; returns the new admission threshold (the kp-th key).
-template <int KS>
-__device__ __noinline__ uint64_t compact_list(uint64_t* list, int cnt, int kp, int lane) {
-    uint64_t v[KS / 32];
+// One query's list (cnt entries: KC in shared memory, the rest in `spill`),
+// held by a warp as keys e = 32 j + lane in v[j].
+template <int KC>
+struct ListRegs {
+    static constexpr int E = (KC + SP) / 32;
+    uint64_t v[E];
+    __device__ __forceinline__ void load(const uint64_t* list, const uint64_t* spill, int cnt, int lane) {
 #pragma unroll
-    for (int i = 0; i < KS / 32; ++i) {
-        const int e = i * 32 + lane;
-        v[i] = e < cnt ? list[e] : kEmptyKey;
+        for (int j = 0; j < E; ++j) {
+            const int e = 32 * j + lane;
+            v[j] = kEmptyKey;
+            if (32 * j < cnt && e < cnt) v[j] = e < KC ? list[e] : __ldcg(spill + (e - KC));
+        }
     }
-    warp_sort<KS>(v, lane);
-    uint64_t th = kEmptyKey;
+    // the keys <= k to list[0 ..]; their number
+    __device__ __forceinline__ int store_le(uint64_t* list, uint64_t k, int lane) const {
+        int n = 0;
 #pragma unroll
-    for (int i = 0; i < KS / 32; ++i) {
-        const int e = i * 32 + lane;
-        if (e < kp) list[e] = v[i];
-        const uint64_t t = shfl_u64(v[i], (kp - 1) & 31);
-        if (i == (kp - 1) / 32) th = t;
+        for (int j = 0; j < E; ++j) {
+            const bool in = v[j] <= k;
+            const uint32_t msk = __ballot_sync(0xffffffffu, in);
+            if (in) list[n + __popc(msk & ((1u << lane) - 1u))] = v[j];
+            n += __popc(msk);
+        }
+        __syncwarp();
+        return n;
     }
-    __syncwarp();
-    return th;
+    __device__ __forceinline__ int count_le(uint64_t k) const {
+        int n = 0;
+#pragma unroll
+        for (int j = 0; j < E; ++j) n += __popc(__ballot_sync(0xffffffffu, v[j] <= k));
+        return n;
+    }
+    // A key that at least kp entries do not exceed and at most `most` do (kp <=
+    // cnt, kp <= most).  For kp <= 32 the kp-th smallest of the lanes' smallest
+    // estimates: kp lanes hold an entry at or below it.  Where that admits too
+    // many (or kp > 32), the exact kp-th key bit by bit.
+    __device__ __forceinline__ uint64_t bound(int kp, int most, int lane) const {
+        if (kp <= 32) {
+            uint32_t m = 0xffffffffu;
+#pragma unroll
+            for (int j = 0; j < E; ++j) m = min(m, (uint32_t)(v[j] >> 32));
+#pragma unroll
+            for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+                for (int d = size >> 1; d > 0; d >>= 1) {
+                    const uint32_t p = __shfl_xor_sync(0xffffffffu, m, d);
+                    const bool asc = size == 32 || (lane & size) == 0;
+                    m = ((lane & d) == 0) == asc ? min(m, p) : max(m, p);
+                }
+            const uint64_t k = ((uint64_t)__shfl_sync(0xffffffffu, m, kp - 1) << 32) | 0xffffffffull;
+            if (count_le(k) <= most && k != kEmptyKey) return k;
+        }
+        uint64_t k = 0;
+#pragma unroll 1
+        for (int b = 63; b >= 0; --b)
+            if (count_le(k | ((1ull << b) - 1ull)) < kp) k |= 1ull << b;
+        return k;
+    }
+};
+
+// v[k] of N registers by a selection tree (no indexed registers).
+template <int N>
+__device__ __forceinline__ float select_reg(const uint32_t (&v)[N], int k) {
+    if constexpr (N == 1) {
+        return __uint_as_float(v[0]);
+    } else {
+        uint32_t h[N / 2];
+#pragma unroll
+        for (int i = 0; i < N / 2; ++i) h[i] = (k & 1) ? v[2 * i + 1] : v[2 * i];
+        return select_reg<N / 2>(h, k >> 1);
+    }
+}
+
+// One candidate of one thread: value v = g + (f_res/2) acc of its row for query
+// q.  Appends its key to the query's list if the key is admitted; returns
+// whether the list went above TRIG.
+template <class C>
+__device__ __forceinline__ bool append_candidate(unsigned char* sm, const int4* iq, uint64_t* spill, int q, float v,
+                                                 uint32_t id) {
+    const uint64_t key = make_key(__int_as_float(iq[q].y) + v, id);
+    if (key > reinterpret_cast<const uint64_t*>(sm + C::Smem::tau)[q]) return false;
+    const int pos = (int)atomicAdd(reinterpret_cast<uint32_t*>(sm + C::Smem::cnt) + q, 1u);
+    if (pos < C::KC) reinterpret_cast<uint64_t*>(sm + C::Smem::lists)[q * C::KC + pos] = key;
+    else if (pos < C::KC + SP) spill[q * SP + pos - C::KC] = key;
+    return pos >= C::TRIG;
 }
 
 // P selects the operand form: 0 FP16 codes and queries (kind::f16, K = 16);
@@ -442,15 +476,21 @@ __device__ __noinline__ uint64_t compact_list(uint64_t* list, int cnt, int kp, i
 // K = 32), a stage covering 128 coordinates (two packed 64-coordinate blocks)
 // in the same 128 bytes per row of tensor memory and query tile as 64 FP16
 // coordinates; 2 the split e4m3 form of B = 5..8 codes (unpack_split), a
-// stage covering 64 coordinates whose query tile holds them twice.
+// stage covering 64 coordinates whose query tile holds them twice; 3 FP16 codes
+// and queries as two FP16 parts (FP32 precision): with a per-query power of two
+// that puts the largest coordinate in [2^13, 2^14), hi = RN16(x) and lo =
+// RN16(x - hi) hold x to 2^-23, the codes are exact, and both products add in
+// the same FP32 accumulator.  Its query tile is the hi rows, then the lo rows.
 template <class C, int P>
 __global__ void __launch_bounds__(THREADS, 1)
     scan_tc_kernel(const __grid_constant__ CUtensorMap codes_map, const __grid_constant__ CUtensorMap codes_map1,
-                   const __grid_constant__ CUtensorMap q_map, tc::Args a) {
-    constexpr bool F8 = P != 0;       // e4m3 operands
-    constexpr bool W2 = P == 1;       // two packed blocks per stage
-    constexpr int QN = C::QN, KC = C::KC, LS = C::LS, NBUF = C::NBUF, TILE_Q = C::TILE_Q, ACOL = C::ACOL;
-    constexpr int EB = C::EB, RAW_BYTES = C::RAW_BYTES;
+                   const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap q_map_lo, tc::Args a) {
+    constexpr bool F8 = P == 1 || P == 2;   // e4m3 operands
+    constexpr bool W2 = P == 1;       // two packed blocks per unit
+    constexpr bool S32 = P == 3;      // two query parts
+    constexpr bool SC = F8 || S32;    // scaled queries
+    static_assert(C::QB == (S32 ? 256 : 128), "query tile");
+    constexpr int QN = C::QN, KC = C::KC, LS = C::LS, NACC = C::NACC, TILE_Q = C::TILE_Q;
     using Smem = typename C::Smem;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -461,49 +501,45 @@ __global__ void __launch_bounds__(THREADS, 1)
     int4* s_itd = reinterpret_cast<int4*>(sm + Smem::itd);
     unsigned long long* s_tq = reinterpret_cast<unsigned long long*>(sm + Smem::tq);
     float* s_qsc = reinterpret_cast<float*>(sm + Smem::qsc);
-    const float4* s_meta = reinterpret_cast<const float4*>(sm + Smem::meta);
     const unsigned long long wlim = a.wait_ns;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nkb = a.nkb;
     const uint32_t blk = (uint32_t)(MR / 32) * 256u * (uint32_t)a.B;    // packed codes of one 128-row K block
-    const uint32_t slot_bytes = (uint32_t)RP * blk * (W2 ? 2u : 1u);
-    // an even number of raw slots: stage g uses slot g % RS and converter set
-    // g % 2, so every slot belongs to one set, which awaits its phases in order
-    // (with an odd RS a set could test a slot's parity one phase early)
-    const int RS = min(RSMAX, (int)(RAW_BYTES / slot_bytes)) & ~1;
+    const uint32_t slot_bytes = blk * (W2 ? 2u : 1u);
+    // a multiple of NSET raw slots: unit U uses slot U % RS and converter set
+    // U % NSET, so every slot belongs to one set, which awaits its phases in order
+    const int RS = min(RSMAX, (int)(C::RAW_BYTES / slot_bytes)) & ~(NSET - 1);
     int64_t nitems = *a.n_items;
     if (!ERQ_DCHECK(nitems >= 0 && nitems <= a.ck.items, a.ck.status, 7)) nitems = 0;   // uniform: every thread reads it
 
     if (tid == 0) {
         for (int s = 0; s < RSMAX; ++s) {
             mbar_init(bars + C::b_full_raw(s), 1);
-            mbar_init(bars + C::b_empty_raw(s), 128);     // the converter set of the stage
+            mbar_init(bars + C::b_empty_raw(s), 4);      // the warps of the unit's converter set
         }
         for (int s = 0; s < LS; ++s) {
             mbar_init(bars + C::b_full_q(s), 1);
-            mbar_init(bars + C::b_empty_st(s), RP);
-            for (int b = 0; b < RP; ++b) mbar_init(bars + C::b_full_a(s, b), 128);
+            mbar_init(bars + C::b_empty_q(s), 1);
         }
-        for (int u = 0; u < NBUF; ++u)
-            for (int b = 0; b < RP; ++b) {
-                mbar_init(bars + C::b_tfull(u, b), 1);
-                mbar_init(bars + C::b_tempty(u, b), 128);
-            }
+        for (int s = 0; s < AS; ++s) {
+            mbar_init(bars + C::b_full_a(s), 4);
+            mbar_init(bars + C::b_empty_a(s), 1);
+        }
+        for (int u = 0; u < NACC; ++u) {
+            mbar_init(bars + C::b_tfull(u), 1);
+            mbar_init(bars + C::b_tempty(u), NEP);
+        }
         for (int m = 0; m < MS; ++m) {
             mbar_init(bars + C::b_full_meta(m), 1);
-            mbar_init(bars + C::b_empty_meta(m), 128);
+            mbar_init(bars + C::b_empty_meta(m), NEP);
         }
         for (int i = 0; i < 2; ++i) {
-            mbar_init(bars + C::b_full_item(i), 32);
+            mbar_init(bars + C::b_full_item(i), 1);
             mbar_init(bars + C::b_empty_item(i), kItemReleasers);
         }
-        mbar_init(bars + C::b_done(), RP);
+        mbar_init(bars + C::b_done(), 1);
         mbar_init(bars + C::b_never(), 1);
-        for (int t = 0; t < EB; ++t) {
-            mbar_init(bars + C::b_tile_full(t), 128);       // the four estimate-tile warps
-            mbar_init(bars + C::b_tile_empty(t), 32 * NFX); // the filter warps
-        }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -516,10 +552,15 @@ __global__ void __launch_bounds__(THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    // one arrival for the warp, after everything its lanes did
+    auto arrive_warp = [&](uint32_t bar) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar);
+    };
 
     if (warp == W_LD) {
         // ------------------------------------------------------------ code loader, item publisher
-        uint32_t g = 0, rbg = 0, li = 0;
+        uint32_t U = 0, rs = 0, rph = 1, blkc = 0, li = 0;     // unit, its raw slot, the slot's awaited phase
         bool ok = true;
         int64_t item = blockIdx.x;
         const uint64_t pol_codes = a.codes_shared ? l2_evict_normal() : l2_evict_first();
@@ -554,12 +595,11 @@ __global__ void __launch_bounds__(THREADS, 1)
                     const int4 v = pv[k];
                     s_iq[ib * QN + q] = v;
                     s_tq[ib * QN + q] = v.x >= 0 ? __ldcg(a.tq + v.x) : kEmptyKey;
-                    if (F8) s_qsc[ib * QN + q] = v.x >= 0 ? a.qscale[v.x] : 0.f;
+                    if (SC) s_qsc[ib * QN + q] = v.x >= 0 ? a.qscale[v.x] : 0.f;
                 }
             }
             if (lane == 0) s_itd[ib] = d;
-            __syncwarp();
-            mbar_arrive(bars + C::b_full_item(ib));
+            arrive_warp(bars + C::b_full_item(ib));
             if (!have) break;
             const int64_t rb0 = rb0_of(d);                 // first padded row (multiple of 32)
             const int nrows = d.z;
@@ -579,37 +619,40 @@ __global__ void __launch_bounds__(THREADS, 1)
             for (int r = 0; r < nrows && ok; r += RP * MR) {
                 if (r + RP * MR >= nrows) claim_next();
                 const int nb = min(RP, (nrows - r + MR - 1) / MR);     // row blocks in this stage group
-                for (int bb = 0; bb < nb && ok; ++bb, ++rbg) {
+                for (int bb = 0; bb < nb && ok; ++bb, ++blkc) {
                     const int nr = min(MR, nrows - r - bb * MR);
-                    const int m = rbg % MS;
-                    if (!mbar_wait_warp(bars + C::b_empty_meta(m), ((rbg / MS) & 1) ^ 1, abort_flag, wlim)) {
+                    const int m = blkc % MS;
+                    if (!mbar_wait_warp(bars + C::b_empty_meta(m), ((blkc / MS) & 1) ^ 1, abort_flag, wlim)) {
                         ok = false;
                         break;
                     }
-                    if (lane == 0) {
+                    if (elect_one()) {
                         mbar_arrive_expect_tx(bars + C::b_full_meta(m), (uint32_t)nr * 16u);
                         bulk_load(smem_u32(sm + Smem::meta + m * MR * 16), a.rowmeta + rb0 + r + bb * MR,
                                   (uint32_t)nr * 16u, bars + C::b_full_meta(m));
                     }
                 }
-                for (int kb = 0; kb < nkb && ok; ++kb, ++g) {
-                    const int s = g % RS;
-                    if (!mbar_wait_warp(bars + C::b_empty_raw(s), ((g / RS) & 1) ^ 1, abort_flag, wlim)) {
-                        ok = false;
-                        break;
-                    }
-                    if (lane == 0) {
-                        // whole 32-row tiles of the item's rows only: a block of
-                        // fewer than 128 rows takes its tiles one by one (the rows
-                        // past them are never admitted: the filters test rr < nr)
-                        const int rem = nrows - r;
-                        const uint32_t tiles = (uint32_t)min(RP * MR / 32, (rem + 31) >> 5);
-                        mbar_arrive_expect_tx(bars + C::b_full_raw(s), tiles * 256u * (uint32_t)a.B * (W2 ? 2u : 1u));
-                        for (int bb = 0; bb < nb; ++bb) {
-                            const uint32_t dst = smem_u32(sm + Smem::raw + s * slot_bytes + bb * blk * (W2 ? 2 : 1));
+                for (int kb = 0; kb < nkb && ok; ++kb)
+                    for (int bb = 0; bb < nb; ++bb, ++U) {
+                        const uint32_t s = rs;
+                        if (!mbar_wait_warp(bars + C::b_empty_raw(s), rph, abort_flag, wlim)) {
+                            ok = false;
+                            break;
+                        }
+                        if (++rs == (uint32_t)RS) {
+                            rs = 0;
+                            rph ^= 1u;
+                        }
+                        if (elect_one()) {
+                            // whole 32-row tiles of the item's rows only: a block of
+                            // fewer than 128 rows takes its tiles one by one (the rows
+                            // past them are never admitted)
+                            const int nt = min(MR / 32, ((nrows - r - bb * MR) + 31) >> 5);
                             const int tile = (int)((rb0 + r + bb * MR) >> 5);
-                            const int nt = min(MR / 32, ((rem - bb * MR) + 31) >> 5);
-                            // (the second block of the last P = 1 stage may lie past D: the TMA fills zeros)
+                            mbar_arrive_expect_tx(bars + C::b_full_raw(s),
+                                                  (uint32_t)nt * 256u * (uint32_t)a.B * (W2 ? 2u : 1u));
+                            const uint32_t dst = smem_u32(sm + Smem::raw + s * slot_bytes);
+                            // (the second block of the last P = 1 unit may lie past D: the TMA fills zeros)
                             for (int h = 0; h < (W2 ? 2 : 1); ++h) {
                                 const int kk = W2 ? 2 * kb + h : kb;
                                 if (nt == MR / 32) {
@@ -622,21 +665,20 @@ __global__ void __launch_bounds__(THREADS, 1)
                                 }
                             }
                         }
+                        __syncwarp();
                     }
-                    __syncwarp();
-                }
             }
             if (!ok) break;
             if (!claimed) claim_next();
         }
         // drain: every copy this warp issued has landed before the CTA exits
-        for (uint32_t k = 0; k < (uint32_t)RS && k < g; ++k) {
-            const uint32_t gg = g - 1 - k;
-            mbar_wait_drain(bars + C::b_full_raw(gg % RS), (gg / RS) & 1);
+        for (uint32_t k = 0; k < (uint32_t)RS && k < U; ++k) {
+            const uint32_t g = U - 1 - k;
+            mbar_wait_drain(bars + C::b_full_raw(g % (uint32_t)RS), (g / (uint32_t)RS) & 1);
         }
-        for (uint32_t k = 0; k < MS && k < rbg; ++k) {
-            const uint32_t gg = rbg - 1 - k;
-            mbar_wait_drain(bars + C::b_full_meta(gg % MS), (gg / MS) & 1);
+        for (uint32_t k = 0; k < MS && k < blkc; ++k) {
+            const uint32_t g = blkc - 1 - k;
+            mbar_wait_drain(bars + C::b_full_meta(g % MS), (g / MS) & 1);
         }
         __syncwarp();
     } else if (warp >= W_QL && warp < W_QL + NQL) {
@@ -666,95 +708,99 @@ __global__ void __launch_bounds__(THREADS, 1)
             for (int t = 0; t < nsteps; ++t, ++g) {
                 if (g % NQL != qj) continue;
                 const int s = g % LS, kb = t % nkb;
-                if (!mbar_wait_warp(bars + C::b_empty_st(s), ((g / LS) & 1) ^ 1, abort_flag, wlim)) {
+                if (!mbar_wait_warp(bars + C::b_empty_q(s), ((g / LS) & 1) ^ 1, abort_flag, wlim)) {
                     ok = false;
                     break;
                 }
-                if (lane == 0) mbar_arrive_expect_tx(bars + C::b_full_q(s), (uint32_t)npad * 128u);
+                if (lane == 0) mbar_arrive_expect_tx(bars + C::b_full_q(s), (uint32_t)npad * (uint32_t)C::QB);
                 __syncwarp();
                 if (4 * lane < npad)
                     tma_gather4_hint(smem_u32(sm + Smem::q + s * TILE_Q + lane * 512), &q_map, kb * 128, y[0], y[1],
                                      y[2], y[3], bars + C::b_full_q(s), pol_q);
+                if (S32 && 4 * lane < npad)
+                    tma_gather4_hint(smem_u32(sm + Smem::q + s * TILE_Q + QN * 128 + lane * 512), &q_map_lo, kb * 128,
+                                     y[0], y[1], y[2], y[3], bars + C::b_full_q(s), pol_q);
                 __syncwarp();
             }
             if (!ok) break;
-            mbar_arrive(bars + C::b_empty_item(ib));
+            arrive_warp(bars + C::b_empty_item(ib));
         }
         for (uint32_t k = 0; k < LS && k < g; ++k) {     // (the stages this loader issued)
             const uint32_t gg = g - 1 - k;
             if (gg % NQL == qj) mbar_wait_drain(bars + C::b_full_q(gg % LS), (gg / LS) & 1);
         }
         __syncwarp();
-    } else if (warp >= W_CV && warp < W_CV + 8) {
+    } else if (warp >= W_CV && warp < W_CV + 4 * NSET) {
         // ------------------------------------------------------------ converters
-        // Two sets of four warps take alternate stages (set cs the stages with
-        // g % 2 == cs) and convert both row blocks of each: thread = one row of a
-        // block (TMEM lane 32 (w % 4) + lane); the TMEM stores of the two blocks
-        // are waited for once, while the other set converts the next stage.
-        const int cs = (warp - W_CV) >> 2, qt = warp & 3;
+        // Set cs converts the units U with U % NSET == cs: thread = one row of the
+        // block (TMEM lane 32 (w % 4) + lane).
+        const uint32_t cs = (uint32_t)(warp - W_CV) >> 2;
+        const int qt = warp & 3;
         const int r = qt * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(qt * 32) << 16;
         const int B = a.B;
         const int roff = (r >> 5) * 256 * B + (r & 31) * 8;   // word 0 of row r in a 128-row block
-        uint32_t g = 0;
+        uint32_t U0 = 0;                                       // units before this item
+        uint32_t rs = cs, rph = 0;                             // raw slot of the set's next unit, its phase
         bool ok = true;
         for (uint32_t li = 0; ok; ++li) {
             const int ib = li & 1;
             if (!mbar_wait_warp(bars + C::b_full_item(ib), (li >> 1) & 1, abort_flag, wlim)) break;
             const int4 d = s_itd[ib];
             if (d.w < 0) break;
-            const int nrows = d.z;
-            for (int r0 = 0; r0 < nrows && ok; r0 += RP * MR) {
-                const int nb = min(RP, (nrows - r0 + MR - 1) / MR);
-                for (int kb = 0; kb < nkb; ++kb, ++g) {
-                    if ((int)(g & 1) != cs) continue;
-                    const int s = g % LS, rs = g % RS;
-                    // the stage's TMEM columns are free (its previous MMAs completed)
-                    // and its raw codes have landed
-                    if (!mbar_wait_warp(bars + C::b_empty_st(s), ((g / LS) & 1) ^ 1, abort_flag, wlim) ||
-                        !mbar_wait_warp(bars + C::b_full_raw(rs), (g / RS) & 1, abort_flag, wlim)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    for (int bb = 0; bb < nb; ++bb) {                  // warp-uniform
-                        uint32_t w[32];
-                        const unsigned char* src = sm + Smem::raw + rs * slot_bytes + bb * blk * (W2 ? 2 : 1) + roff;
-                        if (W2) {
-                            // two packed blocks -> 128 e4m3 codes, four per column
-#pragma unroll
-                            for (int hb = 0; hb < 2; ++hb) {
-                                uint32_t h[32];
-                                unpack_codes_b(B, src + hb * blk, h);
-#pragma unroll
-                                for (int c = 0; c < 16; ++c)
-                                    w[16 * hb + c] = __byte_perm(half2_to_e4m3_pair(h[2 * c]),
-                                                                 half2_to_e4m3_pair(h[2 * c + 1]), 0x6420u);
-                            }
-                        } else if (P == 2) {
-                            unpack_split_b(B, src, w);
-                        } else {
-                            unpack_codes_b(B, src, w);
-                        }
-                        ERQ_TMEM_ST32(tmem + lane_addr + ACOL + (s * RP + bb) * (KB / 2), w);
-                    }
-                    mbar_arrive(bars + C::b_empty_raw(rs));        // the raw slot may be refilled
-                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                    tc_fence_before();
-                    mbar_arrive(bars + C::b_full_a(s, 0));
-                    mbar_arrive(bars + C::b_full_a(s, 1));
+            const uint32_t nu = (uint32_t)((d.z + MR - 1) / MR) * (uint32_t)nkb;
+            for (uint32_t U = U0 + ((cs - U0) & (uint32_t)(NSET - 1)); U < U0 + nu; U += NSET) {
+                const uint32_t s = U % AS;
+                // the slot's TMEM columns are free (its previous MMAs completed)
+                // and its raw codes have landed
+                if (!mbar_wait_warp(bars + C::b_full_raw(rs), rph, abort_flag, wlim)) {
+                    ok = false;
+                    break;
                 }
+                uint32_t w[32];
+                const unsigned char* src = sm + Smem::raw + rs * slot_bytes + roff;
+                if (W2) {
+                    // two packed blocks -> 128 e4m3 codes, four per column
+#pragma unroll
+                    for (int hb = 0; hb < 2; ++hb) {
+                        uint32_t h[32];
+                        unpack_codes_b(B, src + hb * blk, h);
+#pragma unroll
+                        for (int c = 0; c < 16; ++c)
+                            w[16 * hb + c] = __byte_perm(half2_to_e4m3_pair(h[2 * c]),
+                                                         half2_to_e4m3_pair(h[2 * c + 1]), 0x6420u);
+                    }
+                } else if (P == 2) {
+                    unpack_split_b(B, src, w);
+                } else {
+                    unpack_codes_b(B, src, w);
+                }
+                if (!mbar_wait_warp(bars + C::b_empty_a(s), ((U / AS) & 1) ^ 1, abort_flag, wlim)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                ERQ_TMEM_ST32(tmem + lane_addr + ACOL + s * (KB / 2), w);
+                arrive_warp(bars + C::b_empty_raw(rs));        // the raw slot may be refilled
+                rs += NSET;
+                if (rs >= (uint32_t)RS) {
+                    rs -= (uint32_t)RS;
+                    rph ^= 1u;
+                }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                tc_fence_before();
+                arrive_warp(bars + C::b_full_a(s));
             }
             if (!ok) break;
-            mbar_arrive(bars + C::b_empty_item(ib));
+            U0 += nu;
+            arrive_warp(bars + C::b_empty_item(ib));
         }
-    } else if (warp == W_MMA || warp == W_MMA + 1) {
-        // ------------------------------------------------------------ MMA issuers
-        // Issuer b runs the accumulation chain of row block b of each stage group
-        // (tcgen05.mma issue stalls the issuing thread, so two issuers keep two
-        // chains in flight); both commit every stage to its release barrier.
-        const int b = warp - W_MMA;
-        uint32_t g = 0, u = 0;
+    } else if (warp == W_MMA) {
+        // ------------------------------------------------------------ MMA issuer
+        // One elected thread keeps the tensor pipe fed: with the code operand in
+        // tensor memory it issues an MMA per 35 cycles at N = 64 and 64 at
+        // N = 128, the tensor core's own rate (32 and 64).
+        uint32_t g = 0, U = 0, blkc = 0;
         bool ok = true;
         for (uint32_t li = 0; ok; ++li) {
             const int ib = li & 1;
@@ -763,244 +809,218 @@ __global__ void __launch_bounds__(THREADS, 1)
             if (d.w < 0) break;
             const uint32_t idesc = idesc_f16(MR, npad_of(d.w));
             for (int r0 = 0; r0 < d.z && ok; r0 += RP * MR) {
-                const bool has = b < min(RP, (d.z - r0 + MR - 1) / MR);
-                const int buf = u % NBUF;
-                if (has) {
-                    if (!mbar_wait_warp(bars + C::b_tempty(buf, b), ((u / NBUF) & 1) ^ 1, abort_flag, wlim)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                }
-                const uint32_t dt = tmem + (uint32_t)((buf * RP + b) * QN);
-                for (int kb = 0; kb < nkb; ++kb, ++g) {
+                const int nb = min(RP, (d.z - r0 + MR - 1) / MR);
+                for (int kb = 0; kb < nkb && ok; ++kb, ++g) {
                     const int s = g % LS;
-                    if (b == 0 && (long long)g == a.stall_stage &&
+                    if ((long long)g == a.stall_stage &&
                         !mbar_wait_warp(bars + C::b_never(), 0, abort_flag, wlim)) {
                         ok = false;                                // (always: nothing arrives on it)
                         break;
                     }
-                    if (!mbar_wait_warp(bars + C::b_full_a(s, b), (g / LS) & 1, abort_flag, wlim) ||
-                        !mbar_wait_warp(bars + C::b_full_q(s), (g / LS) & 1, abort_flag, wlim)) {
+                    if (!mbar_wait_warp(bars + C::b_full_q(s), (g / LS) & 1, abort_flag, wlim)) {
                         ok = false;
                         break;
                     }
-                    tc_fence_after();
-                    const uint32_t ta = tmem + ACOL + (s * RP + b) * (KB / 2);
                     const uint64_t tq = sdesc(smem_u32(sm + Smem::q + s * TILE_Q));
-                    if (elect_one()) {
-                        if (has) {
+                    for (int b = 0; b < nb; ++b, ++U) {
+                        const uint32_t buf = (blkc + b) % NACC, as = U % AS;
+                        if (kb == 0 && !mbar_wait_warp(bars + C::b_tempty(buf), (((blkc + b) / NACC) & 1) ^ 1,
+                                                       abort_flag, wlim)) {
+                            ok = false;
+                            break;
+                        }
+                        if (!mbar_wait_warp(bars + C::b_full_a(as), (U / AS) & 1, abort_flag, wlim)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint32_t ta = tmem + ACOL + as * (KB / 2), dt = tmem + buf * QN;
+                        if (elect_one()) {
 #pragma unroll
                             for (int k = 0; k < KB / 16; ++k) {         // 32 bytes of K per instruction
                                 if (F8) mma_f8_ta(dt, ta + k * 8, tq + 2 * k, idesc, (kb | k) != 0);
                                 else mma_f16_ta(dt, ta + k * 8, tq + 2 * k, idesc, (kb | k) != 0);
                             }
+                            if (S32) {
+#pragma unroll
+                                for (int k = 0; k < KB / 16; ++k)
+                                    mma_f16_ta(dt, ta + k * 8, tq + 2 * k + (QN * 128 >> 4), idesc, 1);
+                            }
+                            mma_commit(bars + C::b_empty_a(as));       // code slot free
+                            if (b == nb - 1) mma_commit(bars + C::b_empty_q(s));
+                            if (kb == nkb - 1) mma_commit(bars + C::b_tfull(buf));
                         }
-                        mma_commit(bars + C::b_empty_st(s));          // query tile and TMEM stage free
-                        if (has && kb == nkb - 1) mma_commit(bars + C::b_tfull(buf, b));
+                        __syncwarp();
                     }
-                    __syncwarp();
                 }
-                if (has) ++u;
+                blkc += nb;
             }
             if (!ok) break;
-            mbar_arrive(bars + C::b_empty_item(ib));
+            arrive_warp(bars + C::b_empty_item(ib));
         }
         // all issued MMAs complete before TMEM is released
         if (elect_one()) mma_commit(bars + C::b_done());
         __syncwarp();
         mbar_wait_drain(bars + C::b_done(), 0);
         __syncwarp();
-    } else if (warp < W_CV) {
-        // ------------------------------------------------------------ estimate tiles
-        // Warp w moves TMEM lanes 32w..32w+31 (its 32 rows, all queries) of each
-        // finished row-block accumulator into a query-major estimate tile and
-        // frees the accumulator.
-        float* s_est = reinterpret_cast<float*>(sm + Smem::est);
-        uint32_t* s_ids = reinterpret_cast<uint32_t*>(sm + Smem::ids);
-        const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-        const int row = warp * 32 + lane;
-        uint32_t blk = 0, rbg = 0, u[RP] = {};
-        bool ok = true;
-        for (uint32_t li = 0; ok; ++li) {
+    } else {
+        // ------------------------------------------------------------ epilogue
+        uint64_t* lists = reinterpret_cast<uint64_t*>(sm + Smem::lists);
+        uint64_t* s_tau = reinterpret_cast<uint64_t*>(sm + Smem::tau);
+        float* s_thr = reinterpret_cast<float*>(sm + Smem::thr);
+        uint32_t* s_cnt = reinterpret_cast<uint32_t*>(sm + Smem::cnt);
+        const float4* s_meta = reinterpret_cast<const float4*>(sm + Smem::meta);
+        uint64_t* spill = a.spill + (int64_t)blockIdx.x * QN * SP;
+        constexpr int CSTEP = 16 * (NEP / 4);             // 16-column groups go round the warps of a quarter
+        const int quarter = warp & 3, par = warp >> 2;
+        const int row = quarter * 32 + lane;
+        const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
+        const int kp = a.kp;
+        uint32_t blkc = 0;
+        for (uint32_t li = 0;; ++li) {
             const int ib = li & 1;
-            if (!mbar_wait_warp(bars + C::b_full_item(ib), (li >> 1) & 1, abort_flag, wlim)) break;
+            const bool got = mbar_wait_warp(bars + C::b_full_item(ib), (li >> 1) & 1, abort_flag, wlim);
+            // every warp takes the same decision (and has written its lists of the last item)
+            if (bar_or(BAR_EP, 32 * NEP, !got)) break;
             const int4 d = s_itd[ib];
             if (d.w < 0) break;
-            const int nrows = d.z, npad = npad_of(d.w);
-            for (int r0 = 0; r0 < nrows && ok; r0 += RP * MR) {
-                const int nb = min(RP, (nrows - r0 + MR - 1) / MR);
-                for (int rb = 0; rb < nb; ++rb, ++blk) {
-                    const uint32_t mrb = rbg + rb;
-                    const int m = mrb % MS, t = blk % EB, buf = u[rb] % NBUF;
-                    if (!mbar_wait_warp(bars + C::b_full_meta(m), (mrb / MS) & 1, abort_flag, wlim) ||
-                        !mbar_wait_warp(bars + C::b_tfull(buf, rb), (u[rb] / NBUF) & 1, abort_flag, wlim) ||
-                        !mbar_wait_warp(bars + C::b_tile_empty(t), ((blk / EB) & 1) ^ 1, abort_flag, wlim)) {
-                        ok = false;
-                        break;
-                    }
+            const int nrows = d.z, nqi = d.w, npad = npad_of(d.w);
+            const int4* iq = s_iq + ib * QN;
+            for (int q = tid; q < QN; q += 32 * NEP) {
+                const uint64_t t = s_tq[ib * QN + q];
+                s_tau[q] = t;
+                s_cnt[q] = 0u;
+                s_thr[q] = q < nqi ? relaxed_threshold(t == kEmptyKey ? INFINITY : key_value(t), __int_as_float(iq[q].y))
+                                   : __int_as_float(0x7fc00000);
+            }
+            bar_sync(BAR_EP, 32 * NEP);
+            bool dead = false;
+            for (int r = 0; r < nrows; r += MR, ++blkc) {
+                const uint32_t m = blkc % MS, buf = blkc % NACC;
+                bool need = false;                                  // a list of mine went above TRIG
+                dead = !mbar_wait_warp(bars + C::b_full_meta(m), (blkc / MS) & 1, abort_flag, wlim) ||
+                       !mbar_wait_warp(bars + C::b_tfull(buf), (blkc / NACC) & 1, abort_flag, wlim);
+                if (!dead) {
                     tc_fence_after();
-                    float* est_t = s_est + t * (QN * MR);
                     float4 mt = s_meta[m * MR + row];
-                    s_ids[t * MR + row] = __float_as_uint(mt.z);
+                    const uint32_t id = __float_as_uint(mt.z);
                     if (a.ip) {                                     // -<c, q_r> + (f_res / 4) acc: no g, half the factor
                         mt.x = 0.f;
                         mt.y *= 0.5f;
                     }
-                    if (row >= min(MR, nrows - r0 - rb * MR)) {    // past the block's rows: NaN, which no
-                        mt.x = __int_as_float(0x7fc00000);         // threshold admits
+                    if (row >= nrows - r) {                         // past the block's rows: NaN, which no
+                        mt.x = __int_as_float(0x7fc00000);          // threshold admits
                         mt.y = 0.f;
                     }
-                    const uint32_t tacc = tmem + lane_base + (uint32_t)((buf * RP + rb) * QN);
-#pragma unroll 1
-                    for (int cc = 0; cc < npad; cc += 32) {
-                        uint32_t v[32];
-                        ERQ_TMEM_LD32(tacc + cc, v);
-                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                        if (cc + 32 >= npad) {                     // the last columns are in registers:
-                            tc_fence_before();                     // the accumulator is free
-                            mbar_arrive(bars + C::b_tempty(buf, rb));
-                        }
-                        if (F8) {                                  // e4m3 queries carry a power-of-two scale (exact)
-                            const float* sc = s_qsc + ib * QN + cc;
+                    arrive_warp(bars + C::b_empty_meta(m));
+                    const uint32_t tacc = tmem + lane_base + buf * QN;
+                    // 16-column groups 16 (par + 4 g) .. of this warp, all loaded at once so
+                    // that the accumulator is released before the compares
+                    constexpr int NG = QN > CSTEP ? QN / CSTEP : 1;
+                    uint32_t v[16 * NG];
 #pragma unroll
-                            for (int i = 0; i < 32; ++i)
-                                est_t[(cc + i) * MR + row] = fmaf(mt.y, __uint_as_float(v[i]) * sc[i], mt.x);
-                        } else {
+                    for (int g = 0; g < NG; ++g)
+                        if (16 * par + CSTEP * g < npad) ERQ_TMEM_LD16(tacc + 16 * par + CSTEP * g, (v + 16 * g));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    tc_fence_before();
+                    arrive_warp(bars + C::b_tempty(buf));
+                    // straight-line: the compares into a mask
+                    uint32_t mine = 0u;
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) est_t[(cc + i) * MR + row] = fmaf(mt.y, __uint_as_float(v[i]), mt.x);
+                    for (int g = 0; g < NG; ++g) {
+                        const int cc = 16 * par + CSTEP * g;
+                        if (cc < npad) {                            // (uniform)
+#pragma unroll
+                            for (int i = 0; i < 16; i += 4) {
+                                const float4 th = *reinterpret_cast<const float4*>(s_thr + cc + i);
+                                float4 sc = make_float4(1.f, 1.f, 1.f, 1.f);
+                                if (SC) sc = *reinterpret_cast<const float4*>(s_qsc + ib * QN + cc + i);
+                                const float t4[4] = {th.x, th.y, th.z, th.w}, s4[4] = {sc.x, sc.y, sc.z, sc.w};
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) {
+                                    float x = __uint_as_float(v[16 * g + i + j]);
+                                    if (SC) x *= s4[j];             // a power of two: exact
+                                    if (fmaf(mt.y, x, mt.x) <= t4[j]) mine |= 1u << (16 * g + i + j);
+                                }
+                            }
                         }
                     }
-                    ++u[rb];
-                    mbar_arrive(bars + C::b_empty_meta(m));
-                    mbar_arrive(bars + C::b_tile_full(t));
-                }
-                rbg += nb;
-            }
-            if (!ok) break;
-            mbar_arrive(bars + C::b_empty_item(ib));
-        }
-    } else {
-        // ------------------------------------------------------------ filters
-        // NFX warps; warp f owns the query slots q = f + NFX j of every item and
-        // filters their rows of each estimate tile (float pre-filter against the
-        // threshold, exact keys, ballots) into per-query candidate lists; a full
-        // list is compacted by a warp bitonic sort to its k' smallest.  A query
-        // starts from the smallest k'-th key published so far by its items, which
-        // is never below its final k'-th key, so each list stays a superset of
-        // what the item contributes to the query's top-k'.
-        const float* s_est = reinterpret_cast<const float*>(sm + Smem::est);
-        uint64_t* lists_s = reinterpret_cast<uint64_t*>(sm + Smem::lists);
-        // query q's candidate list: shared memory, or its output slot of the item
-        auto list_of = [&](const int4* iq, int q) -> uint64_t* {
-            if (C::LG) return a.inter + ((int64_t)(uint32_t)iq[q].z | ((int64_t)iq[q].w << 32)) * KC;
-            return lists_s + q * KC;
-        };
-        const uint32_t* s_ids = reinterpret_cast<const uint32_t*>(sm + Smem::ids);
-        const int fw = warp - W_FX;
-        const uint32_t below = (1u << lane) - 1u;
-        const int kp = a.kp;
-        uint32_t blk = 0;
-        bool ok = true;
-        for (uint32_t li = 0; ok; ++li) {
-            const int ib = li & 1;
-            if (!mbar_wait_warp(bars + C::b_full_item(ib), (li >> 1) & 1, abort_flag, wlim)) break;
-            const int4 d = s_itd[ib];
-            if (d.w < 0) break;
-            const int nrows = d.z, nqi = d.w;
-            const int4* iq = s_iq + ib * QN;
-            // lane j holds the state of the warp's j-th query slot q = fw + NFX j:
-            // its distance term, admission threshold (key and float), list fill
-            // and the threshold relaxed into the estimate tile's units
-            const int nown = nqi > fw ? (nqi - fw + NFX - 1) / NFX : 0;
-            float my_dq = 0.f, my_tf = -INFINITY, my_thr = -INFINITY;
-            uint64_t my_tau = 0;
-            int my_cnt = 0;
-            if (lane < nown) {
-                const int q = fw + NFX * lane;
-                my_dq = __int_as_float(iq[q].y);
-                my_tau = s_tq[ib * QN + q];
-                my_tf = my_tau == kEmptyKey ? INFINITY : key_value(my_tau);
-                my_thr = relaxed_threshold(my_tf, my_dq);
-            }
-            for (int r = 0; r < nrows; r += MR, ++blk) {
-                const int nr = min(MR, nrows - r);
-                const int t = blk % EB;
-                if (!mbar_wait_warp(bars + C::b_tile_full(t), (blk / EB) & 1, abort_flag, wlim)) {
-                    ok = false;
-                    break;
-                }
-                const float* est_t = s_est + t * (QN * MR);
-                const uint32_t* ids_t = s_ids + t * MR;
-                // the 128 rows of each owned query, rows 4 lane .. 4 lane + 3 in
-                // lane `lane` (rows past the block are NaN): one vote against the
-                // relaxed threshold (a superset of the float test below, which is
-                // a superset of the key test), then per row group the float
-                // test and exact keys
-                for (int jj = 0; jj < nown; ++jj) {
-                    const int q = fw + NFX * jj;
-                    const float thr = __shfl_sync(0xffffffffu, my_thr, jj);
-                    const float4 v4 = *reinterpret_cast<const float4*>(est_t + q * MR + 4 * lane);
-                    if (!__any_sync(0xffffffffu, v4.x <= thr || v4.y <= thr || v4.z <= thr || v4.w <= thr)) continue;
-                    const float dq = __shfl_sync(0xffffffffu, my_dq, jj);
-                    float tf = __shfl_sync(0xffffffffu, my_tf, jj);
-                    uint64_t tau = shfl_u64(my_tau, jj);
-                    int cnt = __shfl_sync(0xffffffffu, my_cnt, jj);
-                    const float e[4] = {dq + v4.x, dq + v4.y, dq + v4.z, dq + v4.w};
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int rr = 4 * lane + j;
-                        const bool pre = rr < nr && e[j] <= tf;
-                        if (!__any_sync(0xffffffffu, pre)) continue;
-                        const uint64_t key = make_key(e[j], ids_t[rr]);
-                        bool pass = pre && key < tau;
-                        uint32_t msk = __ballot_sync(0xffffffffu, pass);
-                        if (msk == 0u) continue;
-                        if (cnt + __popc(msk) > KC) {
-                            // full: keep the k' smallest (KC - k' >= 32 leaves
-                            // room for a group), then test the group again
-                            tau = compact_list<C::KS>(list_of(iq, q), cnt, kp, lane);
-                            tf = key_value(tau);
-                            cnt = kp;
-                            // k' keys of this query are now <= tau and stay in
-                            // its lists (a later compaction keeps the k'
-                            // smallest), so tau bounds its other items too
-                            if (lane == 0) atomicMin(a.tq + iq[q].x, (unsigned long long)tau);
-                            pass = pass && key < tau;
-                            msk = __ballot_sync(0xffffffffu, pass);
-                            if (msk == 0u) continue;
+                    // every thread appends its own candidates: as many rounds as the
+                    // thread with the most has, usually two or three
+                    while (__any_sync(0xffffffffu, mine != 0u)) {
+                        if (mine != 0u) {
+                            const int i = __ffs(mine) - 1, q = 16 * par + (i & 15) + CSTEP * (i >> 4);
+                            mine &= mine - 1u;
+                            float x = select_reg<16 * NG>(v, i);
+                            if (SC) x *= s_qsc[ib * QN + q];
+                            need |= append_candidate<C>(sm, iq, spill, q, fmaf(mt.y, x, mt.x), id);
                         }
-                        if (pass) list_of(iq, q)[cnt + __popc(msk & below)] = key;
-                        cnt += __popc(msk);
                         __syncwarp();
                     }
-                    if (lane == jj) {
-                        my_cnt = cnt;
-                        my_tau = tau;
-                        if (tf != my_tf) my_thr = relaxed_threshold(tf, dq);
-                        my_tf = tf;
+                }
+                // every candidate of the block is in its list; the lists above TRIG are
+                // cut before the next block adds to them
+                if (!bar_or(BAR_EP, 32 * NEP, need || dead)) continue;
+                if (!dead) {
+                    // lane j looks at query warp + NEP j
+                    const int ql = warp + NEP * lane;
+                    for (uint32_t todo = __ballot_sync(0xffffffffu, ql < nqi && s_cnt[min(ql, QN - 1)] > (uint32_t)C::TRIG);
+                         todo; todo &= todo - 1u) {
+                        const int q = warp + NEP * (__ffs(todo) - 1);
+                        int n = (int)s_cnt[q];
+                        ListRegs<KC> L;
+                        L.load(lists + q * KC, spill + q * SP, n, lane);
+                        const uint64_t k = L.bound(kp, C::TRIG, lane);
+                        __syncwarp();
+                        n = L.store_le(lists + q * KC, k, lane);    // (kp <= n, so k is below the empty key)
+                        if (lane == 0) {
+                            s_cnt[q] = (uint32_t)n;
+                            s_tau[q] = k;
+                            s_thr[q] = relaxed_threshold(key_value(k), __int_as_float(iq[q].y));
+                            // k' keys of this query are <= k and stay in its lists, so k
+                            // bounds its other items too
+                            atomicMin(a.tq + iq[q].x, (unsigned long long)k);
+                        }
+                        __syncwarp();
                     }
                 }
-                mbar_arrive(bars + C::b_tile_empty(t));
-            }
-            if (!ok) break;
-            for (int jj = 0; jj < nown; ++jj) {                 // write this warp's lists
-                const int q = fw + NFX * jj;
-                int cnt = __shfl_sync(0xffffffffu, my_cnt, jj);
-                if (cnt >= kp) {                                 // keep the k' smallest; publish the k'-th
-                    const uint64_t th = compact_list<C::KS>(list_of(iq, q), cnt, kp, lane);
-                    cnt = kp;
-                    if (lane == 0) atomicMin(a.tq + iq[q].x, (unsigned long long)th);
+                if (bar_or(BAR_EP, 32 * NEP, dead)) {
+                    dead = true;
+                    break;
                 }
-                const int64_t L = (int64_t)(uint32_t)iq[q].z | ((int64_t)iq[q].w << 32);
-                if (!ERQ_DCHECK(L >= 0 && L < a.ck.lists && cnt >= 0 && cnt <= KC, a.ck.status, 6)) continue;
-                uint64_t* dst = a.inter + L * KC;
-                if (!C::LG)
-                    for (int e = lane; e < cnt; e += 32) dst[e] = lists_s[q * KC + e];
-                if (lane == 0) a.inter_cnt[L] = cnt;
             }
-            __syncwarp();
-            mbar_arrive(bars + C::b_empty_item(ib));
+            if (dead) break;                                        // (uniform: decided at the barrier)
+            // write the lists (lane j: query warp + NEP j); a list of k' or more keys
+            // is cut first and bounds the query's other items
+            {
+                const int ql = warp + NEP * lane;
+                int cl = ql < nqi ? (int)s_cnt[ql] : 0;
+                int64_t ol = 0;
+                if (ql < nqi) {
+                    ol = (int64_t)(uint32_t)iq[ql].z | ((int64_t)iq[ql].w << 32);
+                    if (!ERQ_DCHECK(ol >= 0 && ol < a.ck.lists && cl >= 0 && cl <= C::TRIG, a.ck.status, 6)) cl = 0;
+                }
+                for (uint32_t todo = __ballot_sync(0xffffffffu, cl >= kp); todo; todo &= todo - 1u) {
+                    const int j = __ffs(todo) - 1, q = warp + NEP * j;
+                    ListRegs<KC> L;
+                    L.load(lists + q * KC, spill + q * SP, __shfl_sync(0xffffffffu, cl, j), lane);
+                    const uint64_t k = L.bound(kp, min(C::TRIG, a.lstride), lane);   // (kp <= lstride)
+                    __syncwarp();
+                    const int n = L.store_le(lists + q * KC, k, lane);
+                    if (lane == 0) atomicMin(a.tq + iq[q].x, (unsigned long long)k);
+                    if (lane == j) cl = n;
+                }
+                __syncwarp();
+                if (ql < nqi) a.inter_cnt[ol] = cl;
+                for (uint32_t todo = __ballot_sync(0xffffffffu, cl > 0); todo; todo &= todo - 1u) {
+                    const int j = __ffs(todo) - 1;
+                    const int n = __shfl_sync(0xffffffffu, cl, j);
+                    uint64_t* dst = a.inter + __shfl_sync(0xffffffffu, ol, j) * a.lstride;
+                    const uint64_t* src = lists + (warp + NEP * j) * KC;
+                    for (int e = lane; e < n; e += 32) dst[e] = src[e];
+                }
+            }
+            arrive_warp(bars + C::b_empty_item(ib));
         }
     }
     tc_fence_before();
@@ -1013,7 +1033,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 }
 
 bool tc_available(int precision, int D, int kp) {
-    return (precision == ERQ_PREC_FP16 || precision == ERQ_PREC_FP8) && D % KB == 0 && kp <= KCAP;
+    return precision != ERQ_PREC_INT8 && D % KB == 0 && kp <= KCAP;
 }
 
 // Work-item query counts the tensor-core scan is built for, given k'.
@@ -1024,13 +1044,12 @@ bool scan_tc_shape_ok(int qn, int kp) {
 // Capacity (stride) of the per-(query, item) candidate lists written by the scan.
 int scan_list_stride(int precision, int kp, int qn) {
     (void)qn;
-    if (precision == ERQ_PREC_FP32) return kp;
-    return kp <= 32 ? CfgA::KC : CfgB::KC;
+    if (precision == ERQ_PREC_FP32 && kp > KCAP) return kp;      // the CUDA-core scan
+    return kp <= 32 ? 64 : CfgB::TRIG;   // (a list of k' or more entries is cut to this before it is written)
 }
 
-cudaError_t launch_to_half(const float* x, __half* y, int64_t n, cudaStream_t s);
-
-
+// Entries of the lists' continuation that a launch of `grid` CTAs needs.
+int64_t scan_spill_entries(int qn, int grid) { return (int64_t)grid * std::max(qn, 32) * SP; }
 
 // Per work item: {first padded row (lo, hi), rows, queries} and, per query slot,
 // {query row or -1, ||q_r - c||^2 bits, output list index (lo, hi)}.  One warp per item.
@@ -1056,8 +1075,8 @@ __global__ void item_tables_kernel(const int4* __restrict__ items, const int64_t
     if (lane == 0) {
         itemd[it] = make_int4((int)(uint32_t)rb0, (int)(rb0 >> 32), nrows, nqi);
         const unsigned long long nblk = (unsigned long long)((nrows + MR - 1) / MR);
-        atomicAdd(&stats[2], nblk);
-        atomicAdd(&stats[3], nblk * (unsigned long long)(nqi <= 16 ? 16 : (nqi + 15) & ~15));
+        if (stats) atomicAdd(&stats[2], nblk);
+        if (stats) atomicAdd(&stats[3], nblk * (unsigned long long)(nqi <= 16 ? 16 : (nqi + 15) & ~15));
     }
     for (int q = lane; q < QN; q += 32) {
         int4 v = make_int4(-1, 0, 0, 0);
@@ -1218,27 +1237,28 @@ static bool make_query_map(CUtensorMap* map, const void* base, int64_t nq, int64
 }
 
 template <class C, int P>
-static erq_status scan_tc_launch(const ScanLaunch& L, const tc::Args& a, const void* qbase, int64_t qrow_bytes,
-                                 cudaStream_t s) {
+static erq_status scan_tc_launch(const ScanLaunch& L, const tc::Args& a, const void* qbase, const void* qlo,
+                                 int64_t qrow_bytes, cudaStream_t s) {
     const int smem = C::Smem::total;
-    {   // the kernel's raw-code ring must hold an even number (>= 2) of stage slots
-        const int64_t slot = (int64_t)RP * (MR / 32) * 256 * L.B * (P == 1 ? 2 : 1);
-        if ((std::min<int64_t>(RSMAX, C::RAW_BYTES / slot) & ~1ll) < 2)
+    {   // the kernel's raw-code ring must hold a multiple of NSET unit slots
+        const int64_t slot = (int64_t)(MR / 32) * 256 * L.B * (P == 1 ? 2 : 1);
+        if ((std::min<int64_t>(RSMAX, C::RAW_BYTES / slot) & ~(int64_t)(NSET - 1)) < NSET)
             return fail(ERQ_EUNSUPPORTED, "tensor-core scan: raw-code ring too small for this code width");
     }
     cudaError_t e = cudaFuncSetAttribute(scan_tc_kernel<C, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return cuda_fail(e, "scan_tc smem attribute");
     if (L.grid <= 0) return ERQ_OK;
-    CUtensorMap cmap, cmap1, qmap;
+    CUtensorMap cmap, cmap1, qmap, qmap_lo;
     if (!L.codes_p || ((uintptr_t)L.codes_p & 15) != 0 || (L.D % KB) != 0 || L.B < 1 || L.B > 9 ||
         !make_codes_map(&cmap, L.codes_p, L.Np, L.D, L.B, MR / 32) ||
         !make_codes_map(&cmap1, L.codes_p, L.Np, L.D, L.B, 1))
         return fail(ERQ_ECUDA, "tensor-core scan: cuTensorMapEncodeTiled failed for the code array");
     if (!qbase || ((uintptr_t)qbase & 15) != 0 || qrow_bytes % 128 != 0 || L.nq < 1 ||
-        !make_query_map(&qmap, qbase, L.nq, qrow_bytes))
+        !make_query_map(&qmap, qbase, L.nq, qrow_bytes) || ((uintptr_t)qlo & 15) != 0 ||
+        !make_query_map(&qmap_lo, qlo ? qlo : qbase, L.nq, qrow_bytes))
         return fail(ERQ_ECUDA, "tensor-core scan: cuTensorMapEncodeTiled failed for the query array");
     count_launch();
-    scan_tc_kernel<C, P><<<L.grid, THREADS, smem, s>>>(cmap, cmap1, qmap, a);
+    scan_tc_kernel<C, P><<<L.grid, THREADS, smem, s>>>(cmap, cmap1, qmap, qmap_lo, a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "scan_tc launch");
     return ERQ_OK;
@@ -1247,27 +1267,31 @@ static erq_status scan_tc_launch(const ScanLaunch& L, const tc::Args& a, const v
 template <class C>
 static erq_status scan_tc_form(int P, const ScanLaunch& L, const tc::Args& a, const void* qb, int64_t qrow,
                                cudaStream_t s) {
-    if (P == 1) return scan_tc_launch<C, 1>(L, a, qb, qrow, s);
-    if (P == 2) return scan_tc_launch<C, 2>(L, a, qb, qrow, s);
-    return scan_tc_launch<C, 0>(L, a, qb, qrow, s);
+    if (P == 1) return scan_tc_launch<C, 1>(L, a, qb, nullptr, qrow, s);
+    if (P == 2) return scan_tc_launch<C, 2>(L, a, qb, nullptr, qrow, s);
+    return scan_tc_launch<C, 0>(L, a, qb, nullptr, qrow, s);
 }
 
 erq_status scan_tc(const ScanLaunch& L, int precision, cudaStream_t s) {
     if (!tc_available(precision, L.D, L.kp))
-        return fail(ERQ_EUNSUPPORTED, "tensor-core scan: needs precision fp16 or fp8 and k' <= 128");
-    const bool f8 = precision == ERQ_PREC_FP8;
-    const int P = f8 ? (L.B <= 4 ? 1 : 2) : 0;
+        return fail(ERQ_EUNSUPPORTED, "tensor-core scan: needs precision fp32, fp16 or fp8 and k' <= 128");
+    const bool f8 = precision == ERQ_PREC_FP8, f32 = precision == ERQ_PREC_FP32;
+    const int P = f32 ? 3 : (f8 ? (L.B <= 4 ? 1 : 2) : 0);
     if (P == 2 && L.B > 8)
         return fail(ERQ_EUNSUPPORTED, "tensor-core scan: e4m3 holds the split code parts only for B <= 8");
     if (P == 2 && L.Dq != 2 * (int64_t)L.D) return fail(ERQ_EINVAL, "tensor-core scan: split e4m3 needs doubled query rows");
-    if (!(f8 ? (L.Q8 && L.qscale) : L.Qh != nullptr)) return fail(ERQ_EINVAL, "tensor-core scan: queries missing");
-    if (!L.itemd || !L.itemq || !L.rowmeta || !L.tq || !L.work_ctr)
+    if (!(f8 ? (L.Q8 && L.qscale) : L.Qh != nullptr) || (f32 && (!L.Ql || !L.qscale)))
+        return fail(ERQ_EINVAL, "tensor-core scan: queries missing");
+    if (!L.itemd || !L.itemq || !L.rowmeta || !L.tq || !L.work_ctr || !L.spill)
         return fail(ERQ_EINVAL, "tensor-core scan: item tables missing");
-    if (!scan_tc_shape_ok(L.qn, L.kp)) return fail(ERQ_EINVAL, "tensor-core scan: no kernel for this item shape");
+    if (!scan_tc_shape_ok(L.qn, L.kp) || (f32 && L.qn > CfgA32::QN))
+        return fail(ERQ_EINVAL, "tensor-core scan: no kernel for this item shape");
     tc::Args a;
     a.ck = L.ck;
     a.itemd = L.itemd; a.itemq = L.itemq; a.qn = L.qn; a.rowmeta = L.rowmeta; a.n_items = L.n_items;
     a.work_ctr = L.work_ctr;
+    a.lstride = scan_list_stride(precision, L.kp, L.qn);
+    a.spill = L.spill;
     a.inter = L.inter; a.inter_cnt = L.inter_cnt; a.tq = L.tq; a.qscale = L.qscale; a.status = L.status;
     a.D = L.D; a.B = L.B; a.kp = L.kp; a.ip = L.ip;
     a.nkb = P == 1 ? (int)(L.Dq / 128) : L.D / KB;
@@ -1278,8 +1302,10 @@ erq_status scan_tc(const ScanLaunch& L, int precision, cudaStream_t s) {
     a.stall_stage = L.stall_stage;
     const void* qb = f8 ? L.Q8 : L.Qh;
     const int64_t qrow = f8 ? L.Dq : 2 * (int64_t)L.D;
+    if (f32 && L.qn > CfgB32::QN) return scan_tc_launch<CfgA32, 3>(L, a, L.Qh, L.Ql, qrow, s);
+    if (f32) return scan_tc_launch<CfgB32, 3>(L, a, L.Qh, L.Ql, qrow, s);
     if (L.kp <= 32 && L.qn > CfgA::QN) return scan_tc_form<CfgW>(P, L, a, qb, qrow, s);
-    if (L.kp <= 32) return scan_tc_form<CfgA>(P, L, a, qb, qrow, s);
+    if (L.kp <= 32 && L.qn > CfgB::QN) return scan_tc_form<CfgA>(P, L, a, qb, qrow, s);
     return scan_tc_form<CfgB>(P, L, a, qb, qrow, s);
 }
 

@@ -40,17 +40,31 @@ __device__ __forceinline__ uint64_t now_ns() {
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
     return t;
 }
+// One poll that may suspend the warp for up to `hint` ns while the phase is
+// incomplete, so that waiting roles leave the issue slots to working ones.
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, uint32_t hint) {
+    uint32_t ok;
+    asm volatile(
+        "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, 1, 0, p; }"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity), "r"(hint)
+        : "memory");
+    return ok != 0;
+}
 // Bounded wait; returns false (and raises the abort flag) when limit_ns pass
-// or another role has already aborted.
+// or another role has already aborted.  The nanosecond clock is slow to read,
+// so it is read only every 8 failed polls: a wait that ends soon never does.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                           uint64_t limit_ns = kWaitNs) {
     if (mbar_test(bar, parity)) return true;
-    const uint64_t t0 = now_ns();
+    uint64_t t0 = 0;
     for (uint32_t it = 1;; ++it) {
-        if (mbar_test(bar, parity)) return true;
-        if ((it & 63) == 0) {
+        if (mbar_poll(bar, parity, 100000u)) return true;
+        if ((it & 7) == 0) {
             if (*abort_flag) return false;
-            if (now_ns() - t0 > limit_ns) {
+            const uint64_t t = now_ns();
+            if (t0 == 0) t0 = t;
+            if (t - t0 > limit_ns) {
                 *abort_flag = 1;
                 return false;
             }
@@ -121,6 +135,14 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
                  "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), \
                  "r"(r[31])                                                                                      \
                  : "memory")
+
+#define ERQ_TMEM_LD16(taddr, r)                                                                                   \
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, " \
+                 "[%16];"                                                                                         \
+                 : "=r"((r)[0]), "=r"((r)[1]), "=r"((r)[2]), "=r"((r)[3]), "=r"((r)[4]), "=r"((r)[5]), "=r"((r)[6]),          \
+                   "=r"((r)[7]), "=r"((r)[8]), "=r"((r)[9]), "=r"((r)[10]), "=r"((r)[11]), "=r"((r)[12]), "=r"((r)[13]),      \
+                   "=r"((r)[14]), "=r"((r)[15])                                                                     \
+                 : "r"(taddr))
 
 #define ERQ_TMEM_LD32(taddr, r)                                                                                   \
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"  \
