@@ -60,7 +60,7 @@ void free_index_arrays(erq_index* ix) {
                     ix->P,     ix->C,     ix->Cp,      ix->cnorm2, ix->list_off, ix->list_ids,
                     ix->row_of, ix->cl_of_row, ix->codes, ix->f_add, ix->f_res,  ix->g_const,
                     ix->X,     ix->status, ix->ws,      ix->ws_b,   ix->io,    ix->rowmeta, ix->poff, ix->codes_p,
-                    ix->dstats, ix->PT_hi, ix->C_hi, ix->dctr, ix->rowmeta1, ix->ws_ts};   // PT_lo / C_lo live inside those blocks
+                    ix->dstats, ix->PT_hi, ix->P_hi, ix->C_hi, ix->dctr, ix->rowmeta1, ix->ws_ts};   // PT_lo / P_lo / C_lo live inside those blocks
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (ix->pinned) cudaFreeHost(ix->pinned);
@@ -137,13 +137,18 @@ erq_status derive_gemm_arrays(erq_index* ix, cudaStream_t s) {
         const size_t pd = (size_t)D * D, cd = (size_t)ix->nlist * D;
         if (!ix->PT_hi && cudaMalloc(&ix->PT_hi, 2 * pd * sizeof(__half)) != cudaSuccess)
             return fail(ERQ_ENOMEM, "cudaMalloc P^T split");
+        if (!ix->P_hi && cudaMalloc(&ix->P_hi, 2 * pd * sizeof(__half)) != cudaSuccess)
+            return fail(ERQ_ENOMEM, "cudaMalloc P split");
         if (!ix->C_hi && cudaMalloc(&ix->C_hi, 2 * cd * sizeof(__half)) != cudaSuccess)
             return fail(ERQ_ENOMEM, "cudaMalloc centroid split");
         ix->PT_lo = ix->PT_hi + pd;
+        ix->P_lo = ix->P_hi + pd;
         ix->C_lo = ix->C_hi + cd;
-        ix->device_bytes += (int64_t)(4 * (pd + cd));
+        ix->device_bytes += (int64_t)(4 * (2 * pd + cd));
         if ((e = launch_split_hilo(ix->PT, ix->ePT, D, D, ix->PT_hi, ix->PT_lo, s)) != cudaSuccess)
             return cuda_fail(e, "split P^T");
+        if ((e = launch_split_hilo(ix->P, ix->eP, D, D, ix->P_hi, ix->P_lo, s)) != cudaSuccess)
+            return cuda_fail(e, "split P");
         if ((e = launch_split_hilo(ix->C, ix->eC, ix->nlist, D, ix->C_hi, ix->C_lo, s)) != cudaSuccess)
             return cuda_fail(e, "split centroids");
     }
@@ -1058,18 +1063,20 @@ extern "C" erq_status erq_search_backward_metric(erq_index* ix, const float* Q, 
     if (!Q || !grad_Q || (nc > 0 && (!ids || !grad_scores))) return fail(ERQ_EINVAL, "erq_search_backward: null pointer");
     cudaStream_t s = (cudaStream_t)stream;
     const size_t mat = (size_t)nq * ix->D;
-    ERQ_TRY(ensure_ws(&ix->ws, &ix->ws_bytes, 2 * mat * 4 + (size_t)nq * 4 + 1024));
+    ERQ_TRY(ensure_ws(&ix->ws, &ix->ws_bytes, 3 * mat * 4 + (size_t)nq * 4 + 1024));
     float* V = (float*)ix->ws;
     float* Wv = V + (mat + 63) / 64 * 64;
-    int32_t* eV = (int32_t*)(Wv + (mat + 63) / 64 * 64);
+    __half* Vh = (__half*)(Wv + (mat + 63) / 64 * 64);           // V's FP16 parts, hi then lo
+    __half* Vl = Vh + (mat + 63) / 64 * 64;
+    int32_t* eV = (int32_t*)(Vl + (mat + 63) / 64 * 64);
     cudaError_t e;
     if ((e = launch_backward_gather(Q, ids, grad_scores, nq, nc, ix, metric == ERQ_METRIC_IP ? 1 : 0, V, Wv, s)) !=
         cudaSuccess)
         return cuda_fail(e, "backward gather");
-    // grad_Q = V P^T + Wv  (B = P read as [n][k])
-    if ((e = launch_row_exp(V, nq, ix->D, eV, s)) != cudaSuccess) return cuda_fail(e, "backward exponents");
-    if ((e = launch_gemm_tc(V, eV, nq, ix->P, ix->eP, ix->D, ix->D, grad_Q, ix->D, 0, Wv, nullptr, nullptr, ix->status,
-                            s)) != cudaSuccess)
+    // grad_Q = V P^T + Wv  (B = P read as [n][k]), on the TMA-fed GEMM
+    if ((e = launch_query_prep(V, nq, ix->D, eV, nullptr, Vh, Vl, s)) != cudaSuccess) return cuda_fail(e, "backward split");
+    if ((e = launch_gemm_tma(Vh, Vl, eV, nq, ix->P_hi, ix->P_lo, ix->eP, ix->D, ix->D, grad_Q, ix->D, 0, nullptr, nullptr,
+                             nullptr, ix->status, s, nullptr, Wv)) != cudaSuccess)
         return cuda_fail(e, "backward gemm");
     return ERQ_OK;
 }

@@ -124,6 +124,8 @@ struct erq_index {
     int32_t* eC = nullptr;       // [nlist] row exponents of the centroids
     __half* PT_hi = nullptr;     // [D][D] P^T scaled by 2^-ePT, split into FP16 hi / lo parts
     __half* PT_lo = nullptr;
+    __half* P_hi = nullptr;      // [D][D] P the same way (the backward's product)
+    __half* P_lo = nullptr;
     __half* C_hi = nullptr;      // [nlist][D] centroids scaled by 2^-eC, FP16 hi / lo parts
     __half* C_lo = nullptr;
     float* C = nullptr;          // [nlist][D] centroids

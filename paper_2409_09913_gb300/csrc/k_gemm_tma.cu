@@ -57,6 +57,7 @@ struct Args {
     const float* rown;       // EPI_DIST: [M]
     const float* coln;       // EPI_DIST: [N]
     float* gmin;             // EPI_DIST, optional: [M][ceil(N / 32)] minimum of each 32-column group
+    const float* addend;     // EPI_PLAIN, optional: [M][ldc], added to the product
     __half* Ch;              // optional: an FP16 copy of the output (round to nearest), same layout
     uint32_t* status;
 };
@@ -238,6 +239,20 @@ __global__ void __launch_bounds__(gemm2::THREADS, 1)
                 if (mok) {
                     const int nb = n0 + cc;
                     float* crow = a.C + m * a.ldc + nb;
+                    if (a.addend) {
+                        const float* arow = a.addend + m * a.ldc + nb;
+                        if (nb + 32 <= a.N && (a.ldc % 4) == 0) {
+#pragma unroll
+                            for (int j = 0; j < 32; j += 4) {
+                                const float4 ad = *reinterpret_cast<const float4*>(arow + j);
+                                out[j] += ad.x; out[j + 1] += ad.y; out[j + 2] += ad.z; out[j + 3] += ad.w;
+                            }
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 32; ++j)
+                                if (nb + j < a.N) out[j] += arow[j];
+                        }
+                    }
                     if (nb + 32 <= a.N && (a.ldc % 4) == 0) {
 #pragma unroll
                         for (int j = 0; j < 32; j += 4)
@@ -402,7 +417,7 @@ static bool make_half_map(CUtensorMap* map, const __half* base, int64_t rows, in
 cudaError_t launch_gemm_tma(const __half* Ahi, const __half* Alo, const int32_t* eA, int64_t M, const __half* Bhi,
                             const __half* Blo, const int32_t* eB, int N, int K, float* C, int64_t ldc, int epi,
                             const float* rown, const float* coln, float* gmin, uint32_t* status, cudaStream_t s,
-                            __half* Ch) {
+                            __half* Ch, const float* addend) {
     if (M <= 0 || N <= 0) return cudaSuccess;
     if (K % gemm2::BK != 0 || M > 0x7fffffff) return cudaErrorInvalidValue;
     CUtensorMap mAh, mAl, mBh, mBl;
@@ -411,7 +426,7 @@ cudaError_t launch_gemm_tma(const __half* Ahi, const __half* Alo, const int32_t*
         return cudaErrorInvalidValue;
     gemm2::Args a;
     a.eA = eA; a.eB = eB; a.C = C; a.ldc = ldc; a.M = M; a.N = N; a.K = K; a.epi = epi;
-    a.rown = rown; a.coln = coln; a.gmin = gmin; a.Ch = Ch; a.status = status;
+    a.rown = rown; a.coln = coln; a.gmin = gmin; a.addend = addend; a.Ch = Ch; a.status = status;
     cudaError_t e = cudaFuncSetAttribute(gemm_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm2::SMEM);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 148;

@@ -140,6 +140,22 @@ cudaError_t launch_rotate_fp64_if(const uint32_t* flag, const float* X, const in
 // ---------------------------------------------------------------------------
 enum { EPI_PLAIN = 0, EPI_DIST = 1 };
 
+// Two FP32 multiply-adds in one instruction, each rounded as fmaf (the 64 FMAs of
+// a k step are 32 issue slots: 100,000 x 256 x 768, 0.916 -> 0.887 ms).
+__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ uint64_t pack2(float x, float y) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+
 template <bool NT, int EPI>
 __global__ void __launch_bounds__(256) sgemm_kernel(const float* __restrict__ A, const float* __restrict__ Bm,
                                                     float* __restrict__ Cm, int64_t M, int N, int K, float alpha,
@@ -192,11 +208,11 @@ __global__ void __launch_bounds__(256) sgemm_kernel(const float* __restrict__ A,
             *reinterpret_cast<float4*>(&Bs[buf][lb_k][lb_n]) = rb;
         }
     };
-    float acc[8][8];
+    uint64_t acc2[8][4];                     // columns 2 j, 2 j + 1 of the thread's eight
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < 4; ++j) acc2[i][j] = 0ull;
     const int ty = tid / 16, tx = tid % 16;
     load_regs(0);
     store_smem(0);
@@ -207,19 +223,18 @@ __global__ void __launch_bounds__(256) sgemm_kernel(const float* __restrict__ A,
         if (more) load_regs(k0 + 8);
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk) {
-            float a[8], b[8];
             const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4]);
             const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][64 + ty * 4]);
-            const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]);
-            const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][kk][64 + tx * 4]);
-            a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w;
-            a[4] = a1.x; a[5] = a1.y; a[6] = a1.z; a[7] = a1.w;
-            b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w;
-            b[4] = b1.x; b[5] = b1.y; b[6] = b1.z; b[7] = b1.w;
+            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][tx * 4]);
+            const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][64 + tx * 4]);
+            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            const uint64_t b[4] = {b0.x, b0.y, b1.x, b1.y};
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+            for (int i = 0; i < 8; ++i) {
+                const uint64_t aa = pack2(a[i], a[i]);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < 4; ++j) fma2(acc2[i][j], aa, b[j]);
+            }
         }
         if (more) {
             store_smem(buf ^ 1);
@@ -235,11 +250,13 @@ __global__ void __launch_bounds__(256) sgemm_kernel(const float* __restrict__ A,
         for (int j = 0; j < 8; ++j) {
             const int nn = n0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + (j - 4));
             if (nn >= N) continue;
+            const float2 pr = unpack2(acc2[i][j >> 1]);
+            const float ac = (j & 1) ? pr.y : pr.x;
             float v;
             if (EPI == EPI_DIST) {
-                v = rown[m] + coln[nn] - 2.f * acc[i][j];
+                v = rown[m] + coln[nn] - 2.f * ac;
             } else {
-                v = alpha * acc[i][j];
+                v = alpha * ac;
                 if (addend) v += addend[m * ldc + nn];
             }
             Cm[m * ldc + nn] = v;
