@@ -70,6 +70,7 @@ void free_index_arrays(erq_index* ix) {
         delete[] ix->ev_ring;
     }
     delete ix->host_list_off;
+    delete ix->sizes_desc;
 }
 
 // Bump allocator over a device workspace.
@@ -624,7 +625,8 @@ static erq_status ensure_stage1(erq_index* ix, cudaStream_t s) {
 }
 
 static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const erq_search_params* p, int64_t* ids,
-                              float* dists, cudaStream_t s, const TwoStageReq* ts = nullptr) {
+                              float* dists, cudaStream_t s, const TwoStageReq* ts = nullptr,
+                              bool check_later = false) {
     const int D = ix->D, nlist = ix->nlist;
     const int k = p->k;
     const int kp = std::max(p->k, p->rerank_k);
@@ -665,30 +667,24 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
         T((int32_t*)nullptr, nq);                                        // 4 npr
         T((float*)nullptr, (size_t)nq * maxp);                           // 5 dqc
         T((int32_t*)nullptr, (size_t)nq * maxp);                         // 6 probe_c
-        T((int32_t*)nullptr, (size_t)nq * maxp);                         // 7 slot_nr
+        T((int32_t*)nullptr, (size_t)nq * maxp);                         // 7 slot_pos
         T((int32_t*)nullptr, (size_t)nq * maxp);                         // 8 slot_off
         T((int64_t*)nullptr, nq);                                        // 9 qtot
         T((int64_t*)nullptr, nq + 1);                                    // 10 qbase
-        T((int32_t*)nullptr, 2 * (size_t)nlist);                         // 11 cnt_c (per phase cluster)
-        T((int32_t*)nullptr, 2 * (size_t)nlist);                         // 12 pos_c
-        T((int64_t*)nullptr, 2 * (size_t)nlist);                         // 13 cnt64
-        T((int64_t*)nullptr, 2 * (size_t)nlist);                         // 14 items_c
-        T((int64_t*)nullptr, 2 * (size_t)nlist + 1);                     // 15 qoff
-        T((int64_t*)nullptr, 2 * (size_t)nlist + 1);                     // 16 item_off
-        T((int64_t*)nullptr, (size_t)nq * maxp);                         // 17 qlist
-        T((uint64_t*)nullptr, (size_t)nq * kp);                          // 18 cand
-        T((uint64_t*)nullptr, 1);                                        // 19 (unused)
-        T((__half*)nullptr, prec == ERQ_PREC_FP16 ? (size_t)nq * D : 1); // 20 Qh
-        T((int32_t*)nullptr, nq);                                        // 21 eQ
-        T((uint64_t*)nullptr, tcp ? nq : 1);                             // 22 query-wide thresholds
-        T((__half*)nullptr, (size_t)nq * D);                              // 23 Q hi
-        T((__half*)nullptr, (size_t)nq * D);                              // 24 Q lo
-        T((float*)nullptr, (!explicit_probe && nlist > 1) ? (size_t)nq * ((nlist + 31) / 32) : 1);  // 25 group minima
-        T((unsigned char*)nullptr, prec == ERQ_PREC_FP8 ? (size_t)nq * Dq : 1);   // 26 e4m3 queries
-        T((float*)nullptr, prec == ERQ_PREC_FP16 ? 1 : (size_t)nq);               // 27 scales (e4m3, or FP32's two parts)
-        T((int32_t*)nullptr, nlist);                                     // 28 touch_c
+        T((int32_t*)nullptr, nlist);                                     // 11 cnt_c
+        T((int32_t*)nullptr, nlist);                                     // 12 item_first
+        T((int64_t*)nullptr, 1);                                         // 13 work items
+        T((uint64_t*)nullptr, (size_t)nq * kp);                          // 14 cand
+        T((__half*)nullptr, prec == ERQ_PREC_FP16 ? (size_t)nq * D : 1); // 15 Qh
+        T((int32_t*)nullptr, nq);                                        // 16 eQ
+        T((uint64_t*)nullptr, tcp ? nq : 1);                             // 17 query-wide thresholds
+        T((__half*)nullptr, (size_t)nq * D);                              // 18 Q hi
+        T((__half*)nullptr, (size_t)nq * D);                              // 19 Q lo
+        T((float*)nullptr, (!explicit_probe && nlist > 1) ? (size_t)nq * ((nlist + 31) / 32) : 1);  // 20 group minima
+        T((unsigned char*)nullptr, prec == ERQ_PREC_FP8 ? (size_t)nq * Dq : 1);   // 21 e4m3 queries
+        T((float*)nullptr, prec == ERQ_PREC_FP16 ? 1 : (size_t)nq);               // 22 scales (e4m3, or FP32's two parts)
     };
-    void* sl[29];
+    void* sl[23];
     layout(plan, false, sl);
     ERQ_TRY(ensure_ws(&ix->ws, &ix->ws_bytes, plan.off));
     Carver cv(ix->ws, ix->ws_bytes);
@@ -701,23 +697,22 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     float* dqc = (float*)sl[5];
     PlanArgs pa;
     pa.probe_c = (int32_t*)sl[6];
-    pa.slot_nr = (int32_t*)sl[7];
+    pa.slot_pos = (int32_t*)sl[7];
     pa.slot_off = (int32_t*)sl[8];
     pa.qtot = (int64_t*)sl[9];
     pa.qbase = (int64_t*)sl[10];
     pa.cnt_c = (int32_t*)sl[11];
-    pa.pos_c = (int32_t*)sl[12];
-    pa.cnt64 = (int64_t*)sl[13];
-    pa.items_c = (int64_t*)sl[14];
-    pa.qoff = (int64_t*)sl[15];
-    pa.item_off = (int64_t*)sl[16];
-    pa.qlist = (int64_t*)sl[17];
-    pa.touch_c = (int32_t*)sl[28];
-    uint64_t* cand = (uint64_t*)sl[18];
-    if (!ix->dstats && cudaMalloc(&ix->dstats, 4 * sizeof(unsigned long long)) != cudaSuccess)
+    pa.item_first = (int32_t*)sl[12];
+    pa.n_items = (int64_t*)sl[13];
+    pa.tq = tcp ? (unsigned long long*)sl[17] : nullptr;
+    pa.itemd = pa.itemq = pa.items = nullptr;
+    uint64_t* cand = (uint64_t*)sl[14];
+    if (!ix->dstats && cudaMalloc(&ix->dstats, 8 * sizeof(unsigned long long)) != cudaSuccess)
         return fail(ERQ_ENOMEM, "cudaMalloc search counters");
     if (!ix->dctr && cudaMalloc(&ix->dctr, 256) != cudaSuccess) return fail(ERQ_ENOMEM, "cudaMalloc scan counter");
     pa.stats = ix->dstats;
+    pa.work_ctr = ix->dctr;
+    pa.count_blocks = prec != ERQ_PREC_FP32;
     cudaError_t e;
     const bool timed = (p->flags & ERQ_SEARCH_TIMING) != 0;
     ix->timed = 0;
@@ -733,7 +728,7 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     ERQ_TRY(mark(0));
     // ---- q' = P^T q_r
     const bool simt = (p->flags & ERQ_SEARCH_SIMT_GEMM) != 0;
-    int32_t* eQ = (int32_t*)sl[21];
+    int32_t* eQ = (int32_t*)sl[16];
     const bool need_qn = !explicit_probe && nlist > 1 && !ip;   // ||q_r||^2 for the distance probe
     bool qn_done = false, qh_done = false;
     if (simt) {
@@ -742,21 +737,21 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     } else {
         // row exponents, ||q_r||^2 and the hi/lo split in one pass; the rotation
         // GEMM also writes the FP16 copy of q' that the tensor-core scan reads
-        if ((e = launch_query_prep(Q, nq, D, eQ, need_qn ? qn : nullptr, (__half*)sl[23], (__half*)sl[24], s)) !=
+        if ((e = launch_query_prep(Q, nq, D, eQ, need_qn ? qn : nullptr, (__half*)sl[18], (__half*)sl[19], s)) !=
             cudaSuccess)
             return cuda_fail(e, "query split");
         qn_done = need_qn;
-        __half* qh = prec == ERQ_PREC_FP16 ? (__half*)sl[20] : nullptr;
-        if ((e = launch_gemm_tma((__half*)sl[23], (__half*)sl[24], eQ, nq, ix->PT_hi, ix->PT_lo, ix->ePT, D, D, Qrot,
+        __half* qh = prec == ERQ_PREC_FP16 ? (__half*)sl[15] : nullptr;
+        if ((e = launch_gemm_tma((__half*)sl[18], (__half*)sl[19], eQ, nq, ix->PT_hi, ix->PT_lo, ix->ePT, D, D, Qrot,
                                  D, 0, nullptr, nullptr, nullptr, ix->status, s, qh)) != cudaSuccess)
             return cuda_fail(e, "query rotation");
         qh_done = qh != nullptr;
     }
     if (prec == ERQ_PREC_FP8 &&
-        (e = launch_quant_e4m3(Qrot, nq, D, (int)Dq, split8, (unsigned char*)sl[26], (float*)sl[27], s)) != cudaSuccess)
+        (e = launch_quant_e4m3(Qrot, nq, D, (int)Dq, split8, (unsigned char*)sl[21], (float*)sl[22], s)) != cudaSuccess)
         return cuda_fail(e, "query e4m3");
     if (prec == ERQ_PREC_FP16 && !qh_done &&
-        (e = launch_to_half(Qrot, (__half*)sl[20], (int64_t)nq * D, s)) != cudaSuccess)
+        (e = launch_to_half(Qrot, (__half*)sl[15], (int64_t)nq * D, s)) != cudaSuccess)
         return cuda_fail(e, "query half");
     ERQ_TRY(mark(1));
     // ---- probe
@@ -774,17 +769,17 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
             e = ip ? launch_sgemm(true, Q, ix->C, sqd, nq, nlist, D, -1.f, nullptr, s)
                    : launch_sqdist(Q, qn, ix->C, ix->cnorm2, sqd, nq, nlist, D, s);
         else
-            e = launch_gemm_tma((__half*)sl[23], (__half*)sl[24], eQ, nq, ix->C_hi, ix->C_lo, ix->eC, nlist, D, sqd,
+            e = launch_gemm_tma((__half*)sl[18], (__half*)sl[19], eQ, nq, ix->C_hi, ix->C_lo, ix->eC, nlist, D, sqd,
                                 nlist, ip ? 2 : 1, ip ? nullptr : qn, ip ? nullptr : ix->cnorm2,
-                                maxp <= 32 ? (float*)sl[25] : nullptr, ix->status, s);
+                                maxp <= 32 ? (float*)sl[20] : nullptr, ix->status, s);
         if (e != cudaSuccess) return cuda_fail(e, "centroid distances");
-        e = (!simt && maxp <= 32) ? launch_row_topk_groups(sqd, (float*)sl[25], nq, nlist, nlist, maxp, probe, maxp, s)
+        e = (!simt && maxp <= 32) ? launch_row_topk_groups(sqd, (float*)sl[20], nq, nlist, nlist, maxp, probe, maxp, s)
                                   : launch_row_topk_fast(sqd, nq, nlist, nlist, maxp, probe, nullptr, maxp, s);
         if (e != cudaSuccess) return cuda_fail(e, "probe select");
     }
     if (prec == ERQ_PREC_FP32 && tcp && !ts) {
         // q' in two FP16 parts (over the parts of q, which the probe has read)
-        if ((e = launch_query_prep(Qrot, nq, D, eQ, nullptr, (__half*)sl[23], (__half*)sl[24], s, (float*)sl[27])) !=
+        if ((e = launch_query_prep(Qrot, nq, D, eQ, nullptr, (__half*)sl[18], (__half*)sl[19], s, (float*)sl[22])) !=
             cudaSuccess)
             return cuda_fail(e, "rotated query split");
     }
@@ -800,6 +795,7 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     pa.QT = QT;
     pa.RR = RR;
     pa.list_off = ix->list_off;
+    pa.poff = ix->poff;
     pa.corder = ix->corder;
     pa.npr = npr;
     pa.status = ix->status;
@@ -814,100 +810,114 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     pa.dqc = dqc;
     DevChecks ck;
     ck.status = ix->status;
-    ck.qlist = nq * (int64_t)maxp;
     ck.rows = ix->N;
     ck.nlist = nlist;
-    ck.items = 0;                 // set once phase B is sized; the plan kernels below use qlist only
-    ck.lists = 0;
-    pa.ck = ck;
-    if ((e = launch_plan(pa, s)) != cudaSuccess) return cuda_fail(e, "plan");
-    // dqc needs the validated probe ids
-    if (!dqc_from_probe && (e = launch_dqc(Q, ix->C, pa.probe_c, npr, nq, maxp, D, ip, dqc, s)) != cudaSuccess)
+    if (!dqc_from_probe && !explicit_probe &&
+        (e = launch_dqc(Q, ix->C, probe, p->nprobe_per_query, nq, maxp, D, ip, dqc, s)) != cudaSuccess)
         return cuda_fail(e, "dqc");
-    if (ts) return two_stage_tail(ix, Q, nq, p, ids, dists, s, ts->eps0, ts->stats, pa.probe_c, dqc, Qrot, maxp, kp,
-                                  k, do_rerank, cand, ck);
+    if (ts) {
+        pa.slot_off = nullptr;
+        pa.ck = ck;
+        if ((e = launch_plan_count(pa, s)) != cudaSuccess) return cuda_fail(e, "plan");
+        if (explicit_probe && (e = launch_dqc(Q, ix->C, pa.probe_c, npr, nq, maxp, D, ip, dqc, s)) != cudaSuccess)
+            return cuda_fail(e, "dqc");
+        return two_stage_tail(ix, Q, nq, p, ids, dists, s, ts->eps0, ts->stats, pa.probe_c, dqc, Qrot, maxp, kp, k,
+                              do_rerank, cand, ck);
+    }
     int64_t Ltot = 0, nitems = 0;
-    // host-side bounds assume distinct probed lists per query, which the
-    // centroid search guarantees; explicit probe lists are sized exactly
+    const int lstride = scan_list_stride(prec, kp, QT);
+    // Upper bounds from the list sizes (no read-back).  They assume distinct probed
+    // lists per query, which the centroid search guarantees; explicit probe lists
+    // are sized exactly.
+    //   lists <= nq * (row ranges of the maxp lists with most of them)
+    //   items <= maxR * ceil(nq * maxp / QT) + sum_c nr_c (<= N / RR + nlist), and <= lists
     const bool async = (p->flags & ERQ_SEARCH_ASYNC) != 0 && !explicit_probe;
-    if (async) {
-        // upper bounds from the cluster sizes (no read-back):
-        //   items <= maxR * ceil(nq * maxp / QT) + sum_c nr_c,  lists <= nq * (sum of the maxp largest nr_c)
-        const std::vector<int64_t>& off = *ix->host_list_off;
-        std::vector<int64_t> nr(nlist);
-        int64_t maxR = 0, sumR = 0;
-        for (int c = 0; c < nlist; ++c) {
-            nr[c] = (off[c + 1] - off[c] + RR - 1) / RR;
-            maxR = std::max(maxR, nr[c]);
-            sumR += nr[c];
+    bool bounded = async;
+    if (!explicit_probe && (async || nq * (int64_t)maxp <= kSmallPairs)) {
+        if (!ix->sizes_desc) {
+            const std::vector<int64_t>& off = *ix->host_list_off;
+            ix->sizes_desc = new std::vector<int64_t>(nlist);
+            for (int c = 0; c < nlist; ++c) (*ix->sizes_desc)[c] = off[c + 1] - off[c];
+            std::sort(ix->sizes_desc->begin(), ix->sizes_desc->end(), std::greater<int64_t>());
         }
-        std::partial_sort(nr.begin(), nr.begin() + std::min(maxp, nlist), nr.end(), std::greater<int64_t>());
-        int64_t topR = 0;
-        for (int i = 0; i < std::min(maxp, nlist); ++i) topR += nr[i];
-        nitems = maxR * ceil_div(nq * (int64_t)maxp, QT) + 2 * sumR;   // two phases per cluster
-        Ltot = nq * topR;
-    } else {
+        const std::vector<int64_t>& size = *ix->sizes_desc;
+        for (int i = 0; i < std::min(maxp, nlist); ++i) Ltot += (size[i] + RR - 1) / RR;
+        Ltot *= nq;
+        nitems = std::min((size[0] + RR - 1) / RR * ceil_div(nq * (int64_t)maxp, QT) + ix->N / RR + nlist, Ltot);
+        // a synchronous search takes the bounds too where they are small, and reads
+        // its status once at its end instead of its sizes in the middle
+        bounded = async || (Ltot * lstride * 8 + nitems * (int64_t)QT * 16 <= (32 << 20));
+    }
+    const bool small = bounded && tcp && nq * (int64_t)maxp <= kSmallPairs && nlist <= 16384 && Ltot <= 65536;
+    pa.ck = ck;
+    if (!small) {
+        if ((e = launch_plan_count(pa, s)) != cudaSuccess) return cuda_fail(e, "plan");
+        // dqc of explicit probe lists needs the validated ids
+        if (explicit_probe && (e = launch_dqc(Q, ix->C, pa.probe_c, npr, nq, maxp, D, ip, dqc, s)) != cudaSuccess)
+            return cuda_fail(e, "dqc");
+        if ((e = launch_plan_offsets(pa, s)) != cudaSuccess) return cuda_fail(e, "plan offsets");
+    }
+    if (!bounded) {
         int64_t tot[2] = {0, 0};
         ERQ_CHECK_CUDA(cudaMemcpyAsync(&tot[0], pa.qbase + nq, 8, cudaMemcpyDeviceToHost, s));
-        ERQ_CHECK_CUDA(cudaMemcpyAsync(&tot[1], pa.item_off + 2 * nlist, 8, cudaMemcpyDeviceToHost, s));
+        ERQ_CHECK_CUDA(cudaMemcpyAsync(&tot[1], pa.n_items, 8, cudaMemcpyDeviceToHost, s));
         ERQ_TRY(check_status(ix, s));
         Ltot = tot[0];
         nitems = tot[1];
-        ix->last_stats[2] = nitems;
-        ix->last_stats[3] = Ltot;
     }
     // ---- phase B workspace
-    Carver pb(nullptr, 0);
-    pb.take<int4>(nitems);
-    const int lstride = scan_list_stride(prec, kp, QT);
-    pb.take<uint64_t>((size_t)Ltot * lstride);
-    pb.take<int32_t>(Ltot);
-    pb.take<int64_t>(1);
-    pb.take<int4>(tcp ? nitems : 0);
-    pb.take<int4>(tcp ? nitems * QT : 0);
     const int tc_grid = (int)std::min<int64_t>(nitems, sms);
-    pb.take<uint64_t>(tcp ? scan_spill_entries(QT, tc_grid) : 0);
-    if (async && ix->ws_b_bytes < pb.off)
+    auto layout_b = [&](Carver& c, ScanLaunch* L) {
+        int4* itemd = c.take<int4>(nitems);
+        int4* itemq = c.take<int4>(nitems * QT);
+        int4* items = c.take<int4>(tcp ? 0 : nitems);
+        uint64_t* inter = c.take<uint64_t>((size_t)Ltot * lstride);
+        int32_t* inter_cnt = c.take<int32_t>(Ltot);
+        uint64_t* spill = c.take<uint64_t>(tcp ? scan_spill_entries(QT, tc_grid) : 0);
+        if (L) {
+            pa.itemd = itemd;
+            pa.itemq = itemq;
+            pa.items = tcp ? nullptr : items;
+            L->itemd = itemd;
+            L->itemq = itemq;
+            L->items = items;
+            L->inter = inter;
+            L->inter_cnt = inter_cnt;
+            L->spill = spill;
+        }
+    };
+    ScanLaunch L;
+    Carver pb(nullptr, 0);
+    layout_b(pb, nullptr);
+    if (bounded && ix->ws_b_bytes < pb.off)
         ERQ_CHECK_CUDA(cudaStreamSynchronize(s));   // growing the buffer frees the old one
     ERQ_TRY(ensure_ws(&ix->ws_b, &ix->ws_b_bytes, pb.off));
     Carver cb(ix->ws_b, ix->ws_b_bytes);
-    int4* items = cb.take<int4>(nitems);
-    uint64_t* inter = cb.take<uint64_t>((size_t)Ltot * lstride);
-    int32_t* inter_cnt = cb.take<int32_t>(Ltot);
-    int64_t* n_items_d = cb.take<int64_t>(1);
-    int4* itemd = cb.take<int4>(tcp ? nitems : 0);
-    int4* itemq = cb.take<int4>(tcp ? nitems * QT : 0);
-    uint64_t* spill = cb.take<uint64_t>(tcp ? scan_spill_entries(QT, tc_grid) : 0);
-    ERQ_CHECK_CUDA(cudaMemcpyAsync(n_items_d, pa.item_off + 2 * nlist, 8, cudaMemcpyDeviceToDevice, s));
+    layout_b(cb, &L);
+    uint64_t* inter = L.inter;
+    int32_t* inter_cnt = L.inter_cnt;
     ck.items = nitems;
     ck.lists = Ltot;
     pa.ck = ck;
-    if (Ltot > 0) ERQ_CHECK_CUDA(cudaMemsetAsync(inter_cnt, 0, sizeof(int32_t) * Ltot, s));
-
-    if ((e = launch_plan_items(pa, items, s)) != cudaSuccess) return cuda_fail(e, "plan items");
-    if (tcp && (e = launch_item_tables(items, n_items_d, nitems, ix->list_off, ix->poff, pa.qoff, pa.qlist, dqc,
-                                       pa.qbase, pa.slot_off, maxp, RR, QT, nlist, itemd, itemq,
-                                       prec == ERQ_PREC_FP32 ? nullptr : pa.stats, ck, s)) !=
-                   cudaSuccess)
-        return cuda_fail(e, "item tables");
+    if (small) {
+        if ((e = launch_plan_small(pa, inter_cnt, Ltot, s)) != cudaSuccess) return cuda_fail(e, "plan");
+    } else {
+        if (Ltot > 0) ERQ_CHECK_CUDA(cudaMemsetAsync(inter_cnt, 0, sizeof(int32_t) * Ltot, s));
+        if ((e = launch_plan_fill(pa, s)) != cudaSuccess) return cuda_fail(e, "plan items");
+    }
     ERQ_TRY(mark(3));
     // ---- scan
-    ScanLaunch L;
-    L.Qrot = Qrot; L.Qh = prec == ERQ_PREC_FP32 ? sl[23] : sl[20]; L.Ql = sl[24]; L.Q8 = sl[26]; L.qscale = (const float*)sl[27]; L.Dq = Dq; L.status = ix->status; L.N = ix->N; L.codes = ix->codes; L.g_const = ix->g_const; L.f_res = ix->f_res; L.list_off = ix->list_off;
-    L.list_ids = ix->list_ids; L.qlist = pa.qlist; L.qoff = pa.qoff; L.items = items; L.n_items = n_items_d;
-    L.dqc = dqc; L.slot_off = pa.slot_off; L.qbase = pa.qbase; L.inter = inter; L.inter_cnt = inter_cnt;
+    L.Qrot = Qrot; L.Qh = prec == ERQ_PREC_FP32 ? sl[18] : sl[15]; L.Ql = sl[19]; L.Q8 = sl[21]; L.qscale = (const float*)sl[22]; L.Dq = Dq; L.status = ix->status; L.N = ix->N; L.codes = ix->codes; L.g_const = ix->g_const; L.f_res = ix->f_res; L.list_off = ix->list_off;
+    L.list_ids = ix->list_ids; L.n_items = pa.n_items;
     L.maxp = maxp; L.D = D; L.B = ix->B; L.kp = kp; L.RR = RR; L.qn = QT; L.nlist = nlist;
-    L.itemd = itemd; L.itemq = itemq; L.rowmeta = ix->rowmeta; L.codes_p = ix->codes_p; L.Np = ix->Np;
-    L.tq = (unsigned long long*)sl[22];
+    L.rowmeta = ix->rowmeta; L.codes_p = ix->codes_p; L.Np = ix->Np;
+    L.tq = (unsigned long long*)sl[17];
     L.ip = ip;
     L.ck = ck;
     L.nq = nq;
     L.work_ctr = ix->dctr;
     L.wait_ns = ix->wait_ns;
     L.stall_stage = ix->stall_stage;
-    if (tcp) ERQ_CHECK_CUDA(cudaMemsetAsync(L.tq, 0xff, sizeof(uint64_t) * nq, s));
-    ERQ_CHECK_CUDA(cudaMemsetAsync(ix->dctr, 0, sizeof(unsigned int), s));
-    L.spill = spill;
     L.grid = tcp ? tc_grid : (int)std::min<int64_t>(nitems, (int64_t)sms * scan_fp32_blocks_per_sm(kp, ix->B));
     if (!tcp) {
         if ((e = launch_scan_fp32(L, s)) != cudaSuccess) return cuda_fail(e, "scan fp32");
@@ -916,7 +926,7 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     }
     ERQ_TRY(mark(4));
     // ---- merge, re-rank
-    if ((e = launch_merge(inter, inter_cnt, pa.qbase, nq, kp, lstride, tcp ? (const unsigned long long*)sl[22] : nullptr, cand,
+    if ((e = launch_merge(inter, inter_cnt, pa.qbase, nq, kp, lstride, tcp ? (const unsigned long long*)sl[17] : nullptr, cand,
                           ck, s)) != cudaSuccess)
         return cuda_fail(e, "merge");
     ERQ_TRY(mark(5));
@@ -928,6 +938,7 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
         ix->timed = 1;
         ++ix->timing_seq;
     }
+    if (bounded && !async && !check_later) return check_status(ix, s);   // (read together with the sizes otherwise)
     return ERQ_OK;
 }
 
@@ -1024,9 +1035,10 @@ extern "C" erq_status erq_search_host(erq_index* ix, const float* Q_host, int64_
         cudaError_t e = launch_normalize_rows(Qd, nq, ix->D, Qd, s);
         if (e != cudaSuccess) return cuda_fail(e, "normalize query");
     }
-    ERQ_TRY(search_impl(ix, Qd, nq, &q, idd, dd, s));
+    ERQ_TRY(search_impl(ix, Qd, nq, &q, idd, dd, s, nullptr, true));
     ERQ_CHECK_CUDA(cudaMemcpyAsync(ids_host, idd, ib, cudaMemcpyDeviceToHost, s));
     ERQ_CHECK_CUDA(cudaMemcpyAsync(dists_host, dd, db, cudaMemcpyDeviceToHost, s));
+    if ((p->flags & ERQ_SEARCH_ASYNC) == 0) return check_status(ix, s);
     ERQ_CHECK_CUDA(cudaStreamSynchronize(s));
     return ERQ_OK;
 }
@@ -1329,13 +1341,12 @@ extern "C" uint64_t erq_kernel_launches(void) { return g_launches.load(); }
 
 extern "C" erq_status erq_search_stats(const erq_index* ix, int64_t* out, int32_t n) {
     if (!ix || !out || n < 4) return fail(ERQ_EINVAL, "erq_search_stats: bad arguments");
-    unsigned long long d[4] = {0, 0, 0, 0};
+    unsigned long long d[8] = {};
     if (ix->dstats) {
         ERQ_CHECK_CUDA(cudaDeviceSynchronize());
         ERQ_CHECK_CUDA(cudaMemcpy(d, ix->dstats, sizeof(d), cudaMemcpyDeviceToHost));
     }
-    const int64_t v[6] = {(int64_t)d[0], (int64_t)d[1], ix->last_stats[2], ix->last_stats[3], (int64_t)d[2],
-                          (int64_t)d[3]};
+    const int64_t v[6] = {(int64_t)d[0], (int64_t)d[1], (int64_t)d[5], (int64_t)d[4], (int64_t)d[2], (int64_t)d[3]};
     for (int i = 0; i < n && i < 6; ++i) out[i] = v[i];
     return ERQ_OK;
 }

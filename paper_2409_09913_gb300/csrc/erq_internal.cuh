@@ -55,7 +55,6 @@ struct DevChecks {
     uint32_t* status = nullptr;
     int64_t lists = 0;       // candidate lists allocated (per-(query, item) lists)
     int64_t items = 0;       // work items allocated
-    int64_t qlist = 0;       // entries of the per-cluster query lists
     int64_t rows = 0;        // stored rows N
     int nlist = 0;
 };
@@ -166,7 +165,6 @@ struct erq_index {
     int64_t timing_seq = 0;      // timed searches so far
     int64_t timing_base = 0;     // first timed search not yet summed by erq_search_timing_total
     int timed = 0;               // 1 when the last search was timed
-    int64_t last_stats[4] = {};  // pairs, distinct rows, work items, lists of the last search
     // scan work-item shape (queries per item qn, rows per item rr): forced by
     // erq_set_scan_config, else the autotuned entry of the k' class when its
     // queries x nprobe is within 4x of the search's, else a heuristic
@@ -176,8 +174,9 @@ struct erq_index {
     unsigned int* dctr = nullptr;          // dynamic work-item counter of the tensor-core scan
     unsigned long long wait_ns = 0;        // limit of the scan's bounded waits (0 = the default 2 s)
     long long stall_stage = -1;            // test stall of the scan's bounded-wait path (-1 = none)
-    unsigned long long* dstats = nullptr;  // [4] device counters of the last search: pairs, distinct rows,
-                                           //     tensor-core row blocks, row blocks x padded queries
+    unsigned long long* dstats = nullptr;  // [8] device counters of the last search: pairs, distinct rows, tensor-core
+                                           //     row blocks, row blocks x padded queries, candidate lists, work items
+    std::vector<int64_t>* sizes_desc = nullptr;   // list sizes in decreasing order (bounds of a search's lists and items)
     size_t pinned_bytes = 0;
     int64_t device_bytes = 0;
 };

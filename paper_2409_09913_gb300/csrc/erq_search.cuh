@@ -16,30 +16,32 @@ struct PlanArgs {
     int npr_uniform;
     int64_t nq;
     int maxp, nlist, QT, RR;
-    int two_phase = 0;          // nearest probed cluster of every query in a first phase of work items
     const int64_t* list_off;
+    const int64_t* poff;        // [nlist+1] padded list offsets
     const int32_t* corder;      // [nlist] clusters by decreasing size
     int32_t* npr;               // [nq] effective nprobe
     int32_t* probe_c;           // [nq][maxp] validated cluster or -1
-    int32_t* cnt_c;             // [2 nlist] queries per phase cluster (v = c: nearest probe, nlist + c: others)
-    int32_t* pos_c;             // [2 nlist]
-    int32_t* touch_c;           // [nlist] probes per cluster (distinct probed rows)
-    int32_t* slot_nr;           // [nq][maxp] ranges of the slot's cluster
-    int32_t* slot_off;          // [nq][maxp]
-    int64_t* qtot;              // [nq]
-    int64_t* qbase;             // [nq+1]
-    int64_t* cnt64;             // [2 nlist]
-    int64_t* items_c;           // [2 nlist]
-    int64_t* qoff;              // [2 nlist + 1]
-    int64_t* item_off;          // [2 nlist + 1]
-    int64_t* qlist;             // [nq*maxp]
+    int32_t* cnt_c;             // [nlist] queries per cluster
+    int32_t* slot_pos;          // [nq][maxp] the pair's place among its cluster's queries
+    int32_t* slot_off;          // [nq][maxp] row ranges of the slot's cluster, then its first list within the query
+    int64_t* qtot;              // [nq] candidate lists of the query
+    int64_t* qbase;             // [nq+1] its first list
+    int32_t* item_first;        // [nlist] first work item of the cluster
+    int64_t* n_items;           // device scalar
+    unsigned int* work_ctr;     // the scan's item counter (zeroed)
+    unsigned long long* tq;     // optional [nq] the scan's thresholds (set to all ones)
+    int4* itemd;                // [items] {first padded row lo, hi, rows, queries}
+    int4* itemq;                // [items][QT] {query row, ||q_r - c||^2 bits, output list lo, hi}
+    int4* items;                // optional [items] {cluster, queries, row range, 0} (CUDA-core scan)
     uint32_t* status;
     const float* sqd;           // optional [nq][nlist] probe values (||q_r - c||^2, or -<q_r, c>): when given,
     float* dqc;                 //   the plan copies the probed pairs' values into dqc [nq][maxp]
+    int count_blocks;           // accumulate stats[2], stats[3]
     DevChecks ck;
-    unsigned long long* stats;  // [4]: (query, candidate) pairs, rows of distinct probed clusters,
-                                //      tensor-core row blocks, row blocks x padded queries (item tables)
+    unsigned long long* stats;  // [8]: (query, candidate) pairs, rows of distinct probed clusters, tensor-core row
+                                //      blocks, row blocks x padded queries, candidate lists, work items
 };
+constexpr int64_t kSmallPairs = 2048;   // pairs that plan_small_kernel takes
 
 struct ScanLaunch {
     const float* Qrot;
@@ -55,13 +57,8 @@ struct ScanLaunch {
     const float* f_res;
     const int64_t* list_off;
     const int64_t* list_ids;
-    const int64_t* qlist;
-    const int64_t* qoff;
     const int4* items;
     const int64_t* n_items;
-    const float* dqc;
-    const int32_t* slot_off;
-    const int64_t* qbase;
     uint64_t* inter;
     int32_t* inter_cnt;
     uint64_t* spill;            // tensor-core path: continuation of the CTAs' candidate lists
@@ -117,8 +114,10 @@ cudaError_t launch_excl_scan_i64(const int64_t* in, int64_t* out, int64_t n, cud
 
 cudaError_t launch_dqc(const float* Q, const float* C, const int32_t* probe, const int32_t* npr, int64_t nq, int maxp,
                        int D, int ip, float* dqc, cudaStream_t s);
-cudaError_t launch_plan(const PlanArgs& p, cudaStream_t s);
-cudaError_t launch_plan_items(const PlanArgs& p, int4* items, cudaStream_t s);
+cudaError_t launch_plan_count(const PlanArgs& p, cudaStream_t s);
+cudaError_t launch_plan_offsets(const PlanArgs& p, cudaStream_t s);
+cudaError_t launch_plan_fill(const PlanArgs& p, cudaStream_t s);
+cudaError_t launch_plan_small(const PlanArgs& p, int32_t* inter_cnt, int64_t nlists, cudaStream_t s);
 cudaError_t launch_scan_fp32(const ScanLaunch& L, cudaStream_t s);
 size_t scan_fp32_smem(int kp);
 int scan_fp32_blocks_per_sm(int kp, int B);   // resident FP32-scan blocks per SM at this k' and code width
@@ -132,11 +131,6 @@ cudaError_t launch_merge(const uint64_t* inter, const int32_t* inter_cnt, const 
                          cudaStream_t s);
 int scan_list_stride(int precision, int kp, int qn);
 int64_t scan_spill_entries(int qn, int grid);
-cudaError_t launch_item_tables(const int4* items, const int64_t* n_items, int64_t items_bound, const int64_t* list_off,
-                               const int64_t* poff, const int64_t* qoff, const int64_t* qlist, const float* dqc,
-                               const int64_t* qbase, const int32_t* slot_off, int maxp, int RR, int qn, int nlist,
-                               int4* itemd,
-                               int4* itemq, unsigned long long* stats, const DevChecks& ck, cudaStream_t s);
 bool scan_tc_shape_ok(int qn, int kp);
 cudaError_t launch_scan_layout(const uint8_t* codes, const float* g, const float* f_res, const int64_t* ids,
                                const int64_t* list_off, const int64_t* poff, int nlist, int64_t Np, int D, int B,

@@ -15,9 +15,13 @@
 // The epilogue writes C, the distances, or -C (inner-product probe); for the
 // last two it can also write the minimum of every 32-column group of a row
 // (used by the probe selection).
-// Tile 128 x 256, K block 64 (one 128-byte swizzle row of FP16); a stage is
-// four TMA tiles (A_hi, A_lo 16 KB each; B_hi, B_lo 32 KB each), two stages;
-// two TMEM accumulators of 256 columns, persistent CTAs over output tiles.
+// Tile 128 x BN, K block 64 (one 128-byte swizzle row of FP16); a stage is
+// four TMA tiles (A_hi, A_lo 16 KB each; B_hi, B_lo BN * 128 bytes each); two
+// TMEM accumulators of BN columns, persistent CTAs over output tiles.  BN = 256
+// with two stages is the throughput form (tensor bound); BN = 64 with four
+// stages serves products of fewer 256-column tiles than half the SMs, whose
+// time is one CTA's chain of K blocks (12 MMAs of 48 instead of 128 cycles each):
+// 1 x 960 x 960, 27 -> 14 us.  Both add the same products in the same order.
 // Warp roles: 4 epilogue warps (TMEM lane = output row), 1 TMA warp, 1 MMA
 // warp.  Every wait is bounded (status word on expiry).
 #include <cuda.h>
@@ -32,18 +36,22 @@
 namespace erq {
 
 namespace gemm2 {
-constexpr int BM = 128, BN = 256, BK = 64, STAGES = 2, THREADS = 192;
+constexpr int BM = 128, BK = 64, THREADS = 192;
 constexpr int TILE_A = BM * BK * 2;                   // 16 KB
-constexpr int TILE_B = BN * BK * 2;                   // 32 KB
-constexpr int STAGE = 2 * TILE_A + 2 * TILE_B;        // A_hi, A_lo, B_hi, B_lo
-constexpr int OFF_BARS = STAGES * STAGE;
-constexpr int NBARS = 2 * STAGES + 4 + 1;
-constexpr int OFF_CF = (OFF_BARS + NBARS * 8 + 15) / 16 * 16;   // 4 epilogue warps x 32 column factors (float2)
-constexpr int OFF_EB = OFF_CF + 4 * 32 * 8;                      // 4 epilogue warps x 32 column exponents
-constexpr int OFF_TMEM = OFF_EB + 4 * 32 * 4;
-constexpr int OFF_ABORT = OFF_TMEM + 4;
-constexpr int SMEM = OFF_ABORT + 4 + 1024;
-static_assert(SMEM <= 227 * 1024, "gemm shared memory");
+template <int BN_>
+struct Shape {
+    static constexpr int BN = BN_, STAGES = BN_ == 256 ? 2 : 4, COLS = 2 * BN_;
+    static constexpr int TILE_B = BN * BK * 2;
+    static constexpr int STAGE = 2 * TILE_A + 2 * TILE_B;        // A_hi, A_lo, B_hi, B_lo
+    static constexpr int OFF_BARS = STAGES * STAGE;
+    static constexpr int NBARS = 2 * STAGES + 4 + 1;
+    static constexpr int OFF_CF = (OFF_BARS + NBARS * 8 + 15) / 16 * 16;   // 4 epilogue warps x 32 column factors (float2)
+    static constexpr int OFF_EB = OFF_CF + 4 * 32 * 8;                      // 4 epilogue warps x 32 column exponents
+    static constexpr int OFF_TMEM = OFF_EB + 4 * 32 * 4;
+    static constexpr int OFF_ABORT = OFF_TMEM + 4;
+    static constexpr int SMEM = OFF_ABORT + 4 + 1024;
+    static_assert(SMEM <= 227 * 1024, "gemm shared memory");
+};
 
 enum { EPI_PLAIN = 0, EPI_DIST = 1, EPI_NEGIP = 2 };   // C, ||a||^2 + ||b||^2 - 2C, -C
 
@@ -65,10 +73,14 @@ struct Args {
 
 using namespace tc;
 
+template <class S>
 __global__ void __launch_bounds__(gemm2::THREADS, 1)
     gemm_tma_kernel(const __grid_constant__ CUtensorMap mAh, const __grid_constant__ CUtensorMap mAl,
                     const __grid_constant__ CUtensorMap mBh, const __grid_constant__ CUtensorMap mBl, gemm2::Args a) {
     using namespace gemm2;
+    constexpr int BN = S::BN, STAGES = S::STAGES, TILE_B = S::TILE_B, STAGE = S::STAGE;
+    constexpr int OFF_BARS = S::OFF_BARS, OFF_CF = S::OFF_CF, OFF_EB = S::OFF_EB, OFF_TMEM = S::OFF_TMEM,
+                  OFF_ABORT = S::OFF_ABORT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t* bars = reinterpret_cast<uint64_t*>(sm + OFF_BARS);
@@ -97,7 +109,8 @@ __global__ void __launch_bounds__(gemm2::THREADS, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 5) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "n"(S::COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     tc_fence_before();
@@ -292,7 +305,7 @@ __global__ void __launch_bounds__(gemm2::THREADS, 1)
     if (*abort_flag && tid == 0) atomicOr(a.status, kStatusTimeout);
     if (warp == 5) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(S::COLS));
     }
 }
 
@@ -420,22 +433,27 @@ cudaError_t launch_gemm_tma(const __half* Ahi, const __half* Alo, const int32_t*
                             __half* Ch, const float* addend) {
     if (M <= 0 || N <= 0) return cudaSuccess;
     if (K % gemm2::BK != 0 || M > 0x7fffffff) return cudaErrorInvalidValue;
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // narrow tiles where the wide ones would leave more than half of the SMs idle
+    const bool narrow = 2 * ceil_div(M, gemm2::BM) * ceil_div(N, 256) < sms;
+    const int bn = narrow ? 64 : 256;
     CUtensorMap mAh, mAl, mBh, mBl;
     if (!make_half_map(&mAh, Ahi, M, K, gemm2::BM) || !make_half_map(&mAl, Alo, M, K, gemm2::BM) ||
-        !make_half_map(&mBh, Bhi, N, K, gemm2::BN) || !make_half_map(&mBl, Blo, N, K, gemm2::BN))
+        !make_half_map(&mBh, Bhi, N, K, bn) || !make_half_map(&mBl, Blo, N, K, bn))
         return cudaErrorInvalidValue;
     gemm2::Args a;
     a.eA = eA; a.eB = eB; a.C = C; a.ldc = ldc; a.M = M; a.N = N; a.K = K; a.epi = epi;
     a.rown = rown; a.coln = coln; a.gmin = gmin; a.addend = addend; a.Ch = Ch; a.status = status;
-    cudaError_t e = cudaFuncSetAttribute(gemm_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm2::SMEM);
+    const auto kern = narrow ? gemm_tma_kernel<gemm2::Shape<64>> : gemm_tma_kernel<gemm2::Shape<256>>;
+    const int smem = narrow ? gemm2::Shape<64>::SMEM : gemm2::Shape<256>::SMEM;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t tiles = ceil_div(M, gemm2::BM) * ceil_div(N, gemm2::BN);
+    const int64_t tiles = ceil_div(M, gemm2::BM) * ceil_div(N, bn);
     const int grid = (int)(tiles < sms ? tiles : sms);
     count_launch();
-    gemm_tma_kernel<<<grid, gemm2::THREADS, gemm2::SMEM, s>>>(mAh, mAl, mBh, mBl, a);
+    kern<<<grid, gemm2::THREADS, smem, s>>>(mAh, mAl, mBh, mBl, a);
     return cudaGetLastError();
 }
 

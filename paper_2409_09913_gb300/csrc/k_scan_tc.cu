@@ -592,7 +592,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
                 for (int k = 0; k < QPL; ++k) {
                     const int q = lane + 32 * k;
-                    const int4 v = pv[k];
+                    const int4 v = q < d.w ? pv[k] : make_int4(-1, 0, 0, 0);   // (slots past the item's queries are not written)
                     s_iq[ib * QN + q] = v;
                     s_tq[ib * QN + q] = v.x >= 0 ? __ldcg(a.tq + v.x) : kEmptyKey;
                     if (SC) s_qsc[ib * QN + q] = v.x >= 0 ? a.qscale[v.x] : 0.f;
@@ -1050,58 +1050,6 @@ int scan_list_stride(int precision, int kp, int qn) {
 
 // Entries of the lists' continuation that a launch of `grid` CTAs needs.
 int64_t scan_spill_entries(int qn, int grid) { return (int64_t)grid * std::max(qn, 32) * SP; }
-
-// Per work item: {first padded row (lo, hi), rows, queries} and, per query slot,
-// {query row or -1, ||q_r - c||^2 bits, output list index (lo, hi)}.  One warp per item.
-__global__ void item_tables_kernel(const int4* __restrict__ items, const int64_t* __restrict__ n_items,
-                                   const int64_t* __restrict__ list_off, const int64_t* __restrict__ poff,
-                                   const int64_t* __restrict__ qoff, const int64_t* __restrict__ qlist,
-                                   const float* __restrict__ dqc, const int64_t* __restrict__ qbase,
-                                   const int32_t* __restrict__ slot_off, int maxp, int RR, int QN, int nlist,
-                                   int4* __restrict__ itemd, int4* __restrict__ itemq,
-                                   unsigned long long* __restrict__ stats, DevChecks ck) {
-    const int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (it >= *n_items) return;
-    if (!ERQ_DCHECK(it < ck.items, ck.status, 8)) return;
-    const int4 w = items[it];
-    const int v = w.x, c = v % nlist;                   // phase cluster -> cluster
-    const int64_t qb = qoff[v] + (int64_t)w.y * QN;
-    const int nqi = (int)imin64(QN, qoff[v + 1] - qb);
-    const int64_t size = list_off[c + 1] - list_off[c];
-    const int64_t r0 = (int64_t)w.z * RR;
-    const int64_t rb0 = poff[c] + r0;
-    const int nrows = (int)(imin64(size, r0 + RR) - r0);
-    if (lane == 0) {
-        itemd[it] = make_int4((int)(uint32_t)rb0, (int)(rb0 >> 32), nrows, nqi);
-        const unsigned long long nblk = (unsigned long long)((nrows + MR - 1) / MR);
-        if (stats) atomicAdd(&stats[2], nblk);
-        if (stats) atomicAdd(&stats[3], nblk * (unsigned long long)(nqi <= 16 ? 16 : (nqi + 15) & ~15));
-    }
-    for (int q = lane; q < QN; q += 32) {
-        int4 v = make_int4(-1, 0, 0, 0);
-        if (q < nqi && ERQ_DCHECK(qb + q >= 0 && qb + q < ck.qlist, ck.status, 8)) {
-            const int64_t e = qlist[qb + q];
-            const int64_t qr = e / maxp;
-            const int64_t L = qbase[qr] + slot_off[e] + w.z;
-            v = make_int4((int)qr, __float_as_int(dqc[e]), (int)(uint32_t)L, (int)(L >> 32));
-        }
-        itemq[it * QN + q] = v;
-    }
-}
-
-cudaError_t launch_item_tables(const int4* items, const int64_t* n_items, int64_t items_bound, const int64_t* list_off,
-                               const int64_t* poff, const int64_t* qoff, const int64_t* qlist, const float* dqc,
-                               const int64_t* qbase, const int32_t* slot_off, int maxp, int RR, int qn, int nlist,
-                               int4* itemd, int4* itemq, unsigned long long* stats, const DevChecks& ck,
-                               cudaStream_t s) {
-    if (items_bound <= 0) return cudaSuccess;
-    count_launch();
-    item_tables_kernel<<<(unsigned)ceil_div(items_bound, 8), 256, 0, s>>>(
-        items, n_items, list_off, poff, qoff, qlist, dqc, qbase, slot_off, maxp, RR, qn, nlist, itemd, itemq, stats,
-        ck);
-    return cudaGetLastError();
-}
 
 // Packed scan layout of the index.  One thread per (tile t, K block kb, row r
 // of the tile): padded row p = 32 t + r takes its cluster's stored row (or
