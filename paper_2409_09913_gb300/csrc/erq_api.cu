@@ -502,6 +502,17 @@ static void choose_scan_shape(const erq_index* ix, int prec, int kp, int64_t nq,
     *rr = r;
 }
 
+// List sizes in decreasing order.
+static const std::vector<int64_t>& sizes_desc(erq_index* ix) {
+    if (!ix->sizes_desc) {
+        const std::vector<int64_t>& off = *ix->host_list_off;
+        ix->sizes_desc = new std::vector<int64_t>(ix->nlist);
+        for (int c = 0; c < ix->nlist; ++c) (*ix->sizes_desc)[c] = off[c + 1] - off[c];
+        std::sort(ix->sizes_desc->begin(), ix->sizes_desc->end(), std::greater<int64_t>());
+    }
+    return *ix->sizes_desc;
+}
+
 // Stage 1, pruning, stage 2 and the selection of the two-stage search
 // (k_two_stage.cu), after the probe, then the exact re-rank.
 static erq_status two_stage_tail(erq_index* ix, const float* Q, int64_t nq, const erq_search_params* p, int64_t* ids,
@@ -516,13 +527,9 @@ static erq_status two_stage_tail(erq_index* ix, const float* Q, int64_t nq, cons
     // than 2 GB of scratch, when the exact count is read back instead
     int64_t rows = 0;
     {
-        const std::vector<int64_t>& off = *ix->host_list_off;
-        std::vector<int64_t> sz((size_t)ix->nlist);
-        for (int c = 0; c < ix->nlist; ++c) sz[c] = off[c + 1] - off[c];
-        const int top = std::min(maxp, ix->nlist);
-        std::partial_sort(sz.begin(), sz.begin() + top, sz.end(), std::greater<int64_t>());
+        const std::vector<int64_t>& size = sizes_desc(ix);
         int64_t per_q = 0;
-        for (int i = 0; i < top; ++i) per_q += sz[i];
+        for (int i = 0; i < std::min(maxp, ix->nlist); ++i) per_q += size[i];
         rows = nq * per_q;
     }
     const bool exact = p->probe != nullptr || rows * 20 > (1ll << 31);
@@ -567,6 +574,7 @@ static erq_status two_stage_tail(erq_index* ix, const float* Q, int64_t nq, cons
     L.skey = (uint64_t*)(b + off_skey); L.scratch = (uint32_t*)(b + off_skey);
     L.tau = (float*)(b + off_tau); L.scnt = (int32_t*)(b + off_cnt); L.cand = cand;
     L.nq = nq; L.maxp = maxp; L.D = D; L.B = ix->B; L.kp = kp; L.eps0 = eps0;
+    L.max_list = sizes_desc(ix)[0];
     if ((e = launch_two_stage(L, s)) != cudaSuccess) return cuda_fail(e, "two-stage");
     if ((e = launch_rerank(cand, nq, kp, ix->X, Q, D, k, do_rerank ? 1 : 0, 0, ids, dists, p->cand_ids, p->cand_est,
                            ck, s)) != cudaSuccess)
@@ -754,6 +762,14 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
         (e = launch_to_half(Qrot, (__half*)sl[15], (int64_t)nq * D, s)) != cudaSuccess)
         return cuda_fail(e, "query half");
     ERQ_TRY(mark(1));
+    // ||q_r - c||^2 (or -<q_r, c>) of the probed pairs: the probe's own values
+    // when it computed them (the FP32 expansion ||q_r||^2 + ||c||^2 - 2<q_r, c>
+    // with an FP32-accurate product), else computed directly below
+    // FP32 precision computes them directly: the probe's product drops its low
+    // bits at every tensor-core step, and that bias (1e-5 of an estimate at D =
+    // 960) is most of an FP32 estimate's error
+    const bool dqc_from_probe = !explicit_probe && nlist > 1 && (ts || prec != ERQ_PREC_FP32);
+    float* probe_val = dqc_from_probe ? dqc : nullptr;
     // ---- probe
     const int32_t* probe_use = probe;
     int64_t probe_stride = maxp;
@@ -773,8 +789,8 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
                                 nlist, ip ? 2 : 1, ip ? nullptr : qn, ip ? nullptr : ix->cnorm2,
                                 maxp <= 32 ? (float*)sl[20] : nullptr, ix->status, s);
         if (e != cudaSuccess) return cuda_fail(e, "centroid distances");
-        e = (!simt && maxp <= 32) ? launch_row_topk_groups(sqd, (float*)sl[20], nq, nlist, nlist, maxp, probe, maxp, s)
-                                  : launch_row_topk_fast(sqd, nq, nlist, nlist, maxp, probe, nullptr, maxp, s);
+        e = (!simt && maxp <= 32) ? launch_row_topk_groups(sqd, (float*)sl[20], nq, nlist, nlist, maxp, probe, probe_val, maxp, s)
+                                  : launch_row_topk_fast(sqd, nq, nlist, nlist, maxp, probe, probe_val, maxp, s);
         if (e != cudaSuccess) return cuda_fail(e, "probe select");
     }
     if (prec == ERQ_PREC_FP32 && tcp && !ts) {
@@ -799,14 +815,6 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     pa.corder = ix->corder;
     pa.npr = npr;
     pa.status = ix->status;
-    // ||q_r - c||^2 (or -<q_r, c>) of the probed pairs: the probe's own values
-    // when it computed them (the FP32 expansion ||q_r||^2 + ||c||^2 - 2<q_r, c>
-    // with an FP32-accurate product), else computed directly below
-    // FP32 precision computes them directly: the probe's product drops its low
-    // bits at every tensor-core step, and that bias (1e-5 of an estimate at D =
-    // 960) is most of an FP32 estimate's error
-    const bool dqc_from_probe = !explicit_probe && nlist > 1 && (ts || prec != ERQ_PREC_FP32);
-    pa.sqd = dqc_from_probe ? sqd : nullptr;
     pa.dqc = dqc;
     DevChecks ck;
     ck.status = ix->status;
@@ -834,13 +842,7 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     const bool async = (p->flags & ERQ_SEARCH_ASYNC) != 0 && !explicit_probe;
     bool bounded = async;
     if (!explicit_probe && (async || nq * (int64_t)maxp <= kSmallPairs)) {
-        if (!ix->sizes_desc) {
-            const std::vector<int64_t>& off = *ix->host_list_off;
-            ix->sizes_desc = new std::vector<int64_t>(nlist);
-            for (int c = 0; c < nlist; ++c) (*ix->sizes_desc)[c] = off[c + 1] - off[c];
-            std::sort(ix->sizes_desc->begin(), ix->sizes_desc->end(), std::greater<int64_t>());
-        }
-        const std::vector<int64_t>& size = *ix->sizes_desc;
+        const std::vector<int64_t>& size = sizes_desc(ix);
         for (int i = 0; i < std::min(maxp, nlist); ++i) Ltot += (size[i] + RR - 1) / RR;
         Ltot *= nq;
         nitems = std::min((size[0] + RR - 1) / RR * ceil_div(nq * (int64_t)maxp, QT) + ix->N / RR + nlist, Ltot);

@@ -79,7 +79,7 @@ cudaError_t launch_gemm_tma(const __half* Ahi, const __half* Alo, const int32_t*
                             const float* rown, const float* coln, float* gmin, uint32_t* status, cudaStream_t s,
                             __half* Ch = nullptr, const float* addend = nullptr);
 cudaError_t launch_row_topk_groups(const float* V, const float* gmin, int64_t rows, int ncols, int64_t ld, int p,
-                                   int32_t* out_idx, int64_t ld_out, cudaStream_t s);
+                                   int32_t* out_idx, float* out_val, int64_t ld_out, cudaStream_t s);
 cudaError_t launch_gemm_tc(const float* A, const int32_t* eA, int64_t M, const float* B, const int32_t* eB, int N,
                            int K, float* C, int64_t ldc, int epi, const float* addend, const float* rown,
                            const float* coln, uint32_t* status, cudaStream_t s);

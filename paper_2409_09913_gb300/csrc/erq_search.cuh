@@ -34,8 +34,7 @@ struct PlanArgs {
     int4* itemq;                // [items][QT] {query row, ||q_r - c||^2 bits, output list lo, hi}
     int4* items;                // optional [items] {cluster, queries, row range, 0} (CUDA-core scan)
     uint32_t* status;
-    const float* sqd;           // optional [nq][nlist] probe values (||q_r - c||^2, or -<q_r, c>): when given,
-    float* dqc;                 //   the plan copies the probed pairs' values into dqc [nq][maxp]
+    const float* dqc;           // [nq][maxp] ||q_r - c||^2, or -<q_r, c>, of the pairs
     int count_blocks;           // accumulate stats[2], stats[3]
     DevChecks ck;
     unsigned long long* stats;  // [8]: (query, candidate) pairs, rows of distinct probed clusters, tensor-core row
@@ -102,6 +101,7 @@ struct TwoStageLaunch {
     uint64_t* cand;             // [nq][kp] out: the k' best survivors' keys, ascending
     int64_t nq;
     int maxp, D, B, kp;
+    int64_t max_list;           // rows of the largest list
     float eps0;
 };
 cudaError_t launch_stage1_factors(const float* R, int64_t r0, int64_t m, int D, int B, const uint8_t* codes,

@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(512) dqc_kernel(const float* __restrict__ Q, c
 // per cluster in order of decreasing size (item_first), the pair writes its own
 // query slots of its cluster's items (plan_fill), so no query list is sorted or
 // scattered in between.  16,384 queries x 256 slots over 4,096 lists: 0.40 ms in
-// eight launches before, 0.19 ms in four now.  Up to kSmallPairs pairs run all of it in
+// eight launches before, 0.17 ms in four now.  Up to kSmallPairs pairs run all of it in
 // one block (plan_small_kernel), which is bound by the latency of its five
 // phases instead of by launches.
 // ---------------------------------------------------------------------------
@@ -131,7 +131,7 @@ __device__ __forceinline__ PlanPair plan_pair(const PlanArgs& p, int64_t t) {
     return r;
 }
 
-// One pair: validation, its probe value, its place in its cluster.
+// One pair: validation and its place in its cluster.
 __device__ __forceinline__ void plan_count_one(const PlanArgs& p, int64_t t, unsigned long long& pairs,
                                                unsigned long long& rows) {
     PlanPair r = plan_pair(p, t);
@@ -142,7 +142,6 @@ __device__ __forceinline__ void plan_count_one(const PlanArgs& p, int64_t t, uns
         p.slot_pos[t] = pos;
         if (pos == 0) rows += (unsigned long long)size;
         pairs += (unsigned long long)size;
-        if (p.sqd) p.dqc[t] = p.sqd[r.q * p.nlist + r.c];      // the probe's value of this pair
     }
     p.probe_c[t] = r.c;
     if (p.slot_off) p.slot_off[t] = r.nr;                       // (offsets after plan_query)
@@ -661,54 +660,69 @@ __global__ void __launch_bounds__(256) merge_kernel(const uint64_t* __restrict__
     for (int j = threadIdx.x; j < kp; j += blockDim.x) cand[q * kp + j] = buf[j];
 }
 
-// Merge for k' <= 32: W warps per query (1, or the block's 8 when queries have
-// many lists), each keeping the k' smallest keys it has seen in a sorted
-// 32-entry list across its lanes.  A warp takes 32 lists at a time, numbers
-// their entries through (a scan of the counts) and reads 32 entries at once
-// whatever list they are in; entries above the query's published threshold
-// (tq, optional: never below its k'-th key) or the warp's k'-th key are dropped
-// before the sort.  Bound by the latency of the chunks' loads and sorts: one
-// query over 313 lists took one warp 170 us, 8 warps 12 us.
+// Merge for k' <= 32: W warps per query (1, 8 or 32), each keeping the k'
+// smallest keys it has seen in a sorted 32-entry list across its lanes.  A warp
+// takes an equal share of the query's lists, up to 32 at a time, numbers their
+// entries through (a scan of the counts) and reads 128 entries at once whatever
+// list they are in; entries above the query's published threshold (tq, optional:
+// never below its k'-th key) or the warp's k'-th key are dropped before the sort.
+// Bound by the latency of its loads and sorts: one query over 313 lists took one
+// warp 170 us, 8 warps 26 us, 32 warps 7 us.
 template <int W>
-__global__ void __launch_bounds__(256) merge32_kernel(const uint64_t* __restrict__ inter,
-                                                      const int32_t* __restrict__ inter_cnt,
-                                                      const int64_t* __restrict__ qbase, int64_t nq, int kp, int lstride,
-                                                      const unsigned long long* __restrict__ tq,
-                                                      uint64_t* __restrict__ cand, DevChecks ck) {
-    __shared__ uint64_t part[W > 1 ? 8 * 32 : 1];
+__global__ void __launch_bounds__(W == 32 ? 1024 : 256) merge32_kernel(
+    const uint64_t* __restrict__ inter, const int32_t* __restrict__ inter_cnt, const int64_t* __restrict__ qbase,
+    int64_t nq, int kp, int lstride, const unsigned long long* __restrict__ tq, uint64_t* __restrict__ cand,
+    DevChecks ck) {
+    __shared__ uint64_t part[W > 1 ? W * 32 : 1];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t q = W > 1 ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * 8 + warp;
     if (W == 1 && q >= nq) return;
     const int64_t L0 = qbase[q], L1 = qbase[q + 1];
+    const int per = W > 1 ? (int)imin64(32, (L1 - L0 + W - 1) / W) : 32;       // (0 without lists)
     const uint64_t top = tq ? (uint64_t)tq[q] : kEmptyKey;
     uint64_t list = kEmptyKey, th = kEmptyKey;
-    for (int64_t Lb = L0 + (W > 1 ? 32 * warp : 0); Lb < L1; Lb += 32 * W) {
+    for (int64_t Lb = L0 + (W > 1 ? per * warp : 0); Lb < L1; Lb += per * W) {
         if (!ERQ_DCHECK(Lb >= 0 && L1 <= ck.lists, ck.status, 1)) break;
-        const int nl = (int)imin64(32, L1 - Lb);
+        const int nl = (int)imin64(per, L1 - Lb);
         int n = lane < nl ? inter_cnt[Lb + lane] : 0;
         if (!ERQ_DCHECK(n >= 0 && n <= lstride, ck.status, 1)) n = 0;
         const int incl = warp_incl_scan(n), total = __shfl_sync(0xffffffffu, incl, 31);
-        for (int e0 = 0; e0 < total; e0 += 32) {
-            const int e = e0 + lane;
-            int j = 0;                                             // lists that end at or before entry e
+        for (int e0 = 0; e0 < total; e0 += 128) {
+            uint64_t key[4];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-                if (__shfl_sync(0xffffffffu, incl, j + o - 1) <= e) j += o;
-            j = min(j, 31);                                        // (entries past the last)
-            const int prev = __shfl_sync(0xffffffffu, incl, max(j - 1, 0)), before = j > 0 ? prev : 0;
-            const uint64_t key = e < total ? inter[(Lb + j) * lstride + (e - before)] : kEmptyKey;
-            const bool pass = key <= top && key < th;
-            if (!__any_sync(0xffffffffu, pass)) continue;
-            list = ws_merge32(list, ws_sort32(pass ? key : kEmptyKey, lane), lane);
-            th = ws_shfl(list, kp - 1);
+            for (int u = 0; u < 4; ++u) {
+                key[u] = kEmptyKey;
+                if (e0 + 32 * u >= total) continue;
+                const int e = e0 + 32 * u + lane;
+                int j = 0;                                             // lists that end at or before entry e
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+                    if (__shfl_sync(0xffffffffu, incl, j + o - 1) <= e) j += o;
+                j = min(j, 31);                                        // (entries past the last)
+                const int prev = __shfl_sync(0xffffffffu, incl, max(j - 1, 0)), before = j > 0 ? prev : 0;
+                if (e < total) key[u] = inter[(Lb + j) * lstride + (e - before)];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (e0 + 32 * u >= total) break;
+                const bool pass = key[u] <= top && key[u] < th;
+                if (!__any_sync(0xffffffffu, pass)) continue;
+                list = ws_merge32(list, ws_sort32(pass ? key[u] : kEmptyKey, lane), lane);
+                th = ws_shfl(list, kp - 1);
+            }
         }
     }
     if (W > 1) {
         part[warp * 32 + lane] = list;
-        __syncthreads();
-        if (warp != 0) return;
 #pragma unroll 1
-        for (int w = 1; w < 8; ++w) list = ws_merge32(list, part[w * 32 + lane], lane);
+        for (int h = W / 2; h > 0; h >>= 1) {
+            __syncthreads();
+            if (warp < h) {
+                list = ws_merge32(list, part[(warp + h) * 32 + lane], lane);
+                part[warp * 32 + lane] = list;
+            }
+        }
+        if (warp != 0) return;
     }
     if (lane < kp) cand[q * kp + lane] = list;
 }
@@ -1057,7 +1071,7 @@ cudaError_t launch_dqc(const float* Q, const float* C, const int32_t* probe, con
     return cudaGetLastError();
 }
 
-// The pairs' validation, places and probe values (all that the two-stage search needs).
+// The pairs' validation and places (all that the two-stage search needs).
 cudaError_t launch_plan_count(const PlanArgs& p, cudaStream_t s) {
     const int64_t pairs = p.nq * p.maxp;
     cudaError_t e;
@@ -1185,8 +1199,11 @@ cudaError_t launch_merge(const uint64_t* inter, const int32_t* inter_cnt, const 
     if (kp <= 32) {
         count_launch();
         // eight warps per query where there are lists for them (more than 32 a
-        // query) or too few queries to fill the chip with one warp each
-        if (ck.lists > 32 * nq || nq < 2048)
+        // query) or too few queries to fill the chip with one warp each; a whole
+        // block's 32 while each query can have an SM's half to itself
+        if (nq <= 256 && ck.lists > 32 * nq)
+            merge32_kernel<32><<<(unsigned)nq, 1024, 0, s>>>(inter, inter_cnt, qbase, nq, kp, lstride, tq, cand, ck);
+        else if (ck.lists > 32 * nq || nq < 2048)
             merge32_kernel<8><<<(unsigned)nq, 256, 0, s>>>(inter, inter_cnt, qbase, nq, kp, lstride, tq, cand, ck);
         else
             merge32_kernel<1><<<(unsigned)ceil_div(nq, 8), 256, 0, s>>>(inter, inter_cnt, qbase, nq, kp, lstride, tq, cand,

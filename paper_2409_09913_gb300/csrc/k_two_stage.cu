@@ -27,6 +27,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "erq_kernels.cuh"
 #include "erq_search.cuh"
 
@@ -139,30 +141,42 @@ struct TsArgs {
     float eps0;
 };
 
-// Block per (query, probe slot); thread per row of the probed cluster.
+// Block per (query, probe slot, share of the cluster's 128-row chunks); thread
+// per row.  Bound by the latency of a row's chain of table reads and additions,
+// so a cluster is shared by as many blocks as it has chunks while the chip has
+// room for them (16 queries x 16 lists of 200,000 x 960 in 1,024: 101 us with a
+// block per list, 19 us); four blocks' plane words are fetched ahead of
+// their table reads.  The sum's order is that of one pass over the coordinates.
 __global__ void __launch_bounds__(TS_THREADS) ts_stage1_kernel(TsArgs a) {
     extern __shared__ __align__(16) float tab[];          // [D/4][16]
     const int64_t q = blockIdx.x / a.maxp;
     const int slot = (int)(blockIdx.x % a.maxp);
     const int c = a.probe_c[q * a.maxp + slot];
     if (c < 0) return;
+    const int64_t size = a.list_off[c + 1] - a.list_off[c], pc = a.poff[c];
+    if ((int64_t)blockIdx.y * TS_THREADS >= size) return;
     const int D = a.D, B = a.B, nkb = D / 64;
     const float4* src = reinterpret_cast<const float4*>(a.T + q * (int64_t)D * 4);
     for (int i = threadIdx.x; i < D; i += TS_THREADS) reinterpret_cast<float4*>(tab)[i] = src[i];
     __syncthreads();
-    const int64_t size = a.list_off[c + 1] - a.list_off[c], pc = a.poff[c];
     const float dq = a.dqc[q * a.maxp + slot];
     const float bq = a.eps0 * sqrtf(fmaxf(dq, 0.f));
     const int64_t o0 = a.qoffr[q] + a.rbase[q * a.maxp + slot];
-    for (int64_t j = threadIdx.x; j < size; j += TS_THREADS) {
+    for (int64_t j = (int64_t)blockIdx.y * TS_THREADS + threadIdx.x; j < size; j += (int64_t)gridDim.y * TS_THREADS) {
         const int64_t p = pc + j;
         const uint64_t* w = a.codes_p + ((p >> 5) * nkb * B + (B - 1)) * 32 + (p & 31);
         float s = 0.f;
-        for (int kb = 0; kb < nkb; ++kb) {
-            const uint64_t W = __ldg(w + (int64_t)kb * B * 32);
-            const float* t = tab + kb * 256;
+        for (int k0 = 0; k0 < nkb; k0 += 4) {
+            uint64_t W[4];
 #pragma unroll
-            for (int n = 0; n < 16; ++n) s += t[16 * n + (int)((W >> (4 * n)) & 15u)];
+            for (int u = 0; u < 4; ++u) W[u] = k0 + u < nkb ? __ldg(w + (int64_t)(k0 + u) * B * 32) : 0ull;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (k0 + u >= nkb) break;
+                const float* t = tab + (k0 + u) * 256;
+#pragma unroll
+                for (int n = 0; n < 16; ++n) s += t[16 * n + (int)((W[u] >> (4 * n)) & 15u)];
+            }
         }
         const float4 m = a.meta1[p];
         const float est1 = dq + m.x + m.y * s, bd = bq * m.z;
@@ -185,15 +199,19 @@ __device__ K block_select_kth(const K* keys, int64_t n, int64_t k, unsigned* his
             if ((v & mask) == prefix) atomicAdd(&hist[(int)((v >> shift) & 255)], 1u);
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            int64_t cum = 0;
-            int d = 0;
-            for (; d < 255; ++d) {
-                if (cum + hist[d] >= k) break;
-                cum += hist[d];
+        if (threadIdx.x < 32) {                     // first digit whose running count reaches k, eight a lane
+            unsigned c[8], own = 0;
+#pragma unroll
+            for (int d = 0; d < 8; ++d) own += c[d] = hist[8 * threadIdx.x + d];
+            unsigned run = (unsigned)warp_incl_scan((int)own) - own;
+#pragma unroll
+            for (int d = 0; d < 8; ++d) {
+                if ((int64_t)run < k && (int64_t)(run + c[d]) >= k) {
+                    *s_pre = prefix | ((K)(8 * threadIdx.x + d) << shift);
+                    *s_k = k - run;
+                }
+                run += c[d];
             }
-            *s_pre = prefix | ((K)d << shift);
-            *s_k = k - cum;
         }
         __syncthreads();
         prefix = *s_pre;
@@ -261,49 +279,62 @@ __device__ __forceinline__ float last_bits_dot(const uint64_t* w, const float* x
     return acc;
 }
 
+// The survivors' full estimates (Eq. 4.2) and keys.  Block per (query, probe
+// slot, share of the cluster's 128-row chunks), a warp per 32 rows at a time:
+// survivors are few, so a row's 64-coordinate blocks go to the lanes, G =
+// 32 / W rows side by side with W the power of two that holds them (one row in
+// several rounds beyond 2,048 coordinates); the blocks' sums are then added in
+// order.  A thread per row kept 30 of a warp's lanes waiting for the other two:
+// 134 us for 16 queries x 16 lists of 200,000 x 960 in 1,024, 34 us.  Query
+// coordinates are spaced 65 floats a block so that the lanes' reads fall into
+// different banks.
 template <int B>
-__device__ float last_bits_row(const uint64_t* w0, int nkb, const float* x) {
-    float s = 0.f;
-    for (int kb = 0; kb < nkb; ++kb) s += last_bits_dot<B>(w0 + (int64_t)kb * B * 32, x + 64 * kb);
-    return s;
-}
-
-__device__ float last_bits_row_b(int B, const uint64_t* w0, int nkb, const float* x) {
-    switch (B) {
-        case 1: return 0.f;
-        case 2: return last_bits_row<2>(w0, nkb, x);
-        case 3: return last_bits_row<3>(w0, nkb, x);
-        case 5: return last_bits_row<5>(w0, nkb, x);
-        case 6: return last_bits_row<6>(w0, nkb, x);
-        case 7: return last_bits_row<7>(w0, nkb, x);
-        case 8: return last_bits_row<8>(w0, nkb, x);
-        default: return last_bits_row<9>(w0, nkb, x);
-    }
-}
-
-// Block per (query, probe slot): the survivors' full estimates (Eq. 4.2) and keys.
 __global__ void __launch_bounds__(TS_THREADS) ts_stage2_kernel(TsArgs a) {
-    extern __shared__ __align__(16) float xq[];            // [D] P^T q_r
+    extern __shared__ __align__(16) float xq[];            // [D / 64][65] P^T q_r
     const int64_t q = blockIdx.x / a.maxp;
     const int slot = (int)(blockIdx.x % a.maxp);
     const int c = a.probe_c[q * a.maxp + slot];
     if (c < 0) return;
-    const int D = a.D, B = a.B, nkb = D / 64;
-    for (int i = threadIdx.x; i < D; i += TS_THREADS) xq[i] = a.Qrot[q * D + i];
-    __syncthreads();
     const int64_t size = a.list_off[c + 1] - a.list_off[c], pc = a.poff[c];
+    if ((int64_t)blockIdx.y * TS_THREADS >= size) return;
+    const int D = a.D, nkb = D / 64;
+    for (int i = threadIdx.x; i < D; i += TS_THREADS) xq[(i >> 6) * 65 + (i & 63)] = a.Qrot[q * D + i];
+    __syncthreads();
     const float dq = a.dqc[q * a.maxp + slot], tq = a.tau[q];
     const int64_t o0 = a.qoffr[q] + a.rbase[q * a.maxp + slot];
     const float hi = (float)(1 << (B - 1));
-    for (int64_t j = threadIdx.x; j < size; j += TS_THREADS) {
-        if (a.lb[o0 + j] > tq) continue;
-        const int64_t p = pc + j;
-        const uint64_t* w0 = a.codes_p + ((p >> 5) * nkb * B) * 32 + (p & 31);
-        const float s = fmaf(hi, a.s1[o0 + j], last_bits_row_b(B, w0, nkb, xq));
-        const float4 m = a.rowmeta[p];
-        const float est = dq + fmaf(m.y, s, m.x);
-        const int pos = atomicAdd(a.scnt + q, 1);
-        a.skey[a.qoffr[q] + pos] = make_key(est, __float_as_uint(m.z));
+    const int lane = threadIdx.x & 31;
+    int W = 1;
+    while (W < nkb && W < 32) W <<= 1;
+    const int G = 32 / W, g = lane / W, kl = lane & (W - 1);
+    for (int64_t j0 = (int64_t)blockIdx.y * TS_THREADS + (threadIdx.x & ~31); j0 < size;
+         j0 += (int64_t)gridDim.y * TS_THREADS) {
+        const int64_t j = j0 + lane;
+        // (a comparison that keeps rows without an ordered bound)
+        unsigned live = __ballot_sync(0xffffffffu, j < size && !(a.lb[o0 + j] > tq));
+        while (live) {
+            unsigned rest = live;
+            int r = -1;                                    // my group's row: the (g + 1)-th survivor
+            for (int u = 0; u < G && rest; ++u) {
+                if (u == g) r = __ffs(rest) - 1;
+                rest &= rest - 1;
+            }
+            live = rest;
+            const int64_t p = pc + j0 + max(r, 0);
+            const uint64_t* w0 = a.codes_p + ((p >> 5) * nkb * B) * 32 + (p & 31);
+            float s = 0.f;
+            for (int k0 = 0; k0 < nkb; k0 += W) {
+                const int kb = k0 + kl;
+                const float v = B > 1 && r >= 0 && kb < nkb ? last_bits_dot<B>(w0 + (int64_t)kb * B * 32, xq + 65 * kb) : 0.f;
+                for (int u = 0; u < W && k0 + u < nkb; ++u) s += __shfl_sync(0xffffffffu, v, (lane & ~(W - 1)) + u);
+            }
+            if (r >= 0 && kl == 0) {
+                const float4 m = a.rowmeta[p];
+                const float est = dq + fmaf(m.y, fmaf(hi, a.s1[o0 + j0 + r], s), m.x);
+                const int pos = atomicAdd(a.scnt + q, 1);
+                a.skey[a.qoffr[q] + pos] = make_key(est, __float_as_uint(m.z));
+            }
+        }
     }
 }
 
@@ -386,19 +417,35 @@ cudaError_t launch_two_stage(const TwoStageLaunch& L, cudaStream_t s) {
     a.rowmeta = L.rowmeta; a.meta1 = L.meta1; a.T = L.T; a.Qrot = L.Qrot; a.rbase = L.rbase; a.qoffr = L.qoffr;
     a.ub = L.ub; a.lb = L.lb; a.s1 = L.s1; a.tau = L.tau; a.scnt = L.scnt; a.skey = L.skey;
     a.nq = L.nq; a.maxp = L.maxp; a.D = L.D; a.B = L.B; a.eps0 = L.eps0;
+    // blocks a list: one a 128-row chunk of the largest list, up to sixteen an SM in all
     const int64_t blocks = L.nq * L.maxp;
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t share = std::max<int64_t>(1, std::min<int64_t>(ceil_div(L.max_list, TS_THREADS), 16 * (int64_t)sms / blocks));
+    const dim3 grid((unsigned)blocks, (unsigned)std::min<int64_t>(share, 65535));
     const size_t tab_bytes = (size_t)L.D * 16;
     cudaError_t e = cudaFuncSetAttribute(ts_stage1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tab_bytes);
     if (e != cudaSuccess) return e;
     count_launch();
     msb_table_kernel<<<(unsigned)ceil_div(L.nq * (L.D / 4) * 16, 256), 256, 0, s>>>(L.Qrot, L.nq, L.D, L.T);
     count_launch();
-    ts_stage1_kernel<<<(unsigned)blocks, TS_THREADS, tab_bytes, s>>>(a);
+    ts_stage1_kernel<<<grid, TS_THREADS, tab_bytes, s>>>(a);
     count_launch();
     ts_tau_kernel<<<(unsigned)L.nq, 256, 0, s>>>(L.ub, L.qoffr, L.nq, L.kp, L.tau, L.scratch);
     if ((e = cudaMemsetAsync(L.scnt, 0, sizeof(int32_t) * L.nq, s)) != cudaSuccess) return e;
     count_launch();
-    ts_stage2_kernel<<<(unsigned)blocks, TS_THREADS, (size_t)L.D * 4, s>>>(a);
+    const size_t xq_bytes = (size_t)(L.D / 64) * 65 * 4;
+    switch (L.B) {
+        case 1: ts_stage2_kernel<1><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 2: ts_stage2_kernel<2><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 3: ts_stage2_kernel<3><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 5: ts_stage2_kernel<5><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 6: ts_stage2_kernel<6><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 7: ts_stage2_kernel<7><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 8: ts_stage2_kernel<8><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
+        default: ts_stage2_kernel<9><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
+    }
     count_launch();
     ts_select_kernel<<<(unsigned)L.nq, 256, 0, s>>>(L.skey, L.qoffr, L.scnt, L.nq, L.kp, L.cand);
     return cudaGetLastError();
