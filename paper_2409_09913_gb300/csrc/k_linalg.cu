@@ -319,17 +319,64 @@ __global__ void row_sqnorm_kernel(const float* __restrict__ X, int64_t n, int D,
 // vectors): y = fl32(x / sqrt(sum x^2)) with the sum in FP64, one warp per
 // row; a zero row stays zero.  X and Y may be the same array (each thread
 // rewrites only the elements it read).
-__global__ void normalize_rows_kernel(const float* X, int64_t n, int D, float* Y) {
+//
+// The FP64 pipe does two lanes a clock, and a division is some twenty of its
+// instructions: dividing every element took 184 us for 4,000 x 1,536, 43 us
+// with the division done in FP32 pairs.  1 / norm is split as r + t (one
+// FP64 division a row); x r is formed as a product and its exact remainder, x t
+// is added to the remainder, and the pair (product, remainder) is x / norm to
+// 2^-45.  Its rounding to FP32 is x / norm's unless the part dropped lies within
+// 2^-45 of a rounding boundary; those elements (2^-18 of them), those of a power
+// of two and those too small for an exact remainder are divided in FP64.
+__device__ __forceinline__ float div_by_norm(float x, double nrm, float r, float t) {
+    if (x == 0.f) return x;
+    const float y = x * r;
+    const float e = fmaf(x, t, fmaf(x, r, -y));
+    const float s = y + e, d = e - (s - y);                     // y + e = s + d exactly (|e| << |y|)
+    const uint32_t b = __float_as_uint(s) & 0x7fffffffu;
+    const float half = __uint_as_float(b & 0x7f800000u) * 5.9604644775390625e-8f;   // half the spacing at s: 2^-24
+    if (fabsf(y) >= 1.2621774e-29f && fabsf(y) <= 1e30f && (b & 0x7fffffu) != 0u &&
+        fabsf(d) <= half * 0.999998f)
+        return s;
+    return (float)((double)x / nrm);
+}
+
+__global__ void __launch_bounds__(256) normalize_rows_kernel(const float* X, int64_t n, int D, float* Y) {
     const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (r >= n) return;
     const float* x = X + r * D;
     double s = 0.0;
-    for (int k = lane; k < D; k += 32) s += (double)x[k] * (double)x[k];
+    int k = lane;
+    for (; k + 224 < D; k += 256) {                             // eight loads in flight
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = x[k + 32 * u];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s += (double)v[u] * (double)v[u];
+    }
+    for (; k < D; k += 32) s += (double)x[k] * (double)x[k];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     const double nrm = sqrt(s);
     float* y = Y + r * D;
-    for (int k = lane; k < D; k += 32) y[k] = nrm > 0.0 ? (float)((double)x[k] / nrm) : 0.f;
+    if (!(nrm > 0.0)) {
+        for (k = lane; k < D; k += 32) y[k] = 0.f;
+        return;
+    }
+    const double inv = 1.0 / nrm;
+    if (!(inv > 1e-30 && inv < 1e30)) {                         // (r and t would leave FP32's normal range)
+        for (k = lane; k < D; k += 32) y[k] = (float)((double)x[k] / nrm);
+        return;
+    }
+    const float ir = (float)inv, it = (float)(inv - (double)ir);
+    for (k = lane; k + 224 < D; k += 256) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = x[k + 32 * u];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) y[k + 32 * u] = div_by_norm(v[u], nrm, ir, it);
+    }
+    for (; k < D; k += 32) y[k] = div_by_norm(x[k], nrm, ir, it);
 }
 
 cudaError_t launch_normalize_rows(const float* X, int64_t n, int D, float* Y, cudaStream_t s) {

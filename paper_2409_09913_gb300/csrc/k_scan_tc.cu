@@ -1303,7 +1303,11 @@ __global__ void quant_e4m3_kernel(const float* __restrict__ X, int64_t n, int D,
     if (r >= n) return;
     const float* x = X + r * D;
     float m = 0.f;
-    for (int i = lane; i < D; i += 32) m = fmaxf(m, fabsf(x[i]));
+#pragma unroll 4
+    for (int i = lane * 4; i < D; i += 128) {              // (D % 64 == 0, rows on 16-byte boundaries)
+        const float4 v = *reinterpret_cast<const float4*>(x + i);
+        m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+    }
     m = warp_max(m);
     int e = 0;
     if (m > 0.f) {
@@ -1314,21 +1318,27 @@ __global__ void quant_e4m3_kernel(const float* __restrict__ X, int64_t n, int D,
     const float inv = __int_as_float((127 - e) << 23), s = __int_as_float((127 + e) << 23);
     if (lane == 0) scale[r] = m > 0.f ? s : 1.f;
     unsigned char* y = Y + r * Dq;
-    for (int i = lane * 4; i < Dq; i += 128) {
+#pragma unroll 4
+    for (int c = lane * 4; c < (dup ? D : Dq); c += 128) {
         uint32_t w = 0u;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = dup ? (((i + j) >> 7) << 6) | ((i + j) & 63) : i + j;
-            if (c < D) w |= e4m3_rn(x[c] * inv) << (8 * j);
+        if (c < D) {
+            const float4 v = *reinterpret_cast<const float4*>(x + c);
+            w = e4m3_rn(v.x * inv) | e4m3_rn(v.y * inv) << 8 | e4m3_rn(v.z * inv) << 16 | e4m3_rn(v.w * inv) << 24;
         }
-        *reinterpret_cast<uint32_t*>(y + i) = w;
+        if (dup) {                                             // four coordinates of one block, in both of its copies
+            const int i = ((c >> 6) << 7) | (c & 63);
+            *reinterpret_cast<uint32_t*>(y + i) = w;
+            *reinterpret_cast<uint32_t*>(y + i + 64) = w;
+        } else {
+            *reinterpret_cast<uint32_t*>(y + c) = w;
+        }
     }
 }
 
 cudaError_t launch_quant_e4m3(const float* x, int64_t n, int D, int Dq, int dup, unsigned char* y, float* scale,
                               cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    if (Dq % 4 != 0 || (dup && Dq != 2 * D) || (!dup && Dq < D)) return cudaErrorInvalidValue;
+    if (D % 4 != 0 || ((uintptr_t)x & 15) != 0 || Dq % 4 != 0 || (dup && Dq != 2 * D) || (!dup && Dq < D)) return cudaErrorInvalidValue;
     count_launch();
     quant_e4m3_kernel<<<(unsigned)ceil_div(n * 32, 256), 256, 0, s>>>(x, n, D, Dq, dup, y, scale);
     return cudaGetLastError();
