@@ -28,36 +28,40 @@
 // 64-coordinate K block of the group, a unit one row block of a stage.  Units
 // are numbered through the CTA's life, and so are row blocks.  Warp roles (28
 // warps):
-//   warps 0-7    epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (its 32
-//                rows) of every finished accumulator, 16 queries at a time, the
-//                even 16-column groups in warps 0-3 and the odd ones in 4-7; one
-//                compare per value against the query's threshold (in the units
-//                of g + (f_res/2) acc) and one vote per query; a query with a
-//                candidate gets its exact keys appended to the query's list in
-//                shared memory (one atomic per query and warp).  Lists beyond
-//                their shared capacity continue in global memory; after a row
-//                block the lists above TRIG entries are cut to (about) their k'
-//                smallest, which also lowers the query's threshold;
-//   warps 8-23   converters, four sets of four warps: set U % 4 unpacks unit U,
+//   warps 0-15   epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (its 32
+//                rows) of every finished accumulator, the 16-query column groups
+//                going round the quarter's four warps; the values are held in
+//                registers, the accumulator is released, one compare per value
+//                against the query's threshold (in the units of g + (f_res/2)
+//                acc) gives each thread a mask of its candidates, and every
+//                thread appends its own to the queries' lists in shared memory
+//                (one atomic each; two or three rounds a warp and row block).
+//                Lists beyond their shared capacity continue in global memory;
+//                after a row block the lists above TRIG entries are cut to (about)
+//                their k' smallest, which also lowers the query's threshold;
+//   warps 16-23  converters, two sets of four warps: set U % 2 unpacks unit U,
 //                one thread per row, from the raw ring in shared memory into FP16
 //                (or e4m3) values in TMEM slot U % AS;
 //   warp 24      code loader: publishes the items, per row block a bulk copy of
 //                the rows' factors and ids, per unit one TMA load of the packed
 //                codes into a raw ring that is released as soon as the
 //                converters have read it (the ring's length is a multiple of
-//                four, so that each slot belongs to one converter set, which
+//                two, so that each slot belongs to one converter set, which
 //                awaits its phases in order);
 //   warps 25, 26 query loaders: per stage the item's query rows by TMA gather4
 //                into the stage's swizzled B tile, the stages taken in turn;
 //   warp 27      MMA issuer (one elected thread; owner of the tensor memory).
 //                Row blocks take the accumulators in turn (NACC of them), so
 //                that one is drained while the others fill.
-// Measured before this arrangement (per-role clocks; 10,000 queries x 16 lists
-// of 400k x 960): the issuer waited 44 % of its time for converted codes
-// (a unit takes one warp about 1,200 cycles, so eight converter warps gave one
-// unit per 600 cycles against 128-256 of tensor time), and with 128 queries
-// per item a single estimate tile between four tile warps and ten filter warps
-// serialised both; an admission cost 2,000-3,000 cycles of one filter warp.
+// What bounds it, by per-role clocks: with short lists and wide queries (zipf,
+// 16,384 queries x 256 lists at D = 768) nothing alone - converters are busy half
+// of the time, the issuer waits a quarter of it for an accumulator and a sixth for
+// query tiles, which come from the L2 at 2.4 TB/s; at D = 192 the epilogue (list
+// cuts and appends); with split e4m3 codes the converters. Measured against eight
+// epilogue warps with one vote per query and four converter sets: 10,000 queries x
+// 16 lists of 400,000 x 960, 0.51 -> 0.31 ms; zipf above, 3.64 -> 2.53 ms.  Unrolled
+// appends or a cut inlined three times over made every role slower, bound by the
+// instruction cache.
 // A query starts from the smallest threshold published so far by its items,
 // which is never below its final k'-th key, so each list stays a superset of
 // what the item contributes.
@@ -87,7 +91,6 @@ static_assert(MR == 128, "four 32-row lane quarters per row block");
 constexpr int KB = 64;           // FP16 elements per K block (one 128-byte swizzle row)
 constexpr int RP = 2;            // row blocks per stage group
 constexpr int MS = 4;            // row-factor buffers
-constexpr int AS = 8;            // TMEM slots of converted units (32 columns each)
 constexpr int RSMAX = 16;        // raw-code ring slots at most
 constexpr int NEP = 16;          // epilogue warps 0 .. NEP - 1 (a multiple of four)
 constexpr int W_CV = NEP;        // converter warps: set (w - W_CV) / 4, lane quarter w % 4
@@ -99,19 +102,27 @@ constexpr int W_MMA = W_QL + NQL;       // MMA issuer, TMEM owner
 constexpr int NWARP = W_MMA + 1;
 constexpr int THREADS = 32 * NWARP;
 constexpr int TMEM_COLS = 512;
-constexpr int ACOL = TMEM_COLS - AS * (KB / 2);   // first TMEM column of the code slots
 constexpr int KCAP = 128;        // largest k' of the tensor-core path
 constexpr int SP = 128;          // entries of a list's continuation in global memory
 constexpr int BAR_EP = 1;        // named barrier of the epilogue warps
-static_assert(AS % NSET == 0 && W_CV % 4 == 0, "a set owns whole slots and its warps their lane quarters");
+static_assert(W_CV % 4 == 0, "a set's warps own their lane quarters");
 
 // Work-item capacities: QN queries per item at most (the MMA's N extent), KC
 // shared list entries per query, TRIG entries above which a list is cut after a
-// row block, LS query-tile stages of QB bytes per query, RAWK KB of raw ring.
-template <int QN_, int KC_, int TRIG_, int LS_, int QB_, int RAWK_>
+// row block, LS query-tile stages of QB bytes per query, RAWK KB of raw ring, AS
+// TMEM slots of converted units (32 columns each), EX how a list is cut
+// (ListRegs::bound).  TMEM not taken by the slots holds the accumulators: with
+// 128 queries four slots leave three, so that a stage group's two row blocks
+// start while the last one's second is still read out (16,384 queries x 256 lists
+// at D = 768: 2.67 -> 2.53 ms against eight slots and two accumulators).
+template <int QN_, int KC_, int TRIG_, int LS_, int QB_, int RAWK_, int AS_, bool EX_ = false>
 struct Cfg {
     static constexpr int QN = QN_, KC = KC_, TRIG = TRIG_, LS = LS_, QB = QB_;
+    static constexpr int AS = AS_;
+    static constexpr bool EX = EX_;
+    static constexpr int ACOL = TMEM_COLS - AS * (KB / 2);   // first TMEM column of the code slots
     static constexpr int NACC = ACOL / QN;           // accumulators
+    static_assert(AS % NSET == 0, "a set owns whole slots");
     static constexpr int RAW_BYTES = RAWK_ * 1024;
     static constexpr int TILE_Q = QN * QB;           // one stage's query tile
     static_assert(NACC >= RP && QN % 32 == 0, "a stage group's accumulators fit");
@@ -156,11 +167,15 @@ struct Cfg {
     // a barrier nothing arrives on (the test stall of the bounded-wait path)
     static constexpr int b_never() { return 8 * (B1 + 2 * MS + 5); }
 };
-using CfgA = Cfg<64, 160, 96, 6, 128, 48>;    // k' <= 32, up to 64 queries per item
-using CfgW = Cfg<128, 96, 88, 4, 128, 40>;    // k' <= 32, up to 128 queries per item
-using CfgB = Cfg<32, 256, 160, 6, 128, 48>;   // k' <= 128, up to 32 queries per item
-using CfgA32 = Cfg<64, 160, 96, 4, 256, 48>;  // the same with two query parts (FP32 precision)
-using CfgB32 = Cfg<32, 256, 160, 6, 256, 48>;
+using CfgA = Cfg<64, 160, 96, 6, 128, 48, 8>;    // k' <= 32, up to 64 queries per item
+using CfgW = Cfg<128, 96, 88, 4, 128, 40, 4>;    // k' <= 32, up to 128 queries per item
+using CfgB = Cfg<32, 256, 160, 6, 128, 48, 8>;   // k' <= 128, up to 32 queries per item
+using CfgA32 = Cfg<64, 160, 96, 4, 256, 48, 8>;  // the same with two query parts (FP32 precision)
+using CfgB32 = Cfg<32, 256, 160, 6, 256, 48, 8>;
+using CfgAx = Cfg<64, 160, 96, 6, 128, 48, 8, true>;   // KMIN < k' <= 32
+using CfgWx = Cfg<128, 96, 88, 4, 128, 40, 4, true>;
+using CfgA32x = Cfg<64, 160, 96, 4, 256, 48, 8, true>;
+constexpr int KMIN = 24;
 
 // arrivals that complete a phase of the item-release barrier: one per warp of
 // the epilogue, the converters, the query loaders and the issuer
@@ -383,6 +398,44 @@ __device__ __forceinline__ float relaxed_threshold(float tf, float dq) {
     return (tf - dq) + (0x1p-20f * (fabsf(tf) + fabsf(dq)) + 0x1p-120f);
 }
 
+__device__ __forceinline__ uint32_t sort32_step(uint32_t m, int d, bool asc, int lane) {
+    const uint32_t p = __shfl_xor_sync(0xffffffffu, m, d);
+    return ((lane & d) == 0) == asc ? min(m, p) : max(m, p);
+}
+// Of two ascending lists across the lanes, the 32 smallest, ascending.
+__device__ __forceinline__ uint32_t merge32_u32(uint32_t x, uint32_t y, int lane) {
+    uint32_t m = min(x, __shfl_sync(0xffffffffu, y, 31 - lane));
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) m = sort32_step(m, d, true, lane);
+    return m;
+}
+
+// The kp-th smallest (kp <= 32) estimate, as its order-preserving integer, of a
+// list of cnt keys (kc in shared memory, the rest in `spill`): 128 keys at a time
+// are sorted in runs of 32 side by side, which are merged into the 32 smallest
+// so far.
+__device__ __forceinline__ uint32_t list_kth(const uint64_t* list, const uint64_t* spill, int cnt, int kc, int kp, int lane) {
+    uint32_t best = 0xffffffffu;
+#pragma unroll 1
+    for (int e0 = 0; e0 < cnt; e0 += 128) {
+        uint32_t c[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int e = e0 + 32 * u + lane;
+            c[u] = 0xffffffffu;
+            if (e < cnt) c[u] = (uint32_t)((e < kc ? list[e] : __ldcg(spill + (e - kc))) >> 32);
+        }
+#pragma unroll
+        for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+            for (int d = size >> 1; d > 0; d >>= 1)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) c[u] = sort32_step(c[u], d, size == 32 || (lane & size) == 0, lane);
+        best = merge32_u32(best, merge32_u32(merge32_u32(c[0], c[1], lane), merge32_u32(c[2], c[3], lane), lane), lane);
+    }
+    return __shfl_sync(0xffffffffu, best, kp - 1);
+}
+
 // One query's list (cnt entries: KC in shared memory, the rest in `spill`),
 // held by a warp as keys e = 32 j + lane in v[j].
 template <int KC>
@@ -417,23 +470,29 @@ struct ListRegs {
         return n;
     }
     // A key that at least kp entries do not exceed and at most `most` do (kp <=
-    // cnt, kp <= most).  For kp <= 32 the kp-th smallest of the lanes' smallest
-    // estimates: kp lanes hold an entry at or below it.  Where that admits too
-    // many (or kp > 32), the exact kp-th key bit by bit.
-    __device__ __forceinline__ uint64_t bound(int kp, int most, int lane) const {
+    // cnt, kp <= most).  For kp <= 32 every key of an estimate: with EX the kp-th
+    // smallest (`kth`, list_kth's), else the kp-th smallest of the lanes' smallest (kp lanes
+    // hold an entry at or below it).  Where that admits too many (or kp > 32), the
+    // exact kp-th key bit by bit.
+    // The lanes' minima are the cheaper, but of 128 entries they let 28 stay at kp =
+    // 20, 37 at 24 and 74 at 32, so that lists fill again at once or are cut bit by
+    // bit (64 rounds of votes, 4,000 cycles): EX from kp > KMIN (10,770 queries x 38
+    // lists at D = 192, k' = 32: 1.69 -> 1.23 ms; at k' = 20 the sort costs more than
+    // it saves, 4,000 x 32 at D = 1536: 0.32 -> 0.37 ms).
+    template <bool EX>
+    __device__ __forceinline__ uint64_t bound(uint32_t kth, int kp, int most, int lane) const {
         if (kp <= 32) {
-            uint32_t m = 0xffffffffu;
+            if (!EX) {
+                uint32_t m = 0xffffffffu;
 #pragma unroll
-            for (int j = 0; j < E; ++j) m = min(m, (uint32_t)(v[j] >> 32));
+                for (int j = 0; j < E; ++j) m = min(m, (uint32_t)(v[j] >> 32));
 #pragma unroll
-            for (int size = 2; size <= 32; size <<= 1)
+                for (int size = 2; size <= 32; size <<= 1)
 #pragma unroll
-                for (int d = size >> 1; d > 0; d >>= 1) {
-                    const uint32_t p = __shfl_xor_sync(0xffffffffu, m, d);
-                    const bool asc = size == 32 || (lane & size) == 0;
-                    m = ((lane & d) == 0) == asc ? min(m, p) : max(m, p);
-                }
-            const uint64_t k = ((uint64_t)__shfl_sync(0xffffffffu, m, kp - 1) << 32) | 0xffffffffull;
+                    for (int d = size >> 1; d > 0; d >>= 1) m = sort32_step(m, d, size == 32 || (lane & size) == 0, lane);
+                kth = __shfl_sync(0xffffffffu, m, kp - 1);
+            }
+            const uint64_t k = ((uint64_t)kth << 32) | 0xffffffffull;
             if (count_le(k) <= most && k != kEmptyKey) return k;
         }
         uint64_t k = 0;
@@ -491,6 +550,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     constexpr bool SC = F8 || S32;    // scaled queries
     static_assert(C::QB == (S32 ? 256 : 128), "query tile");
     constexpr int QN = C::QN, KC = C::KC, LS = C::LS, NACC = C::NACC, TILE_Q = C::TILE_Q;
+    constexpr int AS = C::AS, ACOL = C::ACOL;
     using Smem = typename C::Smem;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -969,8 +1029,9 @@ __global__ void __launch_bounds__(THREADS, 1)
                         const int q = warp + NEP * (__ffs(todo) - 1);
                         int n = (int)s_cnt[q];
                         ListRegs<KC> L;
+                        const uint32_t kth = C::EX ? list_kth(lists + q * KC, spill + q * SP, n, KC, kp, lane) : 0u;
                         L.load(lists + q * KC, spill + q * SP, n, lane);
-                        const uint64_t k = L.bound(kp, C::TRIG, lane);
+                        const uint64_t k = L.template bound<C::EX>(kth, kp, C::TRIG, lane);
                         __syncwarp();
                         n = L.store_le(lists + q * KC, k, lane);    // (kp <= n, so k is below the empty key)
                         if (lane == 0) {
@@ -1003,8 +1064,10 @@ __global__ void __launch_bounds__(THREADS, 1)
                 for (uint32_t todo = __ballot_sync(0xffffffffu, cl >= kp); todo; todo &= todo - 1u) {
                     const int j = __ffs(todo) - 1, q = warp + NEP * j;
                     ListRegs<KC> L;
-                    L.load(lists + q * KC, spill + q * SP, __shfl_sync(0xffffffffu, cl, j), lane);
-                    const uint64_t k = L.bound(kp, min(C::TRIG, a.lstride), lane);   // (kp <= lstride)
+                    const int m = __shfl_sync(0xffffffffu, cl, j);
+                    const uint32_t kth = C::EX ? list_kth(lists + q * KC, spill + q * SP, m, KC, kp, lane) : 0u;
+                    L.load(lists + q * KC, spill + q * SP, m, lane);
+                    const uint64_t k = L.template bound<C::EX>(kth, kp, min(C::TRIG, a.lstride), lane);   // (kp <= lstride)
                     __syncwarp();
                     const int n = L.store_le(lists + q * KC, k, lane);
                     if (lane == 0) atomicMin(a.tq + iq[q].x, (unsigned long long)k);
@@ -1250,8 +1313,12 @@ erq_status scan_tc(const ScanLaunch& L, int precision, cudaStream_t s) {
     a.stall_stage = L.stall_stage;
     const void* qb = f8 ? L.Q8 : L.Qh;
     const int64_t qrow = f8 ? L.Dq : 2 * (int64_t)L.D;
+    const bool ex = L.kp > KMIN && L.kp <= 32;
+    if (f32 && L.qn > CfgB32::QN && ex) return scan_tc_launch<CfgA32x, 3>(L, a, L.Qh, L.Ql, qrow, s);
     if (f32 && L.qn > CfgB32::QN) return scan_tc_launch<CfgA32, 3>(L, a, L.Qh, L.Ql, qrow, s);
     if (f32) return scan_tc_launch<CfgB32, 3>(L, a, L.Qh, L.Ql, qrow, s);
+    if (ex && L.qn > CfgA::QN) return scan_tc_form<CfgWx>(P, L, a, qb, qrow, s);
+    if (ex && L.qn > CfgB::QN) return scan_tc_form<CfgAx>(P, L, a, qb, qrow, s);
     if (L.kp <= 32 && L.qn > CfgA::QN) return scan_tc_form<CfgW>(P, L, a, qb, qrow, s);
     if (L.kp <= 32 && L.qn > CfgB::QN) return scan_tc_form<CfgA>(P, L, a, qb, qrow, s);
     return scan_tc_form<CfgB>(P, L, a, qb, qrow, s);
