@@ -294,6 +294,65 @@ static erq_status build_kmeans(const float* X, int64_t N, int D, int nlist, cons
     void* gscr = cv.take<char>(gbytes);
     float* xall = cv.take<float>(N);
     cudaError_t e;
+    // Nearest centroids on the tensor cores (launch_assign) where the product is
+    // worth its five launches (2^31 multiply-adds, 50 us of FP32 pipe) and there is
+    // memory for the parts of up to 1 GB of rows at a time; sample rows that fit are
+    // split once for all iterations.
+    struct Parts {
+        cudaStream_t s;
+        char* base = nullptr;
+        ~Parts() { if (base) cudaFreeAsync(base, s); }
+    } parts{s};
+    const int64_t prow = std::min<int64_t>(chunk, std::max<int64_t>(1, (1ll << 30) / (4ll * D)));
+    __half *xhi = nullptr, *xlo = nullptr, *chi = nullptr, *clo = nullptr;
+    int32_t *ex = nullptr, *ec = nullptr, *list = nullptr;
+    bool tc = (double)S * nlist * D >= 2147483648.0 && prow <= 65535ll * 128 && ((uintptr_t)X & 15) == 0;
+    if (tc) {
+        auto carve = [&](Carver& c) {
+            xhi = c.take<__half>((size_t)prow * D);
+            xlo = c.take<__half>((size_t)prow * D);
+            chi = c.take<__half>((size_t)nlist * D);
+            clo = c.take<__half>((size_t)nlist * D);
+            ex = c.take<int32_t>(prow);
+            ec = c.take<int32_t>(nlist);
+            list = c.take<int32_t>(3 * prow + 2);
+        };
+        Carver size(nullptr, 0);
+        carve(size);
+        if (cudaMallocAsync((void**)&parts.base, size.off, s) == cudaSuccess) {
+            Carver c(parts.base, size.off);
+            carve(c);
+        } else {
+            cudaGetLastError();
+            parts.base = nullptr;
+            tc = false;
+        }
+    }
+    const float* split = nullptr;                     // rows whose parts xhi, xlo hold
+    auto assign_rows = [&](const float* rows, const float* norms, int64_t n, int32_t* out) -> erq_status {
+        if (tc && (e = launch_query_prep(ix->C, nlist, D, ec, nullptr, chi, clo, s)) != cudaSuccess)
+            return cuda_fail(e, "kmeans centroid parts");
+        const int64_t step = tc ? prow : chunk;
+        for (int64_t r0 = 0; r0 < n; r0 += step) {
+            const int64_t m = std::min(step, n - r0);
+            const float* x = rows + r0 * D;
+            if (tc) {
+                if (n > step || split != x) {
+                    if ((e = launch_query_prep(x, m, D, ex, nullptr, xhi, xlo, s)) != cudaSuccess)
+                        return cuda_fail(e, "kmeans row parts");
+                    split = x;
+                }
+                if ((e = launch_assign(x, xhi, xlo, ex, norms + r0, m, ix->C, chi, clo, ec, ix->cnorm2, nlist, D, dist,
+                                       list, out + r0, ix->status, s)) != cudaSuccess)
+                    return cuda_fail(e, "kmeans assign");
+                continue;
+            }
+            if ((e = launch_sqdist(x, norms + r0, ix->C, ix->cnorm2, dist, m, nlist, D, s)) != cudaSuccess)
+                return cuda_fail(e, "kmeans dist");
+            if ((e = launch_row_argmin(dist, m, nlist, out + r0, s)) != cudaSuccess) return cuda_fail(e, "kmeans argmin");
+        }
+        return ERQ_OK;
+    };
     if ((e = launch_strided_ids(sid, S, N, p->seed, s)) != cudaSuccess) return cuda_fail(e, "kmeans ids");
     if ((e = launch_gather_rows(X, sid, S, D, Xs, s)) != cudaSuccess) return cuda_fail(e, "kmeans gather");
     if ((e = launch_row_sqnorm(Xs, S, D, xn, s)) != cudaSuccess) return cuda_fail(e, "kmeans norms");
@@ -306,12 +365,7 @@ static erq_status build_kmeans(const float* X, int64_t N, int D, int nlist, cons
     ERQ_CHECK_CUDA(cudaStreamSynchronize(s));
     for (int it = 0; it < iters; ++it) {
         if ((e = launch_row_sqnorm(ix->C, nlist, D, ix->cnorm2, s)) != cudaSuccess) return cuda_fail(e, "kmeans cn");
-        for (int64_t r0 = 0; r0 < S; r0 += chunk) {
-            const int64_t m = std::min(chunk, S - r0);
-            if ((e = launch_sqdist(Xs + r0 * D, xn + r0, ix->C, ix->cnorm2, dist, m, nlist, D, s)) != cudaSuccess)
-                return cuda_fail(e, "kmeans dist");
-            if ((e = launch_row_argmin(dist, m, nlist, sa + r0, s)) != cudaSuccess) return cuda_fail(e, "kmeans argmin");
-        }
+        ERQ_TRY(assign_rows(Xs, xn, S, sa));
         if ((e = launch_group(sa, S, nlist, soff, sids, nullptr, nullptr, gscr, gbytes, ix->status, s)) != cudaSuccess)
             return cuda_fail(e, "kmeans group");
         if ((e = launch_centroids(Xs, soff, sids, nlist, D, ix->C, 1, s)) != cudaSuccess)
@@ -320,12 +374,7 @@ static erq_status build_kmeans(const float* X, int64_t N, int D, int nlist, cons
     // final assignment of every row
     if ((e = launch_row_sqnorm(ix->C, nlist, D, ix->cnorm2, s)) != cudaSuccess) return cuda_fail(e, "kmeans cn");
     if ((e = launch_row_sqnorm(X, N, D, xall, s)) != cudaSuccess) return cuda_fail(e, "kmeans xn");
-    for (int64_t r0 = 0; r0 < N; r0 += chunk) {
-        const int64_t m = std::min(chunk, N - r0);
-        if ((e = launch_sqdist(X + r0 * D, xall + r0, ix->C, ix->cnorm2, dist, m, nlist, D, s)) != cudaSuccess)
-            return cuda_fail(e, "kmeans dist");
-        if ((e = launch_row_argmin(dist, m, nlist, assign + r0, s)) != cudaSuccess) return cuda_fail(e, "kmeans argmin");
-    }
+    ERQ_TRY(assign_rows(X, xall, N, assign));
     ERQ_CHECK_CUDA(cudaStreamSynchronize(s));
     return ERQ_OK;
 }

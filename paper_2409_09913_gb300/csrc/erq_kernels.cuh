@@ -78,6 +78,10 @@ cudaError_t launch_gemm_tma(const __half* Ahi, const __half* Alo, const int32_t*
                             const __half* Blo, const int32_t* eB, int N, int K, float* C, int64_t ldc, int epi,
                             const float* rown, const float* coln, float* gmin, uint32_t* status, cudaStream_t s,
                             __half* Ch = nullptr, const float* addend = nullptr);
+cudaError_t launch_assign(const float* X, const __half* Xhi, const __half* Xlo, const int32_t* eX, const float* xn,
+                          int64_t rows, const float* C, const __half* Chi, const __half* Clo, const int32_t* eC,
+                          const float* cn, int nc, int D, float* V, int32_t* list, int32_t* out, uint32_t* status,
+                          cudaStream_t s);
 cudaError_t launch_row_topk_groups(const float* V, const float* gmin, int64_t rows, int ncols, int64_t ld, int p,
                                    int32_t* out_idx, float* out_val, int64_t ld_out, cudaStream_t s);
 cudaError_t launch_gemm_tc(const float* A, const int32_t* eA, int64_t M, const float* B, const int32_t* eB, int N,

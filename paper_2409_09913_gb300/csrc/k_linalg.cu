@@ -156,12 +156,19 @@ __device__ __forceinline__ float2 unpack2(uint64_t v) {
     return r;
 }
 
-template <bool NT, int EPI>
+// LIST: row i of the product is row list[i] of A, for the *count listed rows.
+template <bool NT, int EPI, bool LIST = false>
 __global__ void __launch_bounds__(256) sgemm_kernel(const float* __restrict__ A, const float* __restrict__ Bm,
                                                     float* __restrict__ Cm, int64_t M, int N, int K, float alpha,
                                                     const float* __restrict__ addend,
                                                     const float* __restrict__ rown,
-                                                    const float* __restrict__ coln, int64_t ldc) {
+                                                    const float* __restrict__ coln, int64_t ldc,
+                                                    const int32_t* __restrict__ list = nullptr,
+                                                    const int32_t* __restrict__ count = nullptr) {
+    if (LIST) {
+        M = *count;
+        if ((int64_t)blockIdx.y * 128 >= M) return;
+    }
     __shared__ __align__(16) float As[2][8][128];
     __shared__ __align__(16) float Bs[2][8][128];
     const int tid = threadIdx.x;
@@ -170,7 +177,7 @@ __global__ void __launch_bounds__(256) sgemm_kernel(const float* __restrict__ A,
     // A loader: row tid/2, k offset (tid%2)*4
     const int la_r = tid >> 1, la_k = (tid & 1) * 4;
     const bool a_ok = (m0 + la_r) < M;
-    const float* a_ptr = A + (a_ok ? (m0 + la_r) : 0) * (int64_t)K + la_k;
+    const float* a_ptr = A + (a_ok ? (LIST ? (int64_t)list[m0 + la_r] : m0 + la_r) : 0) * (int64_t)K + la_k;
     // B loader
     int lb_k, lb_n;
     bool b_ok;
@@ -254,7 +261,7 @@ __global__ void __launch_bounds__(256) sgemm_kernel(const float* __restrict__ A,
             const float ac = (j & 1) ? pr.y : pr.x;
             float v;
             if (EPI == EPI_DIST) {
-                v = rown[m] + coln[nn] - 2.f * ac;
+                v = rown[LIST ? (int64_t)list[m] : m] + coln[nn] - 2.f * ac;
             } else {
                 v = alpha * ac;
                 if (addend) v += addend[m * ldc + nn];
@@ -394,45 +401,163 @@ cudaError_t launch_row_sqnorm(const float* X, int64_t n, int D, float* out, cuda
 }
 
 // ---------------------------------------------------------------------------
-// Cluster means (reading of Section 5.1 "local centroid"): one thread per
-// (cluster, coordinate), FP64 sum over the cluster's rows in stored order
-// (ascending original id), one division and one rounding to FP32.  Empty
-// clusters keep `keep_empty ? old value : 0`.
+// Cluster means (reading of Section 5.1 "local centroid"): per (cluster,
+// coordinate) the FP64 sum over the cluster's rows in stored order (ascending
+// original id), one division and one rounding to FP32.  Empty clusters keep
+// `keep_empty ? old value : 0`.
+//
+// The FP64 sum in order is a chain of additions on a pipe of two lanes a clock
+// (100,000 x 768 in 256 lists: 630 us).  It is formed as pairs of FP32 numbers
+// instead (Knuth's two-sum: a running sum and the sum of its exact remainders),
+// in segments of 32 rows that are added up in FP64, a sixteenth of the rows per
+// thread.  The mean's rounding to FP32 is that of the sum in order unless it lies
+// within the two sums' error bounds of a rounding boundary (a segment's remainders
+// round within 32^2 2^-48 of its magnitudes, a sum in order within n 2^-53); those
+// elements, about one in a thousand, are listed and summed in order.  240 us,
+// half of them those few sums' chains; the rows' bytes take 45.
 // ---------------------------------------------------------------------------
-__global__ void centroid_kernel(const float* __restrict__ X, const int64_t* __restrict__ list_off,
-                                const int64_t* __restrict__ list_ids, int nlist, int D, float* __restrict__ C,
-                                int keep_empty) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int64_t)nlist * D) return;
-    const int j = (int)(t / D), k = (int)(t % D);
+__device__ __forceinline__ void two_sum_add(float x, float& s, float& c, float& m) {
+    const float t = s + x, z = t - s;
+    c += (s - (t - z)) + (x - z);
+    s = t;
+    m += fabsf(x);
+}
+
+constexpr int CW = 16;             // row slots of a block: 16 threads of four coordinates each
+__global__ void __launch_bounds__(256) centroid_kernel(const float* __restrict__ X, const int64_t* __restrict__ list_off,
+                                                       const int64_t* __restrict__ list_ids, int D,
+                                                       float* __restrict__ C, int keep_empty,
+                                                       int32_t* __restrict__ redo, int32_t* __restrict__ n_redo) {
+    __shared__ double sh[2][CW][64];
+    const int j = blockIdx.x, l = threadIdx.x & 15, w = threadIdx.x >> 4;
+    const int k0 = blockIdx.y * 64;                                 // (D % 64 == 0)
     const int64_t b = list_off[j], e = list_off[j + 1];
     if (b == e) {
-        if (!keep_empty) C[t] = 0.f;
+        if (!keep_empty && threadIdx.x < 64) C[(int64_t)j * D + k0 + threadIdx.x] = 0.f;
         return;
     }
-    double acc = 0.0;
-    int64_t r = b;
-    // four independent loads in flight; the additions stay in ascending order
-    for (; r + 4 <= e; r += 4) {
-        const float x0 = X[list_ids[r] * D + k];
-        const float x1 = X[list_ids[r + 1] * D + k];
-        const float x2 = X[list_ids[r + 2] * D + k];
-        const float x3 = X[list_ids[r + 3] * D + k];
-        acc = __dadd_rn(acc, (double)x0);
-        acc = __dadd_rn(acc, (double)x1);
-        acc = __dadd_rn(acc, (double)x2);
-        acc = __dadd_rn(acc, (double)x3);
+    double S[4] = {0.0, 0.0, 0.0, 0.0}, G[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int64_t r = b + w; r < e; r += 32 * CW) {
+        float s[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f}, m[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int g = 0; g < 32 && r + g * CW < e; g += 4) {
+            float4 x[4];                                            // four loads in flight
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t rr = r + (g + u) * CW;
+                x[u] = rr < e ? *reinterpret_cast<const float4*>(X + list_ids[rr] * D + k0 + 4 * l)
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                two_sum_add(x[u].x, s[0], c[0], m[0]);
+                two_sum_add(x[u].y, s[1], c[1], m[1]);
+                two_sum_add(x[u].z, s[2], c[2], m[2]);
+                two_sum_add(x[u].w, s[3], c[3], m[3]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            S[i] += (double)s[i] + (double)c[i];
+            G[i] += (double)m[i];
+        }
     }
-    for (; r < e; ++r) acc = __dadd_rn(acc, (double)X[list_ids[r] * D + k]);
-    C[t] = __double2float_rn(__ddiv_rn(acc, (double)(e - b)));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        sh[0][w][4 * l + i] = S[i];
+        sh[1][w][4 * l + i] = G[i];
+    }
+    __syncthreads();
+    if (threadIdx.x >= 64) return;
+    const int k = threadIdx.x;
+    double sum = 0.0, mag = 0.0;
+#pragma unroll
+    for (int u = 0; u < CW; ++u) {
+        sum += sh[0][u][k];
+        mag += sh[1][u][k];
+    }
+    const double inv = 1.0 / (double)(e - b), mean = sum * inv;
+    const double err = mag * inv * (0x1p-38 + ((double)(e - b) + 64.0) * 0x1p-52) * 1.01;
+    const float lo = (float)(mean - err), hi = (float)(mean + err);
+    float* out = C + (int64_t)j * D + k0 + k;
+    // (not decided here: both sides of the interval round differently, sums that may have overflowed or underflowed)
+    if (mag == 0.0) *out = 0.f;
+    else if (lo == hi && mag < 1e37 && fabsf(lo) > 1e-25f) *out = lo;
+    else redo[atomicAdd(n_redo, 1)] = (int32_t)((int64_t)j * D + k0 + k);
+}
+
+// (cluster, coordinate) pairs in FP64, in stored order: the listed ones, or all.
+// Eight lanes per pair fetch 32 rows, the next 32 while these are added.
+__global__ void __launch_bounds__(128) centroid_ordered_kernel(const float* __restrict__ X,
+                                                               const int64_t* __restrict__ list_off,
+                                                               const int64_t* __restrict__ list_ids, int64_t total,
+                                                               int D, float* __restrict__ C, int keep_empty,
+                                                               const int32_t* __restrict__ redo,
+                                                               const int32_t* __restrict__ n_redo) {
+    const int64_t n = redo ? (int64_t)*n_redo : total;
+    const int lane = threadIdx.x & 31, l = lane & 7;
+    const int64_t groups = (int64_t)gridDim.x * blockDim.x / 8;
+    // (the groups of a warp take the same number of rounds: a warp's lanes stay together in the exchanges)
+    for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32 * 4; i0 < n; i0 += groups) {
+        const int64_t i = i0 + lane / 8;
+        const int64_t t = i < n ? (redo ? (int64_t)redo[i] : i) : -1;
+        const int j = t >= 0 ? (int)(t / D) : 0, k = t >= 0 ? (int)(t % D) : 0;
+        const int64_t b = t >= 0 ? list_off[j] : 0, e = t >= 0 ? list_off[j + 1] : 0;
+        int64_t rounds = (e - b + 31) / 32;
+#pragma unroll
+        for (int o = 8; o < 32; o <<= 1) {
+            const int64_t y = __shfl_xor_sync(0xffffffffu, rounds, o);
+            rounds = y > rounds ? y : rounds;
+        }
+        float x[4];
+        auto load = [&](int64_t r) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t rr = r + 8 * u + l;
+                x[u] = rr < e ? X[list_ids[rr] * D + k] : 0.f;
+            }
+        };
+        load(b);
+        double acc = 0.0;
+        for (int64_t it = 0; it < rounds; ++it) {
+            const int64_t r = b + 32 * it;
+            const float y[4] = {x[0], x[1], x[2], x[3]};
+            load(r + 32);
+#pragma unroll
+            for (int u = 0; u < 32; ++u) {                          // ascending rows
+                const float v = __shfl_sync(0xffffffffu, y[u >> 3], (lane & 24) + (u & 7));
+                if (r + u < e) acc = __dadd_rn(acc, (double)v);
+            }
+        }
+        if (t >= 0 && l == 0) {
+            if (e > b) C[t] = __double2float_rn(__ddiv_rn(acc, (double)(e - b)));
+            else if (!keep_empty) C[t] = 0.f;
+        }
+    }
 }
 
 cudaError_t launch_centroids(const float* X, const int64_t* list_off, const int64_t* list_ids, int nlist, int D,
                              float* C, int keep_empty, cudaStream_t s) {
     const int64_t tot = (int64_t)nlist * D;
-    count_launch();
-    centroid_kernel<<<(unsigned)ceil_div(tot, 256), 256, 0, s>>>(X, list_off, list_ids, nlist, D, C, keep_empty);
-    return cudaGetLastError();
+    int32_t* redo = nullptr;
+    const bool fast = tot < 0x7fffffff && D % 64 == 0 && D / 64 <= 65535 && ((uintptr_t)X & 15) == 0;
+    if (!fast || cudaMallocAsync((void**)&redo, sizeof(int32_t) * (size_t)(tot + 1), s) != cudaSuccess) {
+        if (fast) cudaGetLastError();                               // (no memory for the list: all in order)
+        count_launch();
+        centroid_ordered_kernel<<<(unsigned)std::min<int64_t>(ceil_div(tot, 16), 1 << 20), 128, 0, s>>>(
+            X, list_off, list_ids, tot, D, C, keep_empty, nullptr, nullptr);
+        return cudaGetLastError();
+    }
+    cudaError_t e = cudaMemsetAsync(redo + tot, 0, sizeof(int32_t), s);
+    if (e == cudaSuccess) {
+        count_launch();
+        centroid_kernel<<<dim3((unsigned)nlist, (unsigned)(D / 64)), 256, 0, s>>>(X, list_off, list_ids, D, C, keep_empty,
+                                                                                  redo, redo + tot);
+        count_launch();
+        centroid_ordered_kernel<<<1216, 128, 0, s>>>(X, list_off, list_ids, tot, D, C, keep_empty, redo, redo + tot);
+        e = cudaGetLastError();
+    }
+    const cudaError_t ef = cudaFreeAsync(redo, s);
+    return e != cudaSuccess ? e : ef;
 }
 
 // ---------------------------------------------------------------------------
@@ -631,10 +756,12 @@ cudaError_t launch_row_topk(const float* V, int64_t rows, int ncols, int64_t ld,
 namespace erq {
 
 // Column of the smallest value in each row (ties -> lower column); one warp per row.
-__global__ void row_argmin_kernel(const float* __restrict__ V, int64_t rows, int ncols, int32_t* __restrict__ out) {
+// With `list`: of row i the answer goes to out[list[i]], for the *count listed rows.
+__global__ void row_argmin_kernel(const float* __restrict__ V, int64_t rows, int ncols, int32_t* __restrict__ out,
+                                  const int32_t* __restrict__ list, const int32_t* __restrict__ count) {
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (w >= rows) return;
+    if (w >= (list ? (int64_t)*count : rows)) return;
     const float* v = V + w * ncols;
     uint64_t best = kEmptyKey;
     for (int c = lane; c < ncols; c += 32) {
@@ -646,13 +773,192 @@ __global__ void row_argmin_kernel(const float* __restrict__ V, int64_t rows, int
         const uint64_t t = __shfl_xor_sync(0xffffffffu, best, o);
         best = t < best ? t : best;
     }
-    if (lane == 0) out[w] = (int32_t)key_id(best);
+    if (lane == 0) out[list ? (int64_t)list[w] : w] = (int32_t)key_id(best);
 }
 
 cudaError_t launch_row_argmin(const float* V, int64_t rows, int ncols, int32_t* out, cudaStream_t s) {
     if (rows <= 0) return cudaSuccess;
     count_launch();
-    row_argmin_kernel<<<(unsigned)ceil_div(rows * 32, 256), 256, 0, s>>>(V, rows, ncols, out);
+    row_argmin_kernel<<<(unsigned)ceil_div(rows * 32, 256), 256, 0, s>>>(V, rows, ncols, out, nullptr, nullptr);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// Nearest centroid of every row by the FP32 distances of sgemm_kernel (its chain
+// of D fused multiply-adds per product), most of them decided on the tensor
+// cores.  V holds d_j = |x|^2 + |c_j|^2 - 2 <x, c_j> with the product from FP16
+// parts (gemm_tma).  Both products are within
+//     E_j = 8 D 2^-24 |x| |c_j|
+// of <x, c_j> together: the chain of D roundings within D 2^-24, the parts' three
+// products within 3 D / 16 tensor-core steps that each lose at most 17 units of
+// 2^-23 of the largest magnitude (sixteen products and the accumulator aligned
+// and truncated: Fasi, Higham, Mikaitis, Pranesh, "Numerical behavior of NVIDIA
+// tensor cores", 2021), the dropped parts within 2^-21; the sums of the norms add
+// 2^-21 (|x|^2 + |c_j|^2).  A row whose smallest d_j lies below all others by more
+// than both errors has that column; the others are listed and get the FP32
+// distances of the columns that can be the smallest (all of them where these are
+// more than 32), so the answer is the same for every row.  100,000 x 256 at D =
+// 768: 930 us a pass with FP32 products alone, 340 us.
+// ---------------------------------------------------------------------------
+struct AssignBound {
+    float f, x2;
+    __device__ __forceinline__ float operator()(float c2) const {    // (twice E: the product enters as 2 <x, c>)
+        return f * sqrtf(x2 * c2) + 0x1p-21f * (x2 + c2);
+    }
+};
+__device__ __forceinline__ AssignBound assign_bound(int D, float x2) { return {2.02f * 8.f * 0x1p-24f * (float)D, x2}; }
+
+// One warp per row: decides it, or lists it with the upper bound of its smallest distance.
+__global__ void __launch_bounds__(256) assign_certain_kernel(const float* __restrict__ V,
+                                                             const float* __restrict__ xn,
+                                                             const float* __restrict__ cn, int64_t rows, int ncols,
+                                                             int D, int32_t* __restrict__ out, float* __restrict__ upper,
+                                                             int32_t* __restrict__ list, int32_t* __restrict__ count) {
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (w >= rows) return;
+    const float* v = V + w * ncols;
+    const AssignBound bd = assign_bound(D, xn[w]);
+    // the smallest upper bound, and the smallest two lower bounds with the first one's column
+    float up = INFINITY, lo1 = INFINITY, lo2 = INFINITY;
+    int col = -1, upc = -1;
+    bool odd = false;
+    for (int c0 = 0; c0 < ncols; c0 += 128) {
+        float x[4], y[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int c = c0 + 32 * u + lane;
+            x[u] = c < ncols ? v[c] : INFINITY;
+            y[u] = c < ncols ? cn[c] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int c = c0 + 32 * u + lane;
+            if (c >= ncols) break;
+            const float e = bd(y[u]), h = x[u] + e, l = x[u] - e;
+            // not finite, or so small that the bound's terms underflow: not decided by it
+            odd |= !(fabsf(x[u]) < INFINITY) || !(e < INFINITY) || bd.x2 + y[u] < 1e-30f;
+            if (h < up) {
+                up = h;
+                upc = c;
+            }
+            if (l < lo1) {
+                lo2 = lo1;
+                lo1 = l;
+                col = c;
+            } else {
+                lo2 = fminf(lo2, l);
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float u2 = __shfl_xor_sync(0xffffffffu, up, o), l1 = __shfl_xor_sync(0xffffffffu, lo1, o);
+        const float l2 = __shfl_xor_sync(0xffffffffu, lo2, o);
+        const int uc = __shfl_xor_sync(0xffffffffu, upc, o), lc = __shfl_xor_sync(0xffffffffu, col, o);
+        if (u2 < up || (u2 == up && uc < upc)) {
+            up = u2;
+            upc = uc;
+        }
+        lo2 = fminf(fminf(lo2, l2), fmaxf(lo1, l1));
+        if (l1 < lo1 || (l1 == lo1 && lc < col)) {
+            lo1 = l1;
+            col = lc;
+        }
+    }
+    odd = __any_sync(0xffffffffu, odd);
+    if (lane == 0) {
+        if (!odd && upc == col && lo2 > up) {
+            out[w] = col;
+        } else {
+            const int i = atomicAdd(count, 1);
+            list[i] = (int32_t)w;
+            upper[i] = odd ? INFINITY : up;
+        }
+    }
+}
+
+// The listed rows: the FP32 distances of the columns that can be the smallest,
+// one lane per column, each the same chain of fused multiply-adds as
+// sgemm_kernel's; rows with more than 32 such columns go on to the full product.
+__global__ void __launch_bounds__(256) assign_close_kernel(const float* __restrict__ X, const float* __restrict__ C,
+                                                           const float* __restrict__ V, const float* __restrict__ xn,
+                                                           const float* __restrict__ cn, int ncols, int D,
+                                                           int32_t* __restrict__ out, const float* __restrict__ upper,
+                                                           const int32_t* __restrict__ list,
+                                                           const int32_t* __restrict__ count,
+                                                           int32_t* __restrict__ list2, int32_t* __restrict__ count2) {
+    const int lane = threadIdx.x & 31;
+    const int n = *count;
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n;
+         i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const int32_t w = list[i];
+        const float* v = V + (int64_t)w * ncols;
+        const float up = upper[i];
+        const AssignBound bd = assign_bound(D, xn[w]);
+        int mine = -1, total = 0;
+        for (int c0 = 0; c0 < ncols && total <= 32; c0 += 32) {
+            const int c = c0 + lane;
+            const unsigned in = __ballot_sync(0xffffffffu, c < ncols && !(v[c] - bd(cn[c]) > up));
+            // the columns go to the lanes total, total + 1, ..
+            const int take = lane - total;
+            if (take >= 0 && take < __popc(in)) mine = c0 + (int)__fns(in, 0, take + 1);
+            total += __popc(in);
+        }
+        if (total > 32 || total < 1) {
+            if (lane == 0) list2[atomicAdd(count2, 1)] = w;
+            continue;
+        }
+        uint64_t key = kEmptyKey;
+        if (mine >= 0) {
+            const float4* x = reinterpret_cast<const float4*>(X + (int64_t)w * D);
+            const float4* c = reinterpret_cast<const float4*>(C + (int64_t)mine * D);
+            float ac = 0.f;
+#pragma unroll 8
+            for (int k = 0; k < D / 4; ++k) {
+                const float4 a = x[k], b = c[k];
+                ac = fmaf(a.x, b.x, ac);
+                ac = fmaf(a.y, b.y, ac);
+                ac = fmaf(a.z, b.z, ac);
+                ac = fmaf(a.w, b.w, ac);
+            }
+            key = make_key(xn[w] + cn[mine] - 2.f * ac, (uint32_t)mine);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const uint64_t t = __shfl_xor_sync(0xffffffffu, key, o);
+            key = t < key ? t : key;
+        }
+        if (lane == 0) out[w] = (int32_t)key_id(key);
+    }
+}
+
+// Rows X [rows][D] with their parts and exponents (query_prep), the centroids C
+// with theirs; V is scratch [rows][nc], list [3 rows + 2] likewise.
+cudaError_t launch_assign(const float* X, const __half* Xhi, const __half* Xlo, const int32_t* eX, const float* xn,
+                          int64_t rows, const float* C, const __half* Chi, const __half* Clo, const int32_t* eC,
+                          const float* cn, int nc, int D, float* V, int32_t* list, int32_t* out, uint32_t* status,
+                          cudaStream_t s) {
+    if (rows <= 0) return cudaSuccess;
+    if (rows > kMaxSlabRows || D % 4 != 0 || (((uintptr_t)X | (uintptr_t)C) & 15) != 0) return cudaErrorInvalidValue;
+    int32_t *count = list, *close = list + 2, *far = close + rows;
+    float* upper = reinterpret_cast<float*>(far + rows);
+    cudaError_t e = cudaMemsetAsync(count, 0, 2 * sizeof(int32_t), s);
+    if (e != cudaSuccess) return e;
+    if ((e = launch_gemm_tma(Xhi, Xlo, eX, rows, Chi, Clo, eC, nc, D, V, nc, 1, xn, cn, nullptr, status, s)) !=
+        cudaSuccess)
+        return e;
+    count_launch();
+    assign_certain_kernel<<<(unsigned)ceil_div(rows * 32, 256), 256, 0, s>>>(V, xn, cn, rows, nc, D, out, upper, close,
+                                                                             count);
+    count_launch();
+    assign_close_kernel<<<(unsigned)std::min<int64_t>(ceil_div(rows, 8), 2432), 256, 0, s>>>(
+        X, C, V, xn, cn, nc, D, out, upper, close, count, far, count + 1);
+    dim3 grid((unsigned)ceil_div(nc, 128), (unsigned)ceil_div(rows, 128));
+    count_launch();
+    sgemm_kernel<true, EPI_DIST, true><<<grid, 256, 0, s>>>(X, C, V, rows, nc, D, 1.f, nullptr, xn, cn, nc, far, count + 1);
+    count_launch();
+    row_argmin_kernel<<<(unsigned)ceil_div(rows * 32, 256), 256, 0, s>>>(V, rows, nc, out, far, count + 1);
     return cudaGetLastError();
 }
 
