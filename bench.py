@@ -527,7 +527,10 @@ def roofline(args, cfg, R, best, nq):
     flops = 2.0 * D * R["work"]["pairs"]
     bytes_alg = (B * D / 8 + 8) * R["work"]["rows"] + nq * D * 4
     sm_mhz = R["clocks"]["sm_mhz"] or 2070.0
-    if best == "fp32":
+    tc = best != "fp32" or max(args.k, args.rerank_k) <= 128      # (FP32 precision: two FP16 query parts up to k' = 128)
+    if best == "fp32" and tc:
+        peak_c, unit_c, bound_c = peaks["bf16_tflops"] / 2.0, "TFLOP/s", "tensor"
+    elif best == "fp32":
         peak_c, unit_c, bound_c = ffma_peak_tflops(sm_mhz), "TFLOP/s", "alu"
     else:
         peak_c = peaks["bf16_tflops"] * (2.0 if best == "fp8" else 1.0)
@@ -546,9 +549,10 @@ def roofline(args, cfg, R, best, nq):
                                                              R["work"].get("items"))
     roof["bytes_alg_per_launch"] = bytes_alg
     roof["flops_per_launch"] = flops
-    roof["kernel"] = "scan_fp32_kernel" if best == "fp32" else "scan_tc_kernel"
+    roof["kernel"] = "scan_tc_kernel" if tc else "scan_fp32_kernel"
     roof["peak_source"] = (peaks["source"] + (" (bf16 x 2 for e4m3)" if best == "fp8" and roof["bound"] == "tensor"
-                                              else "")) if bound_c != "alu" or roof["bound"] == "hbm" else \
+                                              else " (bf16 / 2 for two query parts)" if best == "fp32" and
+                                              roof["bound"] == "tensor" else "")) if bound_c != "alu" or roof["bound"] == "hbm" else \
         f"152 SMs x 128 FFMA x 2 at {sm_mhz:.0f} MHz"
     return roof
 

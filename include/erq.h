@@ -51,7 +51,10 @@ typedef enum {
 
 /* Arithmetic of the code-by-query contraction in erq_search. */
 typedef enum {
-    ERQ_PREC_FP32 = 0,       /* CUDA-core FP32 FFMA scan (reference GPU path)           */
+    ERQ_PREC_FP32 = 0,       /* FP32: codes exact, rotated query as two FP16 parts that
+                                hold it to 2^-23, tcgen05 kind::f16 with FP32
+                                accumulation, up to max(k, rerank_k) = 128; CUDA-core
+                                FP32 FFMA scan above                                     */
     ERQ_PREC_FP16 = 1,       /* tcgen05 kind::f16: codes exact, rotated query in FP16,
                                 FP32 accumulation in tensor memory                       */
     ERQ_PREC_FP8 = 2,        /* tcgen05 kind::f8f6f4: query rounded to e4m3 after a
@@ -295,7 +298,8 @@ erq_status erq_index_load(const char* path, void* stream, erq_index** out);
  * erq_search_timing: device time in milliseconds of the phases of the last
  * erq_search on this index that ran with ERQ_SEARCH_TIMING, measured with CUDA
  * events on the search stream: ms[0] query rotation, ms[1] centroid probe,
- * ms[2] planning (probe inversion, pair scalars, one host read-back),
+ * ms[2] planning (probe inversion, pair scalars; a host read-back unless the
+ * sizes are bounded on the host),
  * ms[3] code scan (estimator + per-item top-k'), ms[4] merge, ms[5] re-rank.
  * Synchronises those events.  n must be >= 6.  Errors: EINVAL (no timed search).
  * erq_kernel_launches: number of kernels this library has launched in the
@@ -305,7 +309,7 @@ erq_status erq_index_load(const char* path, void* stream, erq_index** out);
  * that had to be read at least once), out[2] work items, out[3] per-(query,
  * item) candidate lists, and for the tensor-core scan out[4] 128-row blocks
  * streamed through the tensor cores and out[5] the sum over those blocks of the
- * item's query count padded to the MMA width (0 for the FP32 path).  Fills
+ * item's query count padded to the MMA width (0 for FP32 precision).  Fills
  * min(n, 6) entries; n must be >= 4.  Synchronises the device. */
 erq_status erq_search_timing(const erq_index* index, float* ms, int32_t n);
 /* erq_search_timing_total: per-phase device milliseconds summed over the timed
