@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(512) dqc_kernel(const float* __restrict__ Q, c
 // per cluster in order of decreasing size (item_first), the pair writes its own
 // query slots of its cluster's items (plan_fill), so no query list is sorted or
 // scattered in between.  16,384 queries x 256 slots over 4,096 lists: 0.40 ms in
-// eight launches before, 0.17 ms in four now.  Up to kSmallPairs pairs run all of it in
+// eight launches before, 0.15 ms in four now.  Up to kSmallPairs pairs run all of it in
 // one block (plan_small_kernel), which is bound by the latency of its five
 // phases instead of by launches.
 // ---------------------------------------------------------------------------
@@ -607,8 +607,15 @@ static int fp32_blocks_per_sm(int kp) {
 int scan_fp32_blocks_per_sm(int kp, int B) { return B > 8 ? fp32_blocks_per_sm<2>(kp) : fp32_blocks_per_sm<1>(kp); }
 
 // ---------------------------------------------------------------------------
-// Merge: per query the k' smallest keys over its lists, ascending.
-// Block of 256 threads; running best k' + a chunk, block bitonic sort.
+// Merge for k' > 32: per query the k' smallest keys over its lists, ascending, by
+// one block.  Keys above the query's published threshold (tq, optional: never
+// below its k'-th key) do not count.  Where the others fit the sort buffer they
+// are sorted; where they do not, one pass counts their values in 2,048 equal
+// intervals of their range and only the keys up to the interval of the k'-th are
+// sorted; where even these do not fit (many equal values), a running best k' and
+// a chunk at a time are.  Bound by the latency of the passes over the lists, a
+// warp per list: 100 queries x 79 lists, k' = 100, 79 us with the chunks alone,
+// 20 us.  1,024 threads while every query can have half an SM, else 256.
 // ---------------------------------------------------------------------------
 __device__ void block_bitonic_u64(uint64_t* v, int n) {
     for (int size = 2; size <= n; size <<= 1)
@@ -624,16 +631,98 @@ __device__ void block_bitonic_u64(uint64_t* v, int n) {
         }
 }
 
-__global__ void __launch_bounds__(256) merge_kernel(const uint64_t* __restrict__ inter,
-                                                    const int32_t* __restrict__ inter_cnt,
-                                                    const int64_t* __restrict__ qbase, int kp, int lstride,
-                                                    int sortn, uint64_t* __restrict__ cand, DevChecks ck) {
+__global__ void __launch_bounds__(1024) merge_kernel(const uint64_t* __restrict__ inter,
+                                                     const int32_t* __restrict__ inter_cnt,
+                                                     const int64_t* __restrict__ qbase, int kp, int lstride,
+                                                     int sortn, const unsigned long long* __restrict__ tq,
+                                                     uint64_t* __restrict__ cand, DevChecks ck) {
     extern __shared__ uint64_t buf[];  // [sortn]
+    constexpr int BINS = 2048;
+    __shared__ int hist[BINS];
+    __shared__ uint32_t s_lo[32], s_hi[32];
+    __shared__ int s_n[32];
+    __shared__ int s_bin, s_end;
     __shared__ int s_fill;
     __shared__ uint64_t s_tau;         // entries >= s_tau cannot enter the top k'
     const int64_t q = blockIdx.x;
     const int64_t L0 = qbase[q], L1 = qbase[q + 1];
-    for (int i = threadIdx.x; i < sortn; i += blockDim.x) buf[i] = kEmptyKey;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const uint64_t top = tq ? (uint64_t)tq[q] : kEmptyKey;
+    // every key that counts: a warp per list, the block for long lists
+    auto each = [&](auto f) {
+        const bool wide = lstride > 512;
+        for (int64_t L = L0 + (wide ? 0 : warp); L < L1; L += wide ? 1 : nw) {
+            if (!ERQ_DCHECK(L >= 0 && L < ck.lists, ck.status, 0)) break;
+            int n = inter_cnt[L];
+            if (!ERQ_DCHECK(n >= 0 && n <= lstride, ck.status, 0)) n = 0;
+            for (int j = wide ? tid : lane; j < n; j += wide ? blockDim.x : 32) {
+                const uint64_t key = inter[L * lstride + j];
+                if (key <= top && key != kEmptyKey) f(key);
+            }
+        }
+    };
+    for (int i = tid; i < sortn; i += blockDim.x) buf[i] = kEmptyKey;
+    for (int i = tid; i < BINS; i += blockDim.x) hist[i] = 0;
+    if (tid == 0) s_fill = 0;
+    uint32_t lo = 0xffffffffu, hi = 0u;
+    int cnt = 0;
+    each([&](uint64_t key) {
+        lo = min(lo, (uint32_t)(key >> 32));
+        hi = max(hi, (uint32_t)(key >> 32));
+        ++cnt;
+    });
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0) {
+        s_lo[warp] = lo;
+        s_hi[warp] = hi;
+        s_n[warp] = cnt;
+    }
+    __syncthreads();
+    int total = 0;
+    for (int w = 0; w < nw; ++w) {
+        lo = min(lo, s_lo[w]);
+        hi = max(hi, s_hi[w]);
+        total += s_n[w];
+    }
+    int take = total, bin = BINS - 1;
+    const int shift = hi > lo ? max(0, 21 - __clz(hi - lo)) : 0;   // (hi - lo) >> shift < 2048
+    if (total > sortn) {
+        each([&](uint64_t key) { atomicAdd(&hist[((uint32_t)(key >> 32) - lo) >> shift], 1); });
+        __syncthreads();
+        const int per = BINS / blockDim.x;
+        int own = 0;
+        for (int i = 0; i < per; ++i) own += hist[tid * per + i];
+        const int inc = warp_incl_scan(own);
+        if (lane == 31) s_n[warp] = inc;                           // (read above before the barrier)
+        __syncthreads();
+        int run = inc - own;
+        for (int w = 0; w < warp; ++w) run += s_n[w];
+        for (int i = 0; i < per; ++i) {
+            const int c = hist[tid * per + i];
+            if (run < kp && run + c >= kp) {
+                s_bin = tid * per + i;
+                s_end = run + c;
+            }
+            run += c;
+        }
+        __syncthreads();
+        bin = s_bin;
+        take = s_end;
+    }
+    if (take <= sortn) {
+        each([&](uint64_t key) {
+            if ((int)(((uint32_t)(key >> 32) - lo) >> shift) <= bin) buf[atomicAdd(&s_fill, 1)] = key;
+        });
+        __syncthreads();
+        int n = 2;
+        while (n < take || n < kp) n <<= 1;
+        block_bitonic_u64(buf, n);
+        for (int j = tid; j < kp; j += blockDim.x) cand[q * kp + j] = buf[j];
+        return;
+    }
+    __syncthreads();
     if (threadIdx.x == 0) { s_fill = kp; s_tau = kEmptyKey; }
     __syncthreads();
     for (int64_t L = L0; L < L1; ++L) {
@@ -1214,7 +1303,7 @@ cudaError_t launch_merge(const uint64_t* inter, const int32_t* inter_cnt, const 
     cudaError_t e = cudaFuncSetAttribute(merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sortn * 8);
     if (e != cudaSuccess) return e;
     count_launch();
-    merge_kernel<<<(unsigned)nq, 256, sortn * 8, s>>>(inter, inter_cnt, qbase, kp, lstride, sortn, cand, ck);
+    merge_kernel<<<(unsigned)nq, nq <= 304 ? 1024 : 256, sortn * 8, s>>>(inter, inter_cnt, qbase, kp, lstride, sortn, tq, cand, ck);
     return cudaGetLastError();
 }
 
