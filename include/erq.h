@@ -51,10 +51,11 @@ typedef enum {
 
 /* Arithmetic of the code-by-query contraction in erq_search. */
 typedef enum {
-    ERQ_PREC_FP32 = 0,       /* FP32: codes exact, rotated query as two FP16 parts that
-                                hold it to 2^-23, tcgen05 kind::f16 with FP32
-                                accumulation, up to max(k, rerank_k) = 128; CUDA-core
-                                FP32 FFMA scan above                                     */
+    ERQ_PREC_FP32 = 0,       /* FP32: codes exact, rotated query as whole numbers and
+                                FP16 remainders with an FP32 accumulator each (tcgen05
+                                kind::f16; the sum's error is no larger than that of
+                                FP32 multiply-adds), up to max(k, rerank_k) = 128;
+                                CUDA-core FP32 FFMA scan above                           */
     ERQ_PREC_FP16 = 1,       /* tcgen05 kind::f16: codes exact, rotated query in FP16,
                                 FP32 accumulation in tensor memory                       */
     ERQ_PREC_FP8 = 2,        /* tcgen05 kind::f8f6f4: query rounded to e4m3 after a

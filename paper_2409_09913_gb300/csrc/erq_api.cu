@@ -844,7 +844,7 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
     }
     if (prec == ERQ_PREC_FP32 && tcp && !ts) {
         // q' in two FP16 parts (over the parts of q, which the probe has read)
-        if ((e = launch_query_prep(Qrot, nq, D, eQ, nullptr, (__half*)sl[18], (__half*)sl[19], s, (float*)sl[22])) !=
+        if ((e = launch_query_parts(Qrot, nq, D, ix->B, (__half*)sl[18], (__half*)sl[19], (float*)sl[22], s)) !=
             cudaSuccess)
             return cuda_fail(e, "rotated query split");
     }

@@ -44,8 +44,8 @@ constexpr int64_t kSmallPairs = 2048;   // pairs that plan_small_kernel takes
 
 struct ScanLaunch {
     const float* Qrot;
-    const void* Qh;             // FP16 rotated queries (tensor-core path; FP32 precision: their high parts)
-    const void* Ql;             // FP32 precision: low parts (scaled by 1 / qscale, as Qh then is)
+    const void* Qh;             // FP16 rotated queries (tensor-core path; FP32 precision: their whole-number parts)
+    const void* Ql;             // FP32 precision: remainders (scaled by 1 / qscale, as Qh then is)
     const void* Q8;             // e4m3 rotated queries, rows of Dq bytes (kind::f8f6f4 path)
     const float* qscale;        // per-query power-of-two scales of Q8, or of Qh + Ql
     int64_t Dq;
@@ -135,6 +135,8 @@ bool scan_tc_shape_ok(int qn, int kp);
 cudaError_t launch_scan_layout(const uint8_t* codes, const float* g, const float* f_res, const int64_t* ids,
                                const int64_t* list_off, const int64_t* poff, int nlist, int64_t Np, int D, int B,
                                uint64_t* codes_p, float4* rowmeta, cudaStream_t s);
+cudaError_t launch_query_parts(const float* x, int64_t n, int D, int B, __half* hi, __half* lo, float* scale,
+                               cudaStream_t s);
 cudaError_t launch_quant_e4m3(const float* x, int64_t n, int D, int Dq, int dup, unsigned char* y, float* scale,
                               cudaStream_t s);
 cudaError_t launch_rerank(const uint64_t* cand, int64_t nq, int kp, const float* X, const float* Q, int D, int k,

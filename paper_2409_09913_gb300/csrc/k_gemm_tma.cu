@@ -340,8 +340,7 @@ __global__ void split_hilo_kernel(const float* __restrict__ X, const int32_t* __
 // operations, so the same bits, with the row read twice (the second time from
 // cache) instead of three times by three launches.
 __global__ void query_prep_kernel(const float* __restrict__ X, int64_t M, int K, int32_t* __restrict__ e,
-                                  float* __restrict__ sqn, __half* __restrict__ hi, __half* __restrict__ lo,
-                                  float* __restrict__ scale) {
+                                  float* __restrict__ sqn, __half* __restrict__ hi, __half* __restrict__ lo) {
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (w >= M) return;
@@ -366,7 +365,6 @@ __global__ void query_prep_kernel(const float* __restrict__ X, int64_t M, int K,
     if (lane == 0) {
         e[w] = ex;
         if (sqn) sqn[w] = ss;
-        if (scale) scale[w] = __int_as_float((127 + ex) << 23);   // 2^e
     }
     const float s = __int_as_float((127 - ex) << 23);          // 2^-e
     const int per = K / 8;
@@ -390,11 +388,11 @@ __global__ void query_prep_kernel(const float* __restrict__ X, int64_t M, int K,
 }
 
 cudaError_t launch_query_prep(const float* X, int64_t M, int K, int32_t* e, float* sqn, __half* hi, __half* lo,
-                              cudaStream_t s, float* scale) {
+                              cudaStream_t s) {
     if (M <= 0) return cudaSuccess;
     if (K % 8 != 0) return cudaErrorInvalidValue;
     count_launch();
-    query_prep_kernel<<<(unsigned)ceil_div(M * 32, 256), 256, 0, s>>>(X, M, K, e, sqn, hi, lo, scale);
+    query_prep_kernel<<<(unsigned)ceil_div(M * 32, 256), 256, 0, s>>>(X, M, K, e, sqn, hi, lo);
     return cudaGetLastError();
 }
 

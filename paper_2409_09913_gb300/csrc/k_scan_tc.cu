@@ -121,7 +121,8 @@ struct Cfg {
     static constexpr int AS = AS_;
     static constexpr bool EX = EX_;
     static constexpr int ACOL = TMEM_COLS - AS * (KB / 2);   // first TMEM column of the code slots
-    static constexpr int NACC = ACOL / QN;           // accumulators
+    static constexpr int DCOL = QB == 256 ? 2 * QN : QN;     // columns of an accumulator (two query parts: one sum each)
+    static constexpr int NACC = ACOL / DCOL;         // accumulators
     static_assert(AS % NSET == 0, "a set owns whole slots");
     static constexpr int RAW_BYTES = RAWK_ * 1024;
     static constexpr int TILE_Q = QN * QB;           // one stage's query tile
@@ -170,11 +171,11 @@ struct Cfg {
 using CfgA = Cfg<64, 160, 96, 6, 128, 48, 8>;    // k' <= 32, up to 64 queries per item
 using CfgW = Cfg<128, 96, 88, 4, 128, 40, 4>;    // k' <= 32, up to 128 queries per item
 using CfgB = Cfg<32, 256, 160, 6, 128, 48, 8>;   // k' <= 128, up to 32 queries per item
-using CfgA32 = Cfg<64, 160, 96, 4, 256, 48, 8>;  // the same with two query parts (FP32 precision)
+using CfgA32 = Cfg<64, 160, 96, 4, 256, 48, 4>;  // the same with two query parts (FP32 precision)
 using CfgB32 = Cfg<32, 256, 160, 6, 256, 48, 8>;
 using CfgAx = Cfg<64, 160, 96, 6, 128, 48, 8, true>;   // KMIN < k' <= 32
 using CfgWx = Cfg<128, 96, 88, 4, 128, 40, 4, true>;
-using CfgA32x = Cfg<64, 160, 96, 4, 256, 48, 8, true>;
+using CfgA32x = Cfg<64, 160, 96, 4, 256, 48, 4, true>;
 constexpr int KMIN = 24;
 
 // arrivals that complete a phase of the item-release barrier: one per warp of
@@ -536,10 +537,14 @@ __device__ __forceinline__ bool append_candidate(unsigned char* sm, const int4* 
 // in the same 128 bytes per row of tensor memory and query tile as 64 FP16
 // coordinates; 2 the split e4m3 form of B = 5..8 codes (unpack_split), a
 // stage covering 64 coordinates whose query tile holds them twice; 3 FP16 codes
-// and queries as two FP16 parts (FP32 precision): with a per-query power of two
-// that puts the largest coordinate in [2^13, 2^14), hi = RN16(x) and lo =
-// RN16(x - hi) hold x to 2^-23, the codes are exact, and both products add in
-// the same FP32 accumulator.  Its query tile is the hi rows, then the lo rows.
+// and queries as two FP16 parts (FP32 precision, query_parts_kernel): whole
+// numbers of at most 2^11 and the FP16 remainders.  Each part has its own FP32
+// accumulator.  The tensor core cuts a sum off at every step, so one accumulator
+// for both would lose half a unit of its last bit 2 D / 16 times over, in one
+// direction (2.3 times the error of round-to-nearest multiply-adds in the whole
+// estimate at D = 1536, B = 9); sums of whole numbers below 2^24 lose nothing, and
+// what the remainders' sum loses is 2^-12 of that.  The query tile is the whole
+// numbers' rows, then the remainders'.
 template <class C, int P>
 __global__ void __launch_bounds__(THREADS, 1)
     scan_tc_kernel(const __grid_constant__ CUtensorMap codes_map, const __grid_constant__ CUtensorMap codes_map1,
@@ -894,7 +899,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                             break;
                         }
                         tc_fence_after();
-                        const uint32_t ta = tmem + ACOL + as * (KB / 2), dt = tmem + buf * QN;
+                        const uint32_t ta = tmem + ACOL + as * (KB / 2), dt = tmem + buf * C::DCOL;
                         if (elect_one()) {
 #pragma unroll
                             for (int k = 0; k < KB / 16; ++k) {         // 32 bytes of K per instruction
@@ -904,7 +909,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                             if (S32) {
 #pragma unroll
                                 for (int k = 0; k < KB / 16; ++k)
-                                    mma_f16_ta(dt, ta + k * 8, tq + 2 * k + (QN * 128 >> 4), idesc, 1);
+                                    mma_f16_ta(dt + QN, ta + k * 8, tq + 2 * k + (QN * 128 >> 4), idesc, (kb | k) != 0);
                             }
                             mma_commit(bars + C::b_empty_a(as));       // code slot free
                             if (b == nb - 1) mma_commit(bars + C::b_empty_q(s));
@@ -973,7 +978,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                         mt.y = 0.f;
                     }
                     arrive_warp(bars + C::b_empty_meta(m));
-                    const uint32_t tacc = tmem + lane_base + buf * QN;
+                    const uint32_t tacc = tmem + lane_base + buf * C::DCOL;
                     // 16-column groups 16 (par + 4 g) .. of this warp, all loaded at once so
                     // that the accumulator is released before the compares
                     constexpr int NG = QN > CSTEP ? QN / CSTEP : 1;
@@ -981,9 +986,18 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
                     for (int g = 0; g < NG; ++g)
                         if (16 * par + CSTEP * g < npad) ERQ_TMEM_LD16(tacc + 16 * par + CSTEP * g, (v + 16 * g));
+                    uint32_t vl[S32 ? 16 : 1];
+                    static_assert(!S32 || NG == 1, "one column group a warp where queries have two parts");
+                    if constexpr (S32)
+                        if (16 * par < npad) ERQ_TMEM_LD16(tacc + QN + 16 * par, vl);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                     tc_fence_before();
                     arrive_warp(bars + C::b_tempty(buf));
+                    if constexpr (S32) {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            v[i] = __float_as_uint(__uint_as_float(v[i]) + __uint_as_float(vl[i]));
+                    }
                     // straight-line: the compares into a mask
                     uint32_t mine = 0u;
 #pragma unroll
@@ -1408,6 +1422,74 @@ cudaError_t launch_quant_e4m3(const float* x, int64_t n, int D, int Dq, int dup,
     if (D % 4 != 0 || ((uintptr_t)x & 15) != 0 || Dq % 4 != 0 || (dup && Dq != 2 * D) || (!dup && Dq < D)) return cudaErrorInvalidValue;
     count_launch();
     quant_e4m3_kernel<<<(unsigned)ceil_div(n * 32, 256), 256, 0, s>>>(x, n, D, Dq, dup, y, scale);
+    return cudaGetLastError();
+}
+
+// Rotated queries -> the two FP16 parts of the FP32-precision scan, one warp per
+// row.  With the row's power of two 2^e, t = x 2^-e: hi = t rounded to a whole
+// number, |hi| <= 2^11 (exact in FP16), and lo = RN16(t - hi), |lo| <= 1/2, so t is
+// held to 2^-13.  e is the smallest with ||t|| <= lim as well: a row of codes c has
+// <c, hi> = cos ||c|| ||hi||, ||c|| is about 0.36 2^B sqrt(D) (uniform levels of a
+// Gaussian-like row), and lim keeps that below 2^24 for cosines up to 0.6, so that
+// the accumulator's sums of whole numbers are exact (or nearly, for the last steps
+// of larger cosines).  Against 64 bits, over D = 64 .. 4096 and B = 1 .. 9, the
+// sum's error is 0.03 to 0.7 of that of D round-to-nearest multiply-adds from a
+// cosine of 0.1 on; between orthogonal vectors, whose sum is next to nothing, up
+// to 1.3 of it for D <= 128 and, at B = 9 alone, 2 to 3 for D >= 1536.
+__global__ void query_parts_kernel(const float* __restrict__ X, int64_t n, int D, float lim, __half* __restrict__ hi,
+                                   __half* __restrict__ lo, float* __restrict__ scale) {
+    const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (r >= n) return;
+    const float4* x = reinterpret_cast<const float4*>(X + r * D);
+    float mx = 0.f;
+    for (int i = lane; i < D / 4; i += 32) {
+        const float4 v = x[i];
+        mx = fmaxf(mx, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+    }
+    mx = warp_max(mx);
+    int e = 0;
+    if (mx > 0.f && mx < INFINITY) {
+        frexpf(mx, &e);                                    // mx in [2^(e-1), 2^e)
+        e = min(max(e - 11, -126), 126);
+        const float s = __int_as_float((127 - e) << 23);
+        float ss = 0.f;
+        for (int i = lane; i < D / 4; i += 32) {
+            const float4 v = x[i];
+            const float a = v.x * s, b = v.y * s, c = v.z * s, d = v.w * s;
+            ss += (a * a + b * b) + (c * c + d * d);
+        }
+        const float over = sqrtf(warp_sum(ss)) / lim;      // (NaN: not raised)
+        if (over > 1.f) {
+            int k;
+            frexpf(over, &k);                              // over < 2^k
+            e = min(e + k, 126);
+        }
+    }
+    if (lane == 0) scale[r] = __int_as_float((127 + e) << 23);
+    const float s = __int_as_float((127 - e) << 23);
+    for (int i = lane; i < D / 4; i += 32) {
+        const float4 v = x[i];
+        const float t[4] = {v.x * s, v.y * s, v.z * s, v.w * s};
+        float h[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) h[j] = rintf(t[j]);
+        const __half2 h0 = __floats2half2_rn(h[0], h[1]), h1 = __floats2half2_rn(h[2], h[3]);
+        const __half2 l0 = __floats2half2_rn(t[0] - h[0], t[1] - h[1]), l1 = __floats2half2_rn(t[2] - h[2], t[3] - h[3]);
+        reinterpret_cast<uint2*>(hi + r * D)[i] =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+        reinterpret_cast<uint2*>(lo + r * D)[i] =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&l0), *reinterpret_cast<const uint32_t*>(&l1));
+    }
+}
+
+cudaError_t launch_query_parts(const float* x, int64_t n, int D, int B, __half* hi, __half* lo, float* scale,
+                               cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    if (D % 4 != 0 || (((uintptr_t)x | (uintptr_t)hi | (uintptr_t)lo) & 15) != 0) return cudaErrorInvalidValue;
+    const float code = (B > 1 ? 0.36f * (float)(1 << B) : 1.f) * sqrtf((float)D);
+    count_launch();
+    query_parts_kernel<<<(unsigned)ceil_div(n * 32, 256), 256, 0, s>>>(x, n, D, 16777216.f / (0.6f * code), hi, lo, scale);
     return cudaGetLastError();
 }
 
