@@ -63,12 +63,17 @@ struct DevChecks {
 // Order-preserving map of an FP32 value to uint32 (NaN sorts last).
 __host__ __device__ inline uint32_t float_to_ordered(float f) {
 #ifdef __CUDA_ARCH__
-    uint32_t u = __float_as_uint(f);
+    // (an integer instruction by name: setting the sign bit of a float may be
+    // compiled as its negated magnitude, which leaves a NaN's sign undefined)
+    const uint32_t u = __float_as_uint(f), m = (uint32_t)((int32_t)u >> 31) | 0x80000000u;
+    uint32_t o;
+    asm("xor.b32 %0, %1, %2;" : "=r"(o) : "r"(u), "r"(m));
+    return o;
 #else
     uint32_t u;
     memcpy(&u, &f, 4);
-#endif
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+#endif
 }
 __host__ __device__ inline float ordered_to_float(uint32_t o) {
     uint32_t u = (o & 0x80000000u) ? (o & 0x7fffffffu) : ~o;

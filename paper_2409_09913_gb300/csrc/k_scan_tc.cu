@@ -1014,11 +1014,17 @@ __global__ void __launch_bounds__(THREADS, 1)
                                 for (int j = 0; j < 4; ++j) {
                                     float x = __uint_as_float(v[16 * g + i + j]);
                                     if (SC) x *= s4[j];             // a power of two: exact
-                                    if (fmaf(mt.y, x, mt.x) <= t4[j]) mine |= 1u << (16 * g + i + j);
+                                    const float val = fmaf(mt.y, x, mt.x);
+                                    if (S32 ? !(val > t4[j]) : val <= t4[j]) mine |= 1u << (16 * g + i + j);
                                 }
                             }
                         }
                     }
+                    // FP32 precision ranks estimates that are not numbers last, as the
+                    // CUDA-core scan does (a query with a NaN or one whose distances
+                    // overflow): its comparison admits them, so the rows past the block
+                    // and the padding queries are taken out here
+                    if (S32) mine = row < nrows - r ? mine & ((1u << min(max(nqi - 16 * par, 0), 16)) - 1u) : 0u;
                     // every thread appends its own candidates: as many rounds as the
                     // thread with the most has, usually two or three
                     while (__any_sync(0xffffffffu, mine != 0u)) {
