@@ -801,12 +801,14 @@ cudaError_t launch_row_argmin(const float* V, int64_t rows, int ncols, int32_t* 
 // 768: 930 us a pass with FP32 products alone, 340 us.
 // ---------------------------------------------------------------------------
 struct AssignBound {
-    float f, x2;
+    float fx, x2;                                                    // (|x| and |c| apart: x2 c2 underflows for small rows)
     __device__ __forceinline__ float operator()(float c2) const {    // (twice E: the product enters as 2 <x, c>)
-        return f * sqrtf(x2 * c2) + 0x1p-21f * (x2 + c2);
+        return fx * sqrtf(c2) + 0x1p-21f * (x2 + c2);
     }
 };
-__device__ __forceinline__ AssignBound assign_bound(int D, float x2) { return {2.02f * 8.f * 0x1p-24f * (float)D, x2}; }
+__device__ __forceinline__ AssignBound assign_bound(int D, float x2) {
+    return {2.02f * 8.f * 0x1p-24f * (float)D * sqrtf(x2), x2};
+}
 
 // One warp per row: decides it, or lists it with the upper bound of its smallest distance.
 __global__ void __launch_bounds__(256) assign_certain_kernel(const float* __restrict__ V,
