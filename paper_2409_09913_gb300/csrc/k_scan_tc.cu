@@ -1077,9 +1077,11 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const int ql = warp + NEP * lane;
                 int cl = ql < nqi ? (int)s_cnt[ql] : 0;
                 int64_t ol = 0;
-                if (ql < nqi) {
+                bool put = ql < nqi;                                // this lane's list is written
+                if (put) {
                     ol = (int64_t)(uint32_t)iq[ql].z | ((int64_t)iq[ql].w << 32);
-                    if (!ERQ_DCHECK(ol >= 0 && ol < a.ck.lists && cl >= 0 && cl <= C::TRIG, a.ck.status, 6)) cl = 0;
+                    put = ERQ_DCHECK(ol >= 0 && ol < a.ck.lists && cl >= 0 && cl <= C::TRIG, a.ck.status, 6);
+                    if (!put) cl = 0;
                 }
                 for (uint32_t todo = __ballot_sync(0xffffffffu, cl >= kp); todo; todo &= todo - 1u) {
                     const int j = __ffs(todo) - 1, q = warp + NEP * j;
@@ -1094,7 +1096,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     if (lane == j) cl = n;
                 }
                 __syncwarp();
-                if (ql < nqi) a.inter_cnt[ol] = cl;
+                if (put) a.inter_cnt[ol] = cl;
                 for (uint32_t todo = __ballot_sync(0xffffffffu, cl > 0); todo; todo &= todo - 1u) {
                     const int j = __ffs(todo) - 1;
                     const int n = __shfl_sync(0xffffffffu, cl, j);
