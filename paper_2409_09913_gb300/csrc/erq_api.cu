@@ -63,7 +63,8 @@ void free_index_arrays(erq_index* ix) {
                     ix->dstats, ix->PT_hi, ix->P_hi, ix->C_hi, ix->dctr, ix->rowmeta1, ix->ws_ts};   // PT_lo / P_lo / C_lo live inside those blocks
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    if (ix->pinned) cudaFreeHost(ix->pinned);
+    if (ix->plan_status) cudaFreeHost(ix->plan_status);
+    if (ix->plan_done) cudaEventDestroy(ix->plan_done);
     if (ix->ev_ring) {
         for (int i = 0; i < erq_index::kTimingRing * 7; ++i)
             if (ix->ev_ring[i]) cudaEventDestroy(ix->ev_ring[i]);
@@ -895,8 +896,8 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
         for (int i = 0; i < std::min(maxp, nlist); ++i) Ltot += (size[i] + RR - 1) / RR;
         Ltot *= nq;
         nitems = std::min((size[0] + RR - 1) / RR * ceil_div(nq * (int64_t)maxp, QT) + ix->N / RR + nlist, Ltot);
-        // a synchronous search takes the bounds too where they are small, and reads
-        // its status once at its end instead of its sizes in the middle
+        // a synchronous search takes the bounds too where they are small: nothing is
+        // read back before its kernels are launched
         bounded = async || (Ltot * lstride * 8 + nitems * (int64_t)QT * 16 <= (32 << 20));
     }
     const bool small = bounded && tcp && nq * (int64_t)maxp <= kSmallPairs && nlist <= 16384 && Ltot <= 65536;
@@ -956,6 +957,17 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
         if (Ltot > 0) ERQ_CHECK_CUDA(cudaMemsetAsync(inter_cnt, 0, sizeof(int32_t) * Ltot, s));
         if ((e = launch_plan_fill(pa, s)) != cudaSuccess) return cuda_fail(e, "plan items");
     }
+    // A synchronous search reports what planning found, and returns with the scan,
+    // the merge and the re-rank in flight: the status word as it is here is copied to
+    // the host and awaited once everything is launched.
+    const bool plan_check = bounded && !async && !check_later;
+    if (plan_check) {
+        if (!ix->plan_status && cudaHostAlloc((void**)&ix->plan_status, 4, cudaHostAllocDefault) != cudaSuccess)
+            return fail(ERQ_ENOMEM, "cudaHostAlloc search status");
+        if (!ix->plan_done) ERQ_CHECK_CUDA(cudaEventCreateWithFlags(&ix->plan_done, cudaEventDisableTiming));
+        ERQ_CHECK_CUDA(cudaMemcpyAsync(ix->plan_status, ix->status, 4, cudaMemcpyDeviceToHost, s));
+        ERQ_CHECK_CUDA(cudaEventRecord(ix->plan_done, s));
+    }
     ERQ_TRY(mark(3));
     // ---- scan
     L.Qrot = Qrot; L.Qh = prec == ERQ_PREC_FP32 ? sl[18] : sl[15]; L.Ql = sl[19]; L.Q8 = sl[21]; L.qscale = (const float*)sl[22]; L.Dq = Dq; L.status = ix->status; L.N = ix->N; L.codes = ix->codes; L.g_const = ix->g_const; L.f_res = ix->f_res; L.list_off = ix->list_off;
@@ -989,7 +1001,10 @@ static erq_status search_impl(erq_index* ix, const float* Q, int64_t nq, const e
         ix->timed = 1;
         ++ix->timing_seq;
     }
-    if (bounded && !async && !check_later) return check_status(ix, s);   // (read together with the sizes otherwise)
+    if (plan_check) {
+        ERQ_CHECK_CUDA(cudaEventSynchronize(ix->plan_done));
+        if (*ix->plan_status) return check_status(ix, s);
+    }
     return ERQ_OK;
 }
 

@@ -164,7 +164,8 @@ struct erq_index {
     size_t ws_b_bytes = 0;
     void* io = nullptr;          // device staging of erq_search_host
     size_t io_bytes = 0;
-    void* pinned = nullptr;      // pinned host staging for erq_search_host
+    uint32_t* plan_status = nullptr;      // pinned host copy of the status word after a search's planning,
+    cudaEvent_t plan_done = nullptr;      //     complete at this event (synchronous searches of bounded sizes)
     static constexpr int kTimingRing = 512;   // timed searches whose phase events are kept
     cudaEvent_t* ev_ring = nullptr;  // [kTimingRing][7] phase boundaries of timed searches
     int64_t timing_seq = 0;      // timed searches so far
@@ -182,6 +183,5 @@ struct erq_index {
     unsigned long long* dstats = nullptr;  // [8] device counters of the last search: pairs, distinct rows, tensor-core
                                            //     row blocks, row blocks x padded queries, candidate lists, work items
     std::vector<int64_t>* sizes_desc = nullptr;   // list sizes in decreasing order (bounds of a search's lists and items)
-    size_t pinned_bytes = 0;
     int64_t device_bytes = 0;
 };
