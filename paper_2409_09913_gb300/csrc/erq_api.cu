@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <functional>
 #include <cstdio>
 #include <cstring>
@@ -519,10 +520,16 @@ extern "C" erq_status erq_build_index(const float* X, int64_t N, int32_t D, cons
 // Work-item shape of the scan: queries per item (the tensor-core MMA's N
 // extent) and rows per item; the autotuned or forced shape wins.  For k' <= 32,
 // 128 queries per item (twice the MMA width for one conversion of the codes)
-// when a probed cluster has more than 72 probing queries on average, else 64
-// (10,000 queries x 16 of 2,048 lists, 78 a list: 0.38 ms with 64, 0.31 with
-// 128; 512 x 64 of 512, 64 a list: 0.095 with 64, 0.16 with 128); for larger
-// k' 32.  FP32 precision has two query parts per tile and stops at 64.  Rows:
+// when a probed cluster has more than 72 probing queries on average and there is
+// work enough that the last items do not leave SMs idle for long: items x D of at
+// least 5,000 an SM.  Otherwise 64; for larger k' 32.  The whole search's time with
+// 64 over that with 128, from 72 to 192 queries a list, by items x D an SM (D = 64
+// .. 1536, B = 1 .. 9, FP16 and e4m3, 60 .. 400 rows a list, k' = 20 and 32):
+//   256 lists, 110 .. 2,600: 0.81 .. 1.00    512 lists, 1,300 .. 3,200: 0.85 .. 1.02
+//   1,024 lists, 860: 0.93 .. 0.99           2,048 lists, 1,700: 0.96 .. 1.01
+//   1,024 and 512 lists, 5,200: 0.96 .. 1.09
+//   2,048 lists, 5,200 .. 20,700: 0.97 .. 1.11
+// FP32 precision has two query parts per tile and stops at 64.  Rows:
 // at most 8,192, and few enough that the items can fill the chip twice (a
 // single query's 16 lists of 200 rows are 32 one-block items instead of 16), but
 // no list is cut into more items than there are SMs: queries go where the rows
@@ -538,14 +545,20 @@ static void choose_scan_shape(const erq_index* ix, int prec, int kp, int64_t nq,
     const int cls = kp <= 32 ? 0 : 1;
     const int64_t work = nq * (int64_t)maxp;
     const double per_list = (double)work / ix->nlist;
-    int q = cls == 0 ? (per_list > 72.0 && prec != ERQ_PREC_FP32 ? 128 : 64) : 32;
-    // rows of all items: the probed lists' rows, once per chunk of queries
     const double lists = (double)std::min<int64_t>(ix->nlist, work);
-    const double chunks = std::max(1.0, (double)work / lists / q);
-    const double rows = (double)ix->N * lists / ix->nlist * chunks;
-    int r = 8192;
-    if (rows < 8192.0 * 2 * sms) r = std::max(128, (int)(rows / (2.0 * sms)) / 128 * 128);
-    r = (int)std::min<int64_t>(8192, std::max<int64_t>(r, ceil_div(ix->max_list, (int64_t)sms * 128) * 128));
+    auto rows_of = [&](int qn) {
+        // rows of all items: the probed lists' rows, once per chunk of queries
+        const double rows = (double)ix->N * lists / ix->nlist * std::max(1.0, (double)work / lists / qn);
+        int64_t rr = 8192;
+        if (rows < 8192.0 * 2 * sms) rr = std::max(128, (int)(rows / (2.0 * sms)) / 128 * 128);
+        return (int)std::min<int64_t>(8192, std::max<int64_t>(rr, ceil_div(ix->max_list, (int64_t)sms * 128) * 128));
+    };
+    int q = cls == 0 ? 64 : 32;
+    if (cls == 0 && prec != ERQ_PREC_FP32 && per_list > 72.0) {
+        const double ranges = std::ceil((double)ix->N / ix->nlist / rows_of(128));
+        if (lists * ranges * std::ceil((double)work / lists / 128.0) * ix->D >= 5000.0 * sms) q = 128;
+    }
+    int r = rows_of(q);
     const erq_index::ScanTune& t = ix->tune[cls];
     if (prec != ERQ_PREC_FP32 && t.valid && work <= 4 * t.work && 4 * work >= t.work) {
         q = t.qn;

@@ -1,6 +1,7 @@
-"""Rows of a scan work item where list sizes differ: the largest list is not cut
-into more items than the chip has SMs, whatever the average list holds, and the
-results are those of any other shape."""
+"""Shapes of scan work items.  Rows where list sizes differ: the largest list is
+not cut into more items than the chip has SMs, whatever the average list holds, and
+the results are those of any other shape.  Queries: 128 an item only where lists
+have many queries and the chip has many items."""
 import numpy as np
 import pytest
 import torch
@@ -28,4 +29,18 @@ def test_one_large_list(erq, nq, precision, async_mode):
     assert -(-190_000 // rows) <= sms
     ix.set_scan_config(0, 2048)
     for a, b in zip(got, ix.search(Q, 10, **kw)):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("nlist,D,per_list,rows,want", [(256, 64, 80, 20, 64), (256, 64, 200, 20, 64), (512, 1536, 80, 20, 128),
+                                                         (512, 1536, 60, 20, 64), (512, 960, 80, 20, 64), (4096, 192, 80, 4, 128)])
+def test_queries_of_an_item(erq, nlist, D, per_list, rows, want):
+    N, np_ = nlist * rows, 16
+    X, _ = S.mixture(N, D, 8, 74)
+    ix = erq.build_index(to_dev(X), to_dev(S.random_orthogonal(D, 75)), 3, nlist, assign=to_dev(np.arange(N, dtype=np.int32) % nlist))
+    Q = to_dev(np.resize(S.mixture(997, D, 8, 76, comp_seed=74)[0], (per_list * nlist // np_, D)))
+    got = ix.search(Q, 10, rerank_k=20, nprobe=np_, precision="fp16")
+    assert ix.scan_config()[0] == want
+    ix.set_scan_config(192 - want, 0)                     # the other one gives the same
+    for a, b in zip(got, ix.search(Q, 10, rerank_k=20, nprobe=np_, precision="fp16")):
         assert torch.equal(a, b)
