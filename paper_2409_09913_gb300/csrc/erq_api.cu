@@ -518,7 +518,7 @@ extern "C" erq_status erq_build_index(const float* X, int64_t N, int32_t D, cons
 // Search
 // ---------------------------------------------------------------------------
 // Work-item shape of the scan: queries per item (the tensor-core MMA's N
-// extent) and rows per item; the autotuned or forced shape wins.  For k' <= 32,
+// extent) and rows per item.  For k' <= 32,
 // 128 queries per item (twice the MMA width for one conversion of the codes)
 // when a probed cluster has more than 72 probing queries on average and there is
 // work enough that the last items do not leave SMs idle for long: items x D of at
@@ -536,12 +536,7 @@ extern "C" erq_status erq_build_index(const float* X, int64_t N, int32_t D, cons
 // are, and a query's lists of candidates have to be merged (one query whose
 // nearest list holds 900,000 of 1,000,000 x 128 rows: 0.94 ms in the 7,000 items
 // that the average list asks for, 0.13 in 150; 300,000 rows: 0.40 and 0.10).
-static void choose_scan_shape(const erq_index* ix, int prec, int kp, int64_t nq, int maxp, int sms, int* qn, int* rr) {
-    if (prec == ERQ_PREC_FP32 && kp > 128) {              // the CUDA-core scan
-        *qn = 64;
-        *rr = ix->force_rr > 0 ? ix->force_rr : 4096;
-        return;
-    }
+static void default_scan_shape(const erq_index* ix, int prec, int kp, int64_t nq, int maxp, int sms, int* qn, int* rr) {
     const int cls = kp <= 32 ? 0 : 1;
     const int64_t work = nq * (int64_t)maxp;
     const double per_list = (double)work / ix->nlist;
@@ -558,8 +553,21 @@ static void choose_scan_shape(const erq_index* ix, int prec, int kp, int64_t nq,
         const double ranges = std::ceil((double)ix->N / ix->nlist / rows_of(128));
         if (lists * ranges * std::ceil((double)work / lists / 128.0) * ix->D >= 5000.0 * sms) q = 128;
     }
-    int r = rows_of(q);
-    const erq_index::ScanTune& t = ix->tune[cls];
+    *qn = q;
+    *rr = rows_of(q);
+}
+
+// The forced or autotuned shape, else the default.
+static void choose_scan_shape(const erq_index* ix, int prec, int kp, int64_t nq, int maxp, int sms, int* qn, int* rr) {
+    if (prec == ERQ_PREC_FP32 && kp > 128) {              // the CUDA-core scan
+        *qn = 64;
+        *rr = ix->force_rr > 0 ? ix->force_rr : 4096;
+        return;
+    }
+    int q, r;
+    default_scan_shape(ix, prec, kp, nq, maxp, sms, &q, &r);
+    const int64_t work = nq * (int64_t)maxp;
+    const erq_index::ScanTune& t = ix->tune[kp <= 32 ? 0 : 1];
     if (prec != ERQ_PREC_FP32 && t.valid && work <= 4 * t.work && 4 * work >= t.work) {
         q = t.qn;
         r = t.rr;
@@ -1361,8 +1369,28 @@ extern "C" erq_status erq_autotune(erq_index* ix, const float* Q, int64_t nq, co
     const int kp = std::max(p->k, p->rerank_k);
     const int cls = kp <= 32 ? 0 : 1;
     const int maxp = p->probe ? p->nprobe : (ix->nlist == 1 ? 1 : p->nprobe);
-    const int qns[3] = {32, 64, 128};
-    const int rrs[3] = {2048, 4096, 8192};
+    // the shape that an untuned search takes comes first, then it with half and twice
+    // the rows, then the grid; another one is kept only if it beats the first by more
+    // than the timing's noise, and otherwise later searches stay untuned
+    struct Shape { int qn, rr; };
+    std::vector<Shape> shapes;
+    auto add = [&](int qn, int rr) {
+        for (const Shape& x : shapes)
+            if (x.qn == qn && x.rr == rr) return;
+        shapes.push_back({qn, rr});
+    };
+    {
+        int dev = 0, sms = 148, q0 = 0, r0 = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        default_scan_shape(ix, p->precision, kp, nq, maxp, sms, &q0, &r0);
+        add(q0, r0);
+        add(q0, std::max(128, r0 / 2 / 128 * 128));
+        add(q0, 2 * r0);
+        for (int qn : {32, 64, 128})
+            for (int rr : {2048, 4096, 8192})
+                if (scan_tc_shape_ok(qn, kp)) add(qn, rr);
+    }
     int64_t* ids = nullptr;
     float* dists = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1374,44 +1402,41 @@ extern "C" erq_status erq_autotune(erq_index* ix, const float* Q, int64_t nq, co
         st = fail(ERQ_ECUDA, "erq_autotune: cudaEventCreate");
     const int keep_qn = ix->force_qn, keep_rr = ix->force_rr;
     float best = -1.f;
-    int bq = 0, br = 0;
+    size_t chosen = 0;
     erq_search_params pp = *p;
     pp.flags &= ~ERQ_SEARCH_TIMING;
     pp.cand_ids = nullptr;
     pp.cand_est = nullptr;
-    for (int qi = 0; qi < 3 && st == ERQ_OK; ++qi) {
-        if (!scan_tc_shape_ok(qns[qi], kp)) continue;
-        for (int ri = 0; ri < 3 && st == ERQ_OK; ++ri) {
-            ix->force_qn = qns[qi];
-            ix->force_rr = rrs[ri];
-            if ((st = search_impl(ix, Q, nq, &pp, ids, dists, s)) != ERQ_OK) break;   // warm-up, sizes buffers
-            if (cudaEventRecord(e0, s) != cudaSuccess) { st = fail(ERQ_ECUDA, "erq_autotune: event"); break; }
-            for (int r = 0; r < reps && st == ERQ_OK; ++r) st = search_impl(ix, Q, nq, &pp, ids, dists, s);
-            if (st != ERQ_OK) break;
-            float ms = 0.f;
-            if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
-                cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
-                st = fail(ERQ_ECUDA, "erq_autotune: timing");
-                break;
-            }
-            if (best < 0.f || ms < best) {
-                best = ms;
-                bq = qns[qi];
-                br = rrs[ri];
-            }
+    for (size_t i = 0; i < shapes.size() && st == ERQ_OK; ++i) {
+        ix->force_qn = shapes[i].qn;
+        ix->force_rr = shapes[i].rr;
+        if ((st = search_impl(ix, Q, nq, &pp, ids, dists, s)) != ERQ_OK) break;   // warm-up, sizes buffers
+        if (cudaEventRecord(e0, s) != cudaSuccess) { st = fail(ERQ_ECUDA, "erq_autotune: event"); break; }
+        for (int r = 0; r < reps && st == ERQ_OK; ++r) st = search_impl(ix, Q, nq, &pp, ids, dists, s);
+        if (st != ERQ_OK) break;
+        float ms = 0.f;
+        if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+            cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
+            st = fail(ERQ_ECUDA, "erq_autotune: timing");
+            break;
+        }
+        if (i == 0) best = 0.97f * ms;
+        else if (ms < best) {
+            best = ms;
+            chosen = i;
         }
     }
     ix->force_qn = keep_qn;
     ix->force_rr = keep_rr;
     if (st == ERQ_OK) st = check_status(ix, s);
     if (st == ERQ_OK && best >= 0.f) {
-        ix->tune[cls].valid = 1;
+        ix->tune[cls].valid = chosen != 0;
         ix->tune[cls].work = nq * (int64_t)maxp;
-        ix->tune[cls].qn = bq;
-        ix->tune[cls].rr = br;
+        ix->tune[cls].qn = shapes[chosen].qn;
+        ix->tune[cls].rr = shapes[chosen].rr;
         if (best_out) {
-            best_out[0] = bq;
-            best_out[1] = br;
+            best_out[0] = shapes[chosen].qn;
+            best_out[1] = shapes[chosen].rr;
         }
     }
     if (e0) cudaEventDestroy(e0);

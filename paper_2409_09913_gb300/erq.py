@@ -300,9 +300,10 @@ class Index:
         return dict(zip(("rotate", "probe", "plan", "scan", "merge", "rerank"), list(ms)))
 
     def autotune(self, Q, k, *, rerank_k=0, nprobe=1, precision="fp16", nprobe_per_query=None, reps=3, metric="l2"):
-        """Time every supported scan work-item shape on this query batch and keep
-        the fastest for later searches of this size; returns (queries per item,
-        rows per item)."""
+        """Time the shape an untuned search takes (also with half and twice its rows)
+        and a grid of scan work-item shapes on this query batch and keep the fastest
+        for later searches of this size, none if the untuned one is within 3 %;
+        returns (queries per item, rows per item)."""
         Q = _dev(Q, torch.float32, "Q", 2)
         sp = SearchParams()
         sp.k, sp.rerank_k, sp.nprobe, sp.precision = int(k), int(rerank_k), int(nprobe), PREC[precision]

@@ -1,7 +1,10 @@
 """Shapes of scan work items.  Rows where list sizes differ: the largest list is
 not cut into more items than the chip has SMs, whatever the average list holds, and
 the results are those of any other shape.  Queries: 128 an item only where lists
-have many queries and the chip has many items."""
+have many queries and the chip has many items.  Tuning never leaves a shape much
+slower than the untuned one."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -44,3 +47,32 @@ def test_queries_of_an_item(erq, nlist, D, per_list, rows, want):
     ix.set_scan_config(192 - want, 0)                     # the other one gives the same
     for a, b in zip(got, ix.search(Q, 10, rerank_k=20, nprobe=np_, precision="fp16")):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("nlist,nq,np_", [(1, 100, 1), (1, 1, 1), (64, 1, 8), (64, 300, 16)])
+def test_tuning_is_not_slower_than_the_default(erq, nlist, nq, np_):
+    N, D = 10_000, 128
+    X, _ = S.mixture(N, D, 8, 77)
+    Q = to_dev(S.mixture(nq, D, 8, 78, comp_seed=77)[0])
+    ix = erq.build_index(to_dev(X), to_dev(S.random_orthogonal(D, 79)), 4, nlist, assign=to_dev(np.arange(N, dtype=np.int32) % nlist))
+    kw = dict(rerank_k=20, nprobe=np_, precision="fp16")
+    plain = ix.search(Q, 10, **kw)
+    shape = ix.scan_config()
+
+    def us():
+        best = []
+        for _ in range(7):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            for _ in range(20):
+                ix.search(Q, 10, async_mode=True, **kw)
+            torch.cuda.synchronize()
+            best.append((time.perf_counter() - t0) / 20 * 1e6)
+        return min(best)
+
+    before = us()
+    tuned = ix.autotune(Q, 10, reps=5, **kw)
+    for a, b in zip(plain, ix.search(Q, 10, **kw)):
+        assert torch.equal(a, b)
+    assert ix.scan_config() == tuned
+    assert tuned == shape or us() <= 1.1 * before
