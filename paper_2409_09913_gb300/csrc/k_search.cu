@@ -898,7 +898,8 @@ __global__ void __launch_bounds__(256) rerank_kernel(const uint64_t* __restrict_
 }
 
 // ---------------------------------------------------------------------------
-// Estimates of explicit pairs (FP32).  A block takes up to 128 of a query's ids:
+// Estimates of explicit pairs (FP32), in two forms of the same sums in the same
+// order (launch_estimate).  estimate_kernel: a block takes up to 128 of a query's ids:
 // q_r and P^T q_r stay in shared memory, the ids' rows and clusters are looked
 // up once, and each warp streams its pairs' centroid and code rows through two
 // shared-memory slots of its own with bulk copies (16-byte aligned: D is a
@@ -928,6 +929,33 @@ __device__ __forceinline__ float4 codes4(const uint8_t* p, float off) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) f[i] = fmaf(2.f, __uint_as_float(u[i]) - 8388608.f, -off);
     return make_float4(f[0], f[1], f[2], f[3]);
+}
+
+// Four coordinates of a pair: into ||q_r - c||^2 (or <c, q_r>) and <2 ybar, q'>.
+__device__ __forceinline__ void estimate_add(const float4 cv, const float4 yv, const float4 x, const float4 xr, int ipm,
+                                             float4& dq, float4& ip) {
+    if (ipm) {
+        dq.x = fmaf(cv.x, x.x, dq.x);
+        dq.y = fmaf(cv.y, x.y, dq.y);
+        dq.z = fmaf(cv.z, x.z, dq.z);
+        dq.w = fmaf(cv.w, x.w, dq.w);
+    } else {
+        const float d0 = x.x - cv.x, d1 = x.y - cv.y, d2 = x.z - cv.z, d3 = x.w - cv.w;
+        dq.x = fmaf(d0, d0, dq.x);
+        dq.y = fmaf(d1, d1, dq.y);
+        dq.z = fmaf(d2, d2, dq.z);
+        dq.w = fmaf(d3, d3, dq.w);
+    }
+    ip.x = fmaf(yv.x, xr.x, ip.x);
+    ip.y = fmaf(yv.y, xr.y, ip.y);
+    ip.z = fmaf(yv.z, xr.z, ip.z);
+    ip.w = fmaf(yv.w, xr.w, ip.w);
+}
+// Squared distance ||q_r - c||^2 + g + (f_res/2) <2 ybar, q'>, or inner product
+// <c, q_r> - (f_res/4) <2 ybar, q'>.
+__device__ __forceinline__ float estimate_of(float dq, float ip, int64_t row, const float* __restrict__ g_const,
+                                             const float* __restrict__ f_res, int ipm) {
+    return ipm ? dq - 0.25f * f_res[row] * ip : dq + g_const[row] + 0.5f * f_res[row] * ip;
 }
 
 template <int CB>
@@ -991,37 +1019,61 @@ __global__ void __launch_bounds__(256) estimate_kernel(const float* __restrict__
         float4 dq = make_float4(0.f, 0.f, 0.f, 0.f), ip = dq;
 #pragma unroll 4
         for (int k = lane * 4; k < D; k += 128) {
-            const float4 cv = *reinterpret_cast<const float4*>(c + k), yv = codes4<CB>(code + k * CB, off);
-            const float4 x = *reinterpret_cast<const float4*>(es + k), xr = *reinterpret_cast<const float4*>(es + D + k);
-            if (ipm) {                                 // <c, q_r>
-                dq.x = fmaf(cv.x, x.x, dq.x);
-                dq.y = fmaf(cv.y, x.y, dq.y);
-                dq.z = fmaf(cv.z, x.z, dq.z);
-                dq.w = fmaf(cv.w, x.w, dq.w);
-            } else {
-                const float d0 = x.x - cv.x, d1 = x.y - cv.y, d2 = x.z - cv.z, d3 = x.w - cv.w;
-                dq.x = fmaf(d0, d0, dq.x);
-                dq.y = fmaf(d1, d1, dq.y);
-                dq.z = fmaf(d2, d2, dq.z);
-                dq.w = fmaf(d3, d3, dq.w);
-            }
-            ip.x = fmaf(yv.x, xr.x, ip.x);
-            ip.y = fmaf(yv.y, xr.y, ip.y);
-            ip.z = fmaf(yv.z, xr.z, ip.z);
-            ip.w = fmaf(yv.w, xr.w, ip.w);
+            estimate_add(*reinterpret_cast<const float4*>(c + k), codes4<CB>(code + k * CB, off),
+                         *reinterpret_cast<const float4*>(es + k), *reinterpret_cast<const float4*>(es + D + k), ipm, dq, ip);
         }
         __syncwarp();                                  // the slot has been read
         if (lane == 0 && j + 2 * nw < nj) issue(j + 2 * nw, slot);
         const float dqs = warp_sum((dq.x + dq.y) + (dq.z + dq.w)), ips = warp_sum((ip.x + ip.y) + (ip.z + ip.w));
-        // squared distance ||q_r - c||^2 + g + (f_res/2) <2 ybar, q'>, or inner
-        // product <c, q_r> - (f_res/4) <2 ybar, q'>
         if (lane == 0) {
             const int64_t row = s_row[j];
-            est[q * nc + j0 + j] = row < 0 ? NAN
-                                   : ipm   ? dqs - 0.25f * f_res[row] * ips
-                                           : dqs + g_const[row] + 0.5f * f_res[row] * ips;
+            est[q * nc + j0 + j] = row < 0 ? NAN : estimate_of(dqs, ips, row, g_const, f_res, ipm);
         }
     }
+}
+
+// W lanes per pair (16 for D = 64, one coordinate group a lane; else a warp), both
+// rows and both query rows read as they are: the form for few pairs a query, where
+// staging costs more than it saves, and for long rows.
+template <int CB, int W>
+__global__ void __launch_bounds__(256) estimate_pair_kernel(const float* __restrict__ Q, const float* __restrict__ Qrot,
+                                                            const int64_t* __restrict__ ids, int64_t nq, int nc, int64_t N,
+                                                            const int64_t* __restrict__ row_of,
+                                                            const int32_t* __restrict__ cl_of_row,
+                                                            const float* __restrict__ C,
+                                                            const uint8_t* __restrict__ codes,
+                                                            const float* __restrict__ g_const,
+                                                            const float* __restrict__ f_res, int D, int B, int ipm,
+                                                            float* __restrict__ est, uint32_t* __restrict__ status) {
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / W;
+    const int lane = threadIdx.x & (W - 1);
+    if (w >= nq * nc) return;
+    const int64_t q = w / nc, id = ids[w];
+    if (id < 0 || id >= N) {
+        if (lane == 0) {
+            est[w] = NAN;
+            if (id >= N) atomicOr(status, kStatusBounds);
+        }
+        return;
+    }
+    const int64_t row = row_of[id];
+    const float* c = C + (int64_t)cl_of_row[row] * D;
+    const uint8_t* code = codes + row * D * CB;
+    const float *x = Q + q * D, *xr = Qrot + q * D;
+    const float off = (float)((1 << B) - 1);
+    float4 dq = make_float4(0.f, 0.f, 0.f, 0.f), ip = dq;
+#pragma unroll 4
+    for (int k = lane * 4; k < D; k += 4 * W)
+        estimate_add(*reinterpret_cast<const float4*>(c + k), codes4<CB>(code + k * CB, off),
+                     *reinterpret_cast<const float4*>(x + k), *reinterpret_cast<const float4*>(xr + k), ipm, dq, ip);
+    float dqs = (dq.x + dq.y) + (dq.z + dq.w), ips = (ip.x + ip.y) + (ip.z + ip.w);
+    const unsigned group = W == 32 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);   // (the other half may have left)
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) {
+        dqs += __shfl_xor_sync(group, dqs, o);
+        ips += __shfl_xor_sync(group, ips, o);
+    }
+    if (lane == 0) est[w] = estimate_of(dqs, ips, row, g_const, f_res, ipm);
 }
 
 // ---------------------------------------------------------------------------
@@ -1413,11 +1465,25 @@ cudaError_t launch_rerank(const uint64_t* cand, int64_t nq, int kp, const float*
 cudaError_t launch_estimate(const float* Q, const float* Qrot, const int64_t* ids, int64_t nq, int nc,
                             const erq_index* ix, int ipm, float* est, cudaStream_t s) {
     if (nq <= 0 || nc <= 0) return cudaSuccess;
-    // two row slots for each of eight warps, four where they would not leave room
-    // for a second block on the SM (D > 1280)
-    const size_t row = (size_t)ix->D * (4 + code_bytes(ix->B)), qs = (size_t)ix->D * 8;
-    const int warps = qs + 16 * row <= 112 * 1024 ? 8 : 4;
-    const size_t smem = qs + 2 * warps * row;
+    // The staged form from 32 ids a query and 65,536 pairs on (262,144 above D = 512),
+    // for D = 128 .. 1024: the lanes of a pair take 1.00 to 1.50 of its time there (8,192
+    // x 100 at D = 256: 280 and 215 us; at D = 1024: 633 and 546), 0.14 to 1.0 of it for
+    // fewer ids or pairs (2,048 x 10 at D = 128: 8 and 13 us), for longer rows (2,048 x
+    // 100 at D = 4096: 490 and 775) and at D = 64 (8,192 x 100: 124 and 190), where a
+    // block's staging is not shared by enough pairs or leaves too few warps on the SM.
+    if (nc < 32 || ix->D == 64 || ix->D > 1024 || nq * nc < (ix->D > 512 ? 262144 : 65536)) {
+        count_launch();
+        const int w = ix->D == 64 ? 16 : 32;
+        const auto kern = ix->B > 8 ? (w == 16 ? estimate_pair_kernel<2, 16> : estimate_pair_kernel<2, 32>)
+                                    : (w == 16 ? estimate_pair_kernel<1, 16> : estimate_pair_kernel<1, 32>);
+        kern<<<(unsigned)ceil_div(nq * nc * w, 256), 256, 0, s>>>(Q, Qrot, ids, nq, nc, ix->N, ix->row_of, ix->cl_of_row, ix->C,
+                                                            ix->codes, ix->g_const, ix->f_res, ix->D, ix->B, ipm, est,
+                                                            ix->status);
+        return cudaGetLastError();
+    }
+    constexpr int warps = 8;
+    const size_t row = (size_t)ix->D * (4 + code_bytes(ix->B));
+    const size_t smem = (size_t)ix->D * 8 + 2 * warps * row;    // (at most 106 KB: two blocks an SM)
     const auto kern = ix->B > 8 ? estimate_kernel<2> : estimate_kernel<1>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
