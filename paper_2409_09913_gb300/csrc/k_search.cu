@@ -783,12 +783,15 @@ __global__ void __launch_bounds__(W == 32 ? 1024 : 256) merge32_kernel(
                 key[u] = kEmptyKey;
                 if (e0 + 32 * u >= total) continue;
                 const int e = e0 + 32 * u + lane;
-                int j = 0;                                             // lists that end at or before entry e
+                int j = 0, before = 0;                                 // lists that end at or before entry e
+                if (nl > 1) {                                          // (one list: nothing to number)
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1)
-                    if (__shfl_sync(0xffffffffu, incl, j + o - 1) <= e) j += o;
-                j = min(j, 31);                                        // (entries past the last)
-                const int prev = __shfl_sync(0xffffffffu, incl, max(j - 1, 0)), before = j > 0 ? prev : 0;
+                    for (int o = 16; o > 0; o >>= 1)
+                        if (__shfl_sync(0xffffffffu, incl, j + o - 1) <= e) j += o;
+                    j = min(j, 31);                                    // (entries past the last)
+                    const int prev = __shfl_sync(0xffffffffu, incl, max(j - 1, 0));
+                    before = j > 0 ? prev : 0;
+                }
                 if (e < total) key[u] = inter[(Lb + j) * lstride + (e - before)];
             }
 #pragma unroll
