@@ -280,14 +280,17 @@ __device__ __forceinline__ float last_bits_dot(const uint64_t* w, const float* x
 }
 
 // The survivors' full estimates (Eq. 4.2) and keys.  Block per (query, probe
-// slot, share of the cluster's 128-row chunks), a warp per 32 rows at a time:
-// survivors are few, so a row's 64-coordinate blocks go to the lanes, G =
+// slot, share of the cluster's 128-row chunks), a warp per 32 rows at a time.
+// Most lists have no survivors: their blocks end after one pass over the bounds.
+// Where few of 32 rows survive, a row's 64-coordinate blocks go to the lanes, G =
 // 32 / W rows side by side with W the power of two that holds them (one row in
 // several rounds beyond 2,048 coordinates); the blocks' sums are then added in
 // order.  A thread per row kept 30 of a warp's lanes waiting for the other two:
-// 134 us for 16 queries x 16 lists of 200,000 x 960 in 1,024, 34 us.  Query
-// coordinates are spaced 65 floats a block so that the lanes' reads fall into
-// different banks.
+// 134 us for 16 queries x 16 lists of 200,000 x 960 in 1,024, 34 us.  Where many
+// survive (half of a query's nearest list), a lane per row is better: from 16 of
+// 32 on, from 8 where the blocks fill only half of the W lanes.  512 queries x 8
+// lists of 20,000 x 1,088 in 32: 406 us with lanes for all, 135.  Query coordinates are spaced 65 floats a
+// block so that the lanes' reads fall into different banks.
 template <int B>
 __global__ void __launch_bounds__(TS_THREADS) ts_stage2_kernel(TsArgs a) {
     extern __shared__ __align__(16) float xq[];            // [D / 64][65] P^T q_r
@@ -298,20 +301,42 @@ __global__ void __launch_bounds__(TS_THREADS) ts_stage2_kernel(TsArgs a) {
     const int64_t size = a.list_off[c + 1] - a.list_off[c], pc = a.poff[c];
     if ((int64_t)blockIdx.y * TS_THREADS >= size) return;
     const int D = a.D, nkb = D / 64;
-    for (int i = threadIdx.x; i < D; i += TS_THREADS) xq[(i >> 6) * 65 + (i & 63)] = a.Qrot[q * D + i];
-    __syncthreads();
     const float dq = a.dqc[q * a.maxp + slot], tq = a.tau[q];
     const int64_t o0 = a.qoffr[q] + a.rbase[q * a.maxp + slot];
+    // (a comparison that keeps rows without an ordered bound)
+    bool any = false;
+#pragma unroll 4
+    for (int64_t j = (int64_t)blockIdx.y * TS_THREADS + threadIdx.x; j < size; j += (int64_t)gridDim.y * TS_THREADS)
+        any |= !(a.lb[o0 + j] > tq);
+    if (!__syncthreads_or(any)) return;
+    for (int i = threadIdx.x; i < D; i += TS_THREADS) xq[(i >> 6) * 65 + (i & 63)] = a.Qrot[q * D + i];
+    __syncthreads();
     const float hi = (float)(1 << (B - 1));
     const int lane = threadIdx.x & 31;
     int W = 1;
     while (W < nkb && W < 32) W <<= 1;
     const int G = 32 / W, g = lane / W, kl = lane & (W - 1);
+    const int many = max(8, 16 * nkb / (W * ((nkb + W - 1) / W)));
+    auto put = [&](int64_t p, int64_t j, float s) {
+        const float4 m = a.rowmeta[p];
+        const float est = dq + fmaf(m.y, fmaf(hi, a.s1[o0 + j], s), m.x);
+        const int pos = atomicAdd(a.scnt + q, 1);
+        a.skey[a.qoffr[q] + pos] = make_key(est, __float_as_uint(m.z));
+    };
     for (int64_t j0 = (int64_t)blockIdx.y * TS_THREADS + (threadIdx.x & ~31); j0 < size;
          j0 += (int64_t)gridDim.y * TS_THREADS) {
         const int64_t j = j0 + lane;
-        // (a comparison that keeps rows without an ordered bound)
         unsigned live = __ballot_sync(0xffffffffu, j < size && !(a.lb[o0 + j] > tq));
+        if (B > 1 && __popc(live) >= many) {               // a lane per row
+            if (live >> lane & 1u) {
+                const int64_t p = pc + j;
+                const uint64_t* w0 = a.codes_p + ((p >> 5) * nkb * B) * 32 + (p & 31);
+                float s = 0.f;
+                for (int kb = 0; kb < nkb; ++kb) s += last_bits_dot<B>(w0 + (int64_t)kb * B * 32, xq + 65 * kb);
+                put(p, j, s);
+            }
+            continue;
+        }
         while (live) {
             unsigned rest = live;
             int r = -1;                                    // my group's row: the (g + 1)-th survivor
@@ -328,12 +353,7 @@ __global__ void __launch_bounds__(TS_THREADS) ts_stage2_kernel(TsArgs a) {
                 const float v = B > 1 && r >= 0 && kb < nkb ? last_bits_dot<B>(w0 + (int64_t)kb * B * 32, xq + 65 * kb) : 0.f;
                 for (int u = 0; u < W && k0 + u < nkb; ++u) s += __shfl_sync(0xffffffffu, v, (lane & ~(W - 1)) + u);
             }
-            if (r >= 0 && kl == 0) {
-                const float4 m = a.rowmeta[p];
-                const float est = dq + fmaf(m.y, fmaf(hi, a.s1[o0 + j0 + r], s), m.x);
-                const int pos = atomicAdd(a.scnt + q, 1);
-                a.skey[a.qoffr[q] + pos] = make_key(est, __float_as_uint(m.z));
-            }
+            if (r >= 0 && kl == 0) put(p, j0 + r, s);
         }
     }
 }
@@ -424,6 +444,10 @@ cudaError_t launch_two_stage(const TwoStageLaunch& L, cudaStream_t s) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t share = std::max<int64_t>(1, std::min<int64_t>(ceil_div(L.max_list, TS_THREADS), 16 * (int64_t)sms / blocks));
     const dim3 grid((unsigned)blocks, (unsigned)std::min<int64_t>(share, 65535));
+    // the second stage's blocks mostly end at once: four times as many, so that the
+    // lists with survivors are shared by more of them
+    const int64_t share2 = std::max<int64_t>(1, std::min<int64_t>(ceil_div(L.max_list, TS_THREADS), 64 * (int64_t)sms / blocks));
+    const dim3 grid2((unsigned)blocks, (unsigned)std::min<int64_t>(share2, 65535));
     const size_t tab_bytes = (size_t)L.D * 16;
     cudaError_t e = cudaFuncSetAttribute(ts_stage1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tab_bytes);
     if (e != cudaSuccess) return e;
@@ -437,14 +461,14 @@ cudaError_t launch_two_stage(const TwoStageLaunch& L, cudaStream_t s) {
     count_launch();
     const size_t xq_bytes = (size_t)(L.D / 64) * 65 * 4;
     switch (L.B) {
-        case 1: ts_stage2_kernel<1><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
-        case 2: ts_stage2_kernel<2><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
-        case 3: ts_stage2_kernel<3><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
-        case 5: ts_stage2_kernel<5><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
-        case 6: ts_stage2_kernel<6><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
-        case 7: ts_stage2_kernel<7><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
-        case 8: ts_stage2_kernel<8><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
-        default: ts_stage2_kernel<9><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 1: ts_stage2_kernel<1><<<grid2, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 2: ts_stage2_kernel<2><<<grid2, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 3: ts_stage2_kernel<3><<<grid2, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 5: ts_stage2_kernel<5><<<grid2, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 6: ts_stage2_kernel<6><<<grid2, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 7: ts_stage2_kernel<7><<<grid2, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 8: ts_stage2_kernel<8><<<grid2, TS_THREADS, xq_bytes, s>>>(a); break;
+        default: ts_stage2_kernel<9><<<grid2, TS_THREADS, xq_bytes, s>>>(a); break;
     }
     count_launch();
     ts_select_kernel<<<(unsigned)L.nq, 256, 0, s>>>(L.skey, L.qoffr, L.scnt, L.nq, L.kp, L.cand);
