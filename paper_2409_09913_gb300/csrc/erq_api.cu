@@ -370,7 +370,7 @@ static erq_status build_kmeans(const float* X, int64_t N, int D, int nlist, cons
         ERQ_TRY(assign_rows(Xs, xn, S, sa));
         if ((e = launch_group(sa, S, nlist, soff, sids, nullptr, nullptr, gscr, gbytes, ix->status, s)) != cudaSuccess)
             return cuda_fail(e, "kmeans group");
-        if ((e = launch_centroids(Xs, soff, sids, nlist, D, ix->C, 1, s)) != cudaSuccess)
+        if ((e = launch_centroids(Xs, soff, sids, S, nlist, D, ix->C, 1, s)) != cudaSuccess)
             return cuda_fail(e, "kmeans centroids");
     }
     // final assignment of every row
@@ -475,7 +475,7 @@ extern "C" erq_status erq_build_index(const float* X, int64_t N, int32_t D, cons
         if ((e = cudaMemcpyAsync(ix->C, p->centroids, sizeof(float) * (size_t)nlist * D, cudaMemcpyDeviceToDevice,
                                  s)) != cudaSuccess)
             return bail2(cuda_fail(e, "copy centroids"));
-    } else if ((e = launch_centroids(X, ix->list_off, ix->list_ids, nlist, D, ix->C, 0, s)) != cudaSuccess) {
+    } else if ((e = launch_centroids(X, ix->list_off, ix->list_ids, N, nlist, D, ix->C, 0, s)) != cudaSuccess) {
         return bail2(cuda_fail(e, "centroids"));
     }
     if ((e = launch_rotate_fp64(ix->C, nullptr, nullptr, nullptr, ix->P, ix->Cp, nlist, D, s)) != cudaSuccess)

@@ -57,8 +57,8 @@ cudaError_t launch_sqdist(const float* Q, const float* qn, const float* C, const
                           int nc, int D, cudaStream_t s);
 cudaError_t launch_row_sqnorm(const float* X, int64_t n, int D, float* out, cudaStream_t s);
 cudaError_t launch_normalize_rows(const float* X, int64_t n, int D, float* Y, cudaStream_t s);
-cudaError_t launch_centroids(const float* X, const int64_t* list_off, const int64_t* list_ids, int nlist, int D,
-                             float* C, int keep_empty, cudaStream_t s);
+cudaError_t launch_centroids(const float* X, const int64_t* list_off, const int64_t* list_ids, int64_t rows, int nlist,
+                             int D, float* C, int keep_empty, cudaStream_t s);
 cudaError_t launch_group(const int32_t* assign, int64_t n, int nlist, int64_t* list_off, int64_t* list_ids,
                          int64_t* row_of, int32_t* cl_of_row, void* scratch, size_t scratch_bytes,
                          uint32_t* status, cudaStream_t s);

@@ -535,10 +535,42 @@ __global__ void __launch_bounds__(128) centroid_ordered_kernel(const float* __re
     }
 }
 
-cudaError_t launch_centroids(const float* X, const int64_t* list_off, const int64_t* list_ids, int nlist, int D,
-                             float* C, int keep_empty, cudaStream_t s) {
+// The ordered sums of short lists: a thread per (cluster, coordinate), neighbouring
+// coordinates side by side, four rows in flight.
+__global__ void __launch_bounds__(256) centroid_short_kernel(const float* __restrict__ X,
+                                                             const int64_t* __restrict__ list_off,
+                                                             const int64_t* __restrict__ list_ids, int64_t total, int D,
+                                                             float* __restrict__ C, int keep_empty) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= total) return;
+    const int64_t j = t / D;
+    const int k = (int)(t - j * D);
+    const int64_t b = list_off[j], e = list_off[j + 1];
+    double acc = 0.0;
+    for (int64_t r = b; r < e; r += 4) {
+        float x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = r + u < e ? X[list_ids[r + u] * D + k] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (r + u < e) acc = __dadd_rn(acc, (double)x[u]);
+    }
+    if (e > b) C[t] = __double2float_rn(__ddiv_rn(acc, (double)(e - b)));
+    else if (!keep_empty) C[t] = 0.f;
+}
+
+cudaError_t launch_centroids(const float* X, const int64_t* list_off, const int64_t* list_ids, int64_t rows, int nlist,
+                             int D, float* C, int keep_empty, cudaStream_t s) {
     const int64_t tot = (int64_t)nlist * D;
     int32_t* redo = nullptr;
+    // Up to 32 rows a list on average, the sums in order at once: one launch instead of
+    // two with a list allocated between them, and chains too short to wait for (an
+    // iteration of k-means over 4,000 x 64 in 256 lists: 135 -> 120 us).
+    if (rows <= 32 * (int64_t)nlist) {
+        count_launch();
+        centroid_short_kernel<<<(unsigned)ceil_div(tot, 256), 256, 0, s>>>(X, list_off, list_ids, tot, D, C, keep_empty);
+        return cudaGetLastError();
+    }
     const bool fast = tot < 0x7fffffff && D % 64 == 0 && D / 64 <= 65535 && ((uintptr_t)X & 15) == 0;
     if (!fast || cudaMallocAsync((void**)&redo, sizeof(int32_t) * (size_t)(tot + 1), s) != cudaSuccess) {
         if (fast) cudaGetLastError();                               // (no memory for the list: all in order)
