@@ -521,14 +521,15 @@ extern "C" erq_status erq_build_index(const float* X, int64_t N, int32_t D, cons
 // extent) and rows per item.  For k' <= 32,
 // 128 queries per item (twice the MMA width for one conversion of the codes)
 // when a probed cluster has more than 72 probing queries on average and there is
-// work enough that the last items do not leave SMs idle for long: items x D of at
-// least 5,000 an SM.  Otherwise 64; for larger k' 32.  The whole search's time with
+// work enough that the last items do not leave SMs idle for long: eight items, or
+// items x D of 5,000, an SM.  Otherwise 64; for larger k' 32.  The whole search's time with
 // 64 over that with 128, from 72 to 192 queries a list, by items x D an SM (D = 64
 // .. 1536, B = 1 .. 9, FP16 and e4m3, 60 .. 400 rows a list, k' = 20 and 32):
 //   256 lists, 110 .. 2,600: 0.81 .. 1.00    512 lists, 1,300 .. 3,200: 0.85 .. 1.02
 //   1,024 lists, 860: 0.93 .. 0.99           2,048 lists, 1,700: 0.96 .. 1.01
 //   1,024 and 512 lists, 5,200: 0.96 .. 1.09
 //   2,048 lists, 5,200 .. 20,700: 0.97 .. 1.11
+// and with 384 queries a list, 512 lists of 390 x 384 (10 items, 3,900): 1.06 and 1.13.
 // FP32 precision has two query parts per tile and stops at 64.  Rows:
 // at most 8,192, and few enough that the items can fill the chip twice (a
 // single query's 16 lists of 200 rows are 32 one-block items instead of 16), but
@@ -551,7 +552,8 @@ static void default_scan_shape(const erq_index* ix, int prec, int kp, int64_t nq
     int q = cls == 0 ? 64 : 32;
     if (cls == 0 && prec != ERQ_PREC_FP32 && per_list > 72.0) {
         const double ranges = std::ceil((double)ix->N / ix->nlist / rows_of(128));
-        if (lists * ranges * std::ceil((double)work / lists / 128.0) * ix->D >= 5000.0 * sms) q = 128;
+        const double items = lists * ranges * std::ceil((double)work / lists / 128.0);
+        if (items >= 8.0 * sms || items * ix->D >= 5000.0 * sms) q = 128;
     }
     *qn = q;
     *rr = rows_of(q);

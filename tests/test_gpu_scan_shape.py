@@ -36,7 +36,8 @@ def test_one_large_list(erq, nq, precision, async_mode):
 
 
 @pytest.mark.parametrize("nlist,D,per_list,rows,want", [(256, 64, 80, 20, 64), (256, 64, 200, 20, 64), (512, 1536, 80, 20, 128),
-                                                         (512, 1536, 60, 20, 64), (512, 960, 80, 20, 64), (4096, 192, 80, 4, 128)])
+                                                         (512, 1536, 60, 20, 64), (512, 960, 80, 20, 64), (4096, 192, 80, 4, 128),
+                                                         (32, 64, 8192, 40, 128), (2048, 64, 80, 4, 128)])
 def test_queries_of_an_item(erq, nlist, D, per_list, rows, want):
     N, np_ = nlist * rows, 16
     X, _ = S.mixture(N, D, 8, 74)
