@@ -289,8 +289,8 @@ __device__ __forceinline__ float last_bits_dot(const uint64_t* w, const float* x
 // 134 us for 16 queries x 16 lists of 200,000 x 960 in 1,024, 34 us.  Where many
 // survive (half of a query's nearest list), a lane per row is better: from 16 of
 // 32 on, from 8 where the blocks fill only half of the W lanes.  512 queries x 8
-// lists of 20,000 x 1,088 in 32: 406 us with lanes for all, 135.  Query coordinates are spaced 65 floats a
-// block so that the lanes' reads fall into different banks.
+// lists of 20,000 x 1,088 in 32: 406 us with lanes for all, 135.  Query coordinates
+// are spaced 65 floats a block so that the lanes' reads fall into different banks.
 template <int B>
 __global__ void __launch_bounds__(TS_THREADS) ts_stage2_kernel(TsArgs a) {
     extern __shared__ __align__(16) float xq[];            // [D / 64][65] P^T q_r
@@ -304,12 +304,15 @@ __global__ void __launch_bounds__(TS_THREADS) ts_stage2_kernel(TsArgs a) {
     const float dq = a.dqc[q * a.maxp + slot], tq = a.tau[q];
     const int64_t o0 = a.qoffr[q] + a.rbase[q * a.maxp + slot];
     // (a comparison that keeps rows without an ordered bound)
-    bool any = false;
+    bool any = B == 1;
+    if (B > 1) {
 #pragma unroll 4
-    for (int64_t j = (int64_t)blockIdx.y * TS_THREADS + threadIdx.x; j < size; j += (int64_t)gridDim.y * TS_THREADS)
-        any |= !(a.lb[o0 + j] > tq);
-    if (!__syncthreads_or(any)) return;
-    for (int i = threadIdx.x; i < D; i += TS_THREADS) xq[(i >> 6) * 65 + (i & 63)] = a.Qrot[q * D + i];
+        for (int64_t j = (int64_t)blockIdx.y * TS_THREADS + threadIdx.x; j < size; j += (int64_t)gridDim.y * TS_THREADS)
+            any |= !(a.lb[o0 + j] > tq);
+    }
+    if (!__syncthreads_or(any)) return;                    // (B = 1: nothing to complete, and nothing staged)
+    if (B > 1)
+        for (int i = threadIdx.x; i < D; i += TS_THREADS) xq[(i >> 6) * 65 + (i & 63)] = a.Qrot[q * D + i];
     __syncthreads();
     const float hi = (float)(1 << (B - 1));
     const int lane = threadIdx.x & 31;
@@ -461,7 +464,7 @@ cudaError_t launch_two_stage(const TwoStageLaunch& L, cudaStream_t s) {
     count_launch();
     const size_t xq_bytes = (size_t)(L.D / 64) * 65 * 4;
     switch (L.B) {
-        case 1: ts_stage2_kernel<1><<<grid2, TS_THREADS, xq_bytes, s>>>(a); break;
+        case 1: ts_stage2_kernel<1><<<grid, TS_THREADS, xq_bytes, s>>>(a); break;
         case 2: ts_stage2_kernel<2><<<grid2, TS_THREADS, xq_bytes, s>>>(a); break;
         case 3: ts_stage2_kernel<3><<<grid2, TS_THREADS, xq_bytes, s>>>(a); break;
         case 5: ts_stage2_kernel<5><<<grid2, TS_THREADS, xq_bytes, s>>>(a); break;
