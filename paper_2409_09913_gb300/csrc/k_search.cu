@@ -615,7 +615,7 @@ int scan_fp32_blocks_per_sm(int kp, int B) { return B > 8 ? fp32_blocks_per_sm<2
 // sorted; where even these do not fit (many equal values), a running best k' and
 // a chunk at a time are.  Bound by the latency of the passes over the lists, a
 // warp per list: 100 queries x 79 lists, k' = 100, 79 us with the chunks alone,
-// 20 us.  1,024 threads while every query can have half an SM, else 256.
+// 20 us.  1,024 threads or 256 (launch_merge).
 // ---------------------------------------------------------------------------
 __device__ void block_bitonic_u64(uint64_t* v, int n) {
     for (int size = 2; size <= n; size <<= 1)
@@ -1330,6 +1330,13 @@ cudaError_t launch_one_list_per_query(int64_t nq, int m, int32_t* counts, int64_
     return cudaGetLastError();
 }
 
+static int sm_count() {
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
 int merge_sortn(int kp, int lstride) {
     int sortn = 128;
     while (sortn < 4 * kp || sortn < kp + lstride + 32) sortn <<= 1;
@@ -1340,14 +1347,17 @@ cudaError_t launch_merge(const uint64_t* inter, const int32_t* inter_cnt, const 
                          int lstride, const unsigned long long* tq, uint64_t* cand, const DevChecks& ck,
                          cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
+    const int sms = sm_count();
     if (kp <= 32) {
         count_launch();
-        // eight warps per query where there are lists for them (more than 32 a
-        // query) or too few queries to fill the chip with one warp each; a whole
-        // block's 32 while each query can have an SM's half to itself
-        if (nq <= 256 && ck.lists > 32 * nq)
+        // Eight warps per query where there are lists for them (more than 32 a query)
+        // or too few queries to fill the chip with one warp each (1,000 queries x 8 lists:
+        // 10.7 us with eight, 12.0 with one; 1,500: 14.1 and 14.2; 2,000: 17.4 and 13.9);
+        // a whole block's 32 while each query can have an SM to itself (128 queries x 64
+        // lists: 9.7 us with 32, 12.7 with eight; 200: 16.6 and 14.4).
+        if (nq <= sms && ck.lists > 32 * nq)
             merge32_kernel<32><<<(unsigned)nq, 1024, 0, s>>>(inter, inter_cnt, qbase, nq, kp, lstride, tq, cand, ck);
-        else if (ck.lists > 32 * nq || nq < 2048)
+        else if (ck.lists > 32 * nq || nq < 10 * sms)
             merge32_kernel<8><<<(unsigned)nq, 256, 0, s>>>(inter, inter_cnt, qbase, nq, kp, lstride, tq, cand, ck);
         else
             merge32_kernel<1><<<(unsigned)ceil_div(nq, 8), 256, 0, s>>>(inter, inter_cnt, qbase, nq, kp, lstride, tq, cand,
@@ -1358,13 +1368,15 @@ cudaError_t launch_merge(const uint64_t* inter, const int32_t* inter_cnt, const 
     cudaError_t e = cudaFuncSetAttribute(merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sortn * 8);
     if (e != cudaSuccess) return e;
     count_launch();
-    merge_kernel<<<(unsigned)nq, nq <= 304 ? 1024 : 256, sortn * 8, s>>>(inter, inter_cnt, qbase, kp, lstride, sortn, tq, cand, ck);
+    // (k' = 100, 64 lists: 300 queries 18.5 us with 1,024 threads, 23.1 with 256; 400: 26.9 and 29.6; 608: 34.0 and 31.4)
+    merge_kernel<<<(unsigned)nq, nq <= 3 * sms ? 1024 : 256, sortn * 8, s>>>(inter, inter_cnt, qbase, kp, lstride, sortn, tq, cand, ck);
     return cudaGetLastError();
 }
 
-// Exact re-rank for k' <= 32: one block of NW warps per query (eight; 32 where
-// there are too few queries to fill the chip, so that all candidates' rows are
-// fetched at once: one query, 9.7 -> 5.4 us), the query row in shared memory; warp
+// Exact re-rank for k' <= 32: one block of NW warps per query (eight; 32 while each
+// query can have an SM to itself, so that all candidates' rows are fetched at once:
+// 128 queries, k' = 20, D = 960: 4.9 -> 3.6 us; 200: 5.2 and 5.9), the query row in
+// shared memory; warp
 // w computes ||x - q||^2 for candidates w, w + NW, ...
 // with each lane keeping up to eight 16-byte loads of the row in flight (the
 // first row's loads are issued before the query row is waited for), then warp
@@ -1449,7 +1461,7 @@ cudaError_t launch_rerank(const uint64_t* cand, int64_t nq, int kp, const float*
         const size_t smem = (size_t)D * sizeof(float);
         // (at most 16 KB of shared memory)
         count_launch();
-        if (nq <= 256)
+        if (nq <= sm_count())
             rerank32_kernel<32><<<(unsigned)nq, 1024, smem, s>>>(cand, kp, X, Q, D, k, ip, ids, dists, cand_ids, cand_est, ck);
         else
             rerank32_kernel<8><<<(unsigned)nq, 256, smem, s>>>(cand, kp, X, Q, D, k, ip, ids, dists, cand_ids, cand_est, ck);
