@@ -18,8 +18,8 @@
 // of the sequential FP64 sum: dropped pairs and tails (2.1 D), the floor of the
 // last accumulator, and the FP64 sum's own rounding (D 2^-53 sum |x p|, Cauchy-
 // Schwarz).  Where I - delta and I + delta round to the same FP32 value, that is
-// the result; the other elements (about 6 in 10,000) go to a list and are summed
-// in FP64 in order by rotate_fix_kernel.  A list that overflows, a row that is
+// the result; the other elements (1 in 480 at D = 768, 1 in 115 at D = 4096) go to a
+// list and are summed in FP64 in order by rotate_fix_kernel.  A list that overflows, a row that is
 // not finite or a wait that runs out sets a flag, and rotate_fp64_kernel then
 // computes the whole block.
 //
@@ -379,7 +379,10 @@ cudaError_t launch_rotate_tc(const float* X, const int64_t* gather, const float*
         cudaStreamIsCapturing(s, &cap_st) != cudaSuccess || cap_st != cudaStreamCaptureStatusNone)
         return cudaErrorNotSupported;
     const int64_t block = std::min<int64_t>(n, std::max<int64_t>(2048, ((256ll << 20) / (ND * 2 * (int64_t)D)) / BM * BM));
-    const size_t cap = (size_t)(block * D / 128 + 8192);
+    // doubtful elements of ordinary rows: 1 in 480 at D = 768, 1 in 180 at 2,048, 1 in 115
+    // at 3,072 and 4,096; a list that is too short costs the whole block again in FP64
+    // (65,536 x 3,072 with room for 1 in 128: 1,600 ms, 62 with room for 1 in 32)
+    const size_t cap = (size_t)(block * D / 32 + 8192);
     size_t off = 0;
     auto part = [&](size_t bytes) {
         const size_t at = off;
