@@ -254,7 +254,8 @@ erq_status erq_search_two_stage(erq_index* index, const float* Q, int64_t nq, co
                                 float eps0, int64_t* ids, float* dists, int64_t* stats, void* stream);
 
 /* The same search from HOST buffers: Q_host[nq][D] is copied to the device,
- * searched, and ids_host/dists_host are copied back before the call returns.
+ * searched, and ids_host/dists_host are copied back before the call returns.  Without
+ * ERQ_SEARCH_ASYNC a device-side error of the search is returned by this call.
  * Pinned (page-locked) host memory gives asynchronous copies. */
 erq_status erq_search_host(erq_index* index, const float* Q_host, int64_t nq, const erq_search_params* params,
                            int64_t* ids_host, float* dists_host, void* stream);
